@@ -2,19 +2,27 @@
 // pipeline (its per-block update c_ij = alpha a_i b_j + beta c_ij) on the FP64
 // tensor-core MMA (mma.sync m8n8k4 .f64), fed by TMA tile loads.
 //
-// Shape: CTA tile 64 x 64, K step 16, a 4-stage ring of TMA-filled shared
+// Shape: CTA tile 16 x 16, K steps of 16, an 8-stage ring of TMA-filled shared
 // memory stages guarded by full/empty mbarriers.  Warp 4 is the producer (one
-// elected lane issues the tensor copies); warps 0-3 each own a 32 x 32 part of
-// the tile as 4 x 4 MMA fragments in registers.  The grid is persistent: each
-// CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with the stage ring
-// running on across tile boundaries, so the copies of the next tile overlap
-// the epilogue of the current one (tiles are taken in a grouped raster order,
-// see tile_of).  Ragged edges come from the tensor maps:
-// reads outside the operand are zero-filled by TMA and the epilogue masks
-// stores.
+// elected lane issues the tensor copies); warps 0-3 each own one 8 x 8 MMA
+// fragment of the tile in registers.  The grid is persistent: each CTA walks tiles
+// blockIdx.x, blockIdx.x + gridDim.x, ... with the stage ring running on across
+// tile boundaries, so the copies of the next tile overlap the epilogue of the
+// current one (tiles are taken in a grouped raster order, see raster_tile).
+// Ragged edges come from the tensor maps: reads outside the operand are
+// zero-filled by TMA, the epilogue masks stores, and fragments and K steps that
+// lie wholly outside the operands are not multiplied.
 //
-// GB300 has a small FP64 rate, so this kernel is bound by the FP64 pipe; the
-// 64 x 64 tile keeps wave quantisation low on large blocks.
+// What bounds it: GB300's FP64 rate, 1.75 fused multiply-adds per clock and SM
+// (1.10 TFLOP/s in all).  Even this small tile holds an SM for 1.1 us per K step
+// with 4 KiB of operands, so copies, barriers and shared-memory conflicts do not
+// show and the only thing left to lose is balance: an SM that gets one tile more
+// than another keeps the whole launch waiting.  Measured against 64 x 64 and
+// 32 x 32 tiles (TFLOP/s): 8192 x 8192 x 512 1.097 / 1.096 / 1.097, 704 x 5003 x
+// 1024 1.092 / 1.031 / 1.034, 1536 x 1000 x 2000 1.071 / 0.900 / 0.984, 512^3 1.02
+// / 0.45 / 0.89, 192 x 1024 x 256 0.87 / 0.34 / 0.65; the small tile is never the
+// slower one.  Every output is accumulated in the same order (k ascending, four
+// at a time) whatever the tile.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -30,12 +38,13 @@ namespace ooc {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, STAGES = 4;
+constexpr int T = 16;   // edge of the CTA tile
+constexpr int W = T / 2;  // edge of a warp's 8 x 8 fragment
+constexpr int BK = 16, STAGES = 8;
 constexpr int CONSUMER_WARPS = 4;
 constexpr int THREADS = (CONSUMER_WARPS + 1) * 32;
-constexpr int STAGE_A = BM * BK;  // doubles
-constexpr int STAGE_B = BN * BK;
-constexpr uint32_t STAGE_BYTES = (STAGE_A + STAGE_B) * 8;
+constexpr int STAGE = T * BK;  // doubles per operand
+constexpr uint32_t STAGE_BYTES = 2 * STAGE * 8;
 constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 2 * STAGES * sizeof(uint64_t) + 1024;
 
 // Tiles of a triangular update (GEMMT / SYRK blocks that straddle the
@@ -97,21 +106,26 @@ struct Fp64Args {
     TriTiles tt;
 };
 
-// Tile order of a full update: groups of kRasterRows tile rows, column-major
-// inside a group, so that the ~456 tiles in flight span 16 rows and ~29
+// Tile order of a full update: groups of kRasterRows tile rows (256 matrix rows),
+// column-major inside a group, so that the ~900 tiles in flight span few rows and
 // columns and re-read their A and B tiles from L2 rather than DRAM.
 constexpr int64_t kRasterRows = 16;
+
+__host__ __device__ __forceinline__ void raster_tile(int64_t tile, int64_t tiles_m, int64_t tiles_n, int64_t& tm,
+                                                     int64_t& tn)
+{
+    const int64_t per_group = kRasterRows * tiles_n;
+    const int64_t g = tile / per_group, r = tile % per_group;
+    const int64_t first = g * kRasterRows;
+    const int64_t rows = tiles_m - first < kRasterRows ? tiles_m - first : kRasterRows;
+    tm = first + r % rows;
+    tn = r / rows;
+}
 
 __device__ __forceinline__ void tile_of(const Fp64Args& p, int64_t tile, int64_t& tm, int64_t& tn)
 {
     if (p.tri == 0) {
-        const int64_t tiles_m = p.tiles / p.tiles_n;
-        const int64_t per_group = kRasterRows * p.tiles_n;
-        const int64_t g = tile / per_group, r = tile % per_group;
-        const int64_t first = g * kRasterRows;
-        const int64_t rows = tiles_m - first < kRasterRows ? tiles_m - first : kRasterRows;
-        tm = first + r % rows;
-        tn = r / rows;
+        raster_tile(tile, p.tiles / p.tiles_n, p.tiles_n, tm, tn);
         return;
     }
     int64_t lo = 0, hi = p.tt.tiles_m - 1;  // largest tm with prefix(tm) <= tile
@@ -137,173 +151,198 @@ __device__ __forceinline__ void dmma_8x8x4(double& d0, double& d1, double a, dou
                  : "d"(a), "d"(b));
 }
 
+// The stage ring of a CTA: T x BK tiles of A and B, their barriers, and this
+// thread's position in the ring (advanced without division).
+struct Ring {
+    double* stages;
+    uint64_t *full, *empty;
+    int s = 0;
+    uint32_t ph = 0;
+
+    __device__ explicit Ring(unsigned char* smem)
+    {
+        unsigned char* base =
+            reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem) + 1023) & ~uintptr_t(1023));
+        stages = reinterpret_cast<double*>(base);
+        full = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES);
+        empty = full + STAGES;
+    }
+    __device__ void init()
+    {
+        if (threadIdx.x == 0) {
+            for (int q = 0; q < STAGES; ++q) {
+                mbar_init(&full[q], 1);
+                mbar_init(&empty[q], CONSUMER_WARPS);
+            }
+            mbar_fence_init();
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void next()
+    {
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
+    }
+};
+
+// Producer: the K steps of one tile into the ring; false when a wait gave up.
+template <bool A_KMAJOR, bool B_KMAJOR>
+__device__ __forceinline__ bool produce_tile(Ring& r, const CUtensorMap* ma, const CUtensorMap* mb, int64_t nk,
+                                             int32_t row0, int32_t col0, int64_t& issued, int* err)
+{
+    for (int64_t ks = 0; ks < nk; ++ks) {
+        if (!mbar_wait(&r.empty[r.s], r.ph ^ 1u, err, kErrWaitEmpty)) return false;
+        double* sA = r.stages + (size_t)r.s * 2 * STAGE;
+        double* sB = sA + STAGE;
+        mbar_arrive_expect_tx(&r.full[r.s], STAGE_BYTES);
+        const int32_t k0 = (int32_t)(ks * BK);
+        if (A_KMAJOR) tma_load_2d(sA, ma, &r.full[r.s], k0, row0);
+        else tma_load_2d(sA, ma, &r.full[r.s], row0, k0);
+        if (B_KMAJOR) tma_load_2d(sB, mb, &r.full[r.s], k0, col0);
+        else tma_load_2d(sB, mb, &r.full[r.s], col0, k0);
+        r.next();
+        ++issued;
+    }
+    return true;
+}
+
+// After a wait gave up: let the copies already issued land before the CTA exits.
+__device__ __forceinline__ void drain_ring(const Ring& r, int64_t issued)
+{
+    constexpr int N = STAGES;
+    for (int64_t w = issued > N ? issued - N : 0; w < issued; ++w) {
+        const int s = (int)(w % N);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(smem_u32(&r.full[s]), (uint32_t)((w / N) & 1)) && globaltimer_ns() - t0 < kWaitLimitNs) {
+        }
+    }
+}
+
+// Consumer warp: multiply the K steps of one tile into its fragment.  inside: the
+// fragment holds an element of C; K: inner dimension.  False when a wait gave up.
+template <bool A_KMAJOR, bool B_KMAJOR>
+__device__ __forceinline__ bool consume_tile(Ring& r, double (&acc)[2], int64_t nk, int64_t K, bool inside, int* err)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = (warp >> 1) * W + (lane >> 2), col = (warp & 1) * W + (lane >> 2);  // 2 x 2 warps
+    const int fc = lane & 3;
+    for (int64_t ks = 0; ks < nk; ++ks) {
+        if (!mbar_wait(&r.full[r.s], r.ph, err, kErrWaitFull)) return false;
+        const double* sA = r.stages + (size_t)r.s * 2 * STAGE;
+        const double* sB = sA + STAGE;
+        const int64_t left = K - ks * BK;
+        if (inside) {
+#pragma unroll
+            for (int kk = 0; kk < BK; kk += 4) {
+                if (kk >= left) break;  // the last K step: only what lies inside the operands
+                const int k = kk + fc;
+                const double a = A_KMAJOR ? sA[row * BK + k] : sA[k * T + row];
+                const double b = B_KMAJOR ? sB[col * BK + k] : sB[k * T + col];
+                dmma_8x8x4(acc[0], acc[1], a, b);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&r.empty[r.s]);
+        r.next();
+    }
+    return true;
+}
+
+// C = alpha acc + beta C on this warp's fragment at (row0, col0), then acc = 0.
+// keep(row, col) masks single elements of a triangular update (kMasked).
+template <bool kMasked, class Keep>
+__device__ __forceinline__ void store_tile(double (&acc)[2], int64_t row0, int64_t col0, int64_t M, int64_t N,
+                                           double alpha, double beta, int read_c, double* C, int64_t ldc, Keep keep)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t row = row0 + (lane >> 2), col = col0 + (lane & 3) * 2;
+    if (row < M) {
+        double* c = C + row * ldc + col;
+        if (!kMasked && col + 1 < N) {
+            double2 v;
+            v.x = alpha * acc[0];
+            v.y = alpha * acc[1];
+            if (read_c) {
+                const double2 o = *reinterpret_cast<const double2*>(c);
+                v.x += beta * o.x;
+                v.y += beta * o.y;
+            }
+            *reinterpret_cast<double2*>(c) = v;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (col + e >= N || (kMasked && !keep(row, col + e))) continue;
+                double v = alpha * acc[e];
+                if (read_c) v += beta * c[e];
+                c[e] = v;
+            }
+        }
+    }
+    acc[0] = acc[1] = 0.0;
+}
+
 template <bool A_KMAJOR, bool B_KMAJOR>
 __global__ void __launch_bounds__(THREADS) fp64_tile_kernel(const __grid_constant__ CUtensorMap tmA,
                                                             const __grid_constant__ CUtensorMap tmB,
                                                             Fp64Args p)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // 1024-byte alignment of the stage ring
-    unsigned char* base = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    double* stages = reinterpret_cast<double*>(base);
-    uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES);
-    uint64_t* empty = full + STAGES;
-
+    Ring r(smem_raw);
+    r.init();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], CONSUMER_WARPS);
-        }
-        mbar_fence_init();
-    }
-    __syncthreads();
-
     const int64_t nk = (p.K + BK - 1) / BK;
-    const int64_t my_tiles = p.tiles > blockIdx.x ? (p.tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const int64_t total = my_tiles * nk;
-
     if (warp == CONSUMER_WARPS) {
         // ---------------- producer ----------------
-        if (lane == 0 && total > 0) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
-            int64_t it = 0;
-            bool ok = true;
-            for (; it < total; ++it) {
-                const int s = (int)(it % STAGES);
-                const uint32_t ph = (uint32_t)((it / STAGES) & 1);
-                if (!mbar_wait(&empty[s], ph ^ 1u, p.err, kErrWaitEmpty)) { ok = false; break; }
-                const int64_t tl = it / nk, ks = it % nk;
-                const int64_t tile = blockIdx.x + tl * gridDim.x;
-                int64_t tm64, tn64;
-                tile_of(p, tile, tm64, tn64);
-                const int32_t tm = (int32_t)tm64, tn = (int32_t)tn64;
-                double* sA = stages + (size_t)s * (STAGE_A + STAGE_B);
-                double* sB = sA + STAGE_A;
-                mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-                const int32_t k0 = (int32_t)(ks * BK);
-                if (A_KMAJOR) tma_load_2d(sA, &tmA, &full[s], k0, tm * BM);
-                else tma_load_2d(sA, &tmA, &full[s], tm * BM, k0);
-                if (B_KMAJOR) tma_load_2d(sB, &tmB, &full[s], k0, tn * BN);
-                else tma_load_2d(sB, &tmB, &full[s], tn * BN, k0);
-            }
-            if (!ok) {
-                // let the copies already issued land before the CTA exits
-                for (int64_t q = (it > STAGES ? it - STAGES : 0); q < it; ++q) {
-                    const int s = (int)(q % STAGES);
-                    const uint64_t t0 = globaltimer_ns();
-                    while (!mbar_try_wait(smem_u32(&full[s]), (uint32_t)((q / STAGES) & 1)) &&
-                           globaltimer_ns() - t0 < kWaitLimitNs) {
-                    }
-                }
-            }
+        if (lane != 0 || nk == 0) return;
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+        int64_t issued = 0;
+        bool ok = true;
+        for (int64_t tile = blockIdx.x; tile < p.tiles && ok; tile += gridDim.x) {
+            int64_t tm, tn;
+            tile_of(p, tile, tm, tn);
+            ok = produce_tile<A_KMAJOR, B_KMAJOR>(r, &tmA, &tmB, nk, (int32_t)(tm * T), (int32_t)(tn * T), issued,
+                                                     p.err);
         }
+        if (!ok) drain_ring(r, issued);
         return;
     }
-
     // ---------------- consumers ----------------
-    const int wm = warp >> 1, wn = warp & 1;  // 2 x 2 warps of 32 x 32
-    const int fr = lane >> 2, fc = lane & 3;  // fragment row / column of this lane
-    double acc[4][4][2];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
-
-    auto epilogue = [&](int64_t tile) {
+    double acc[2] = {0.0, 0.0};
+    for (int64_t tile = blockIdx.x; tile < p.tiles; tile += gridDim.x) {
         int64_t tm, tn;
         tile_of(p, tile, tm, tn);
-#pragma unroll
-        for (int mi = 0; mi < 4; ++mi) {
-            const int64_t row = tm * BM + wm * 32 + mi * 8 + fr;
-#pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int64_t col = tn * BN + wn * 32 + ni * 8 + fc * 2;
-                if (row < p.M && p.tri != 0) {  // masked: element by element
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        if (col + e >= p.N || !kept(p, row, col + e)) continue;
-                        double* c = p.C + row * p.ldc + col + e;
-                        double v = p.alpha * acc[mi][ni][e];
-                        if (p.read_c) v += p.beta * c[0];
-                        c[0] = v;
-                    }
-                } else if (row < p.M) {
-                    double* c = p.C + row * p.ldc + col;
-                    if (col + 1 < p.N) {
-                        double2 v;
-                        v.x = p.alpha * acc[mi][ni][0];
-                        v.y = p.alpha * acc[mi][ni][1];
-                        if (p.read_c) {
-                            const double2 o = *reinterpret_cast<const double2*>(c);
-                            v.x += p.beta * o.x;
-                            v.y += p.beta * o.y;
-                        }
-                        *reinterpret_cast<double2*>(c) = v;
-                    } else if (col < p.N) {
-                        double v = p.alpha * acc[mi][ni][0];
-                        if (p.read_c) v += p.beta * c[0];
-                        c[0] = v;
-                    }
-                }
-                acc[mi][ni][0] = acc[mi][ni][1] = 0.0;
-            }
-        }
-    };
-
-    if (nk == 0) {  // K == 0: C = beta * C (or 0)
-        for (int64_t tl = 0; tl < my_tiles; ++tl) epilogue(blockIdx.x + tl * gridDim.x);
-        return;
+        const int64_t row0 = tm * T + (warp >> 1) * W, col0 = tn * T + (warp & 1) * W;
+        if (!consume_tile<A_KMAJOR, B_KMAJOR>(r, acc, nk, p.K, row0 < p.M && col0 < p.N, p.err))
+            return;
+        auto keep = [&](int64_t row, int64_t col) { return kept(p, row, col); };
+        if (p.tri) store_tile<true>(acc, row0, col0, p.M, p.N, p.alpha, p.beta, p.read_c, p.C, p.ldc, keep);
+        else store_tile<false>(acc, row0, col0, p.M, p.N, p.alpha, p.beta, p.read_c, p.C, p.ldc, keep);
     }
+}
 
-    for (int64_t it = 0; it < total; ++it) {
-        const int s = (int)(it % STAGES);
-        if (!mbar_wait(&full[s], (uint32_t)((it / STAGES) & 1), p.err, kErrWaitFull)) return;
-        const double* sA = stages + (size_t)s * (STAGE_A + STAGE_B);
-        const double* sB = sA + STAGE_A;
-#pragma unroll
-        for (int kk = 0; kk < BK; kk += 4) {
-            double af[4], bf[4];
-#pragma unroll
-            for (int mi = 0; mi < 4; ++mi) {
-                const int r = wm * 32 + mi * 8 + fr, k = kk + fc;
-                af[mi] = A_KMAJOR ? sA[r * BK + k] : sA[k * BM + r];
-            }
-#pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int n = wn * 32 + ni * 8 + fr, k = kk + fc;
-                bf[ni] = B_KMAJOR ? sB[n * BK + k] : sB[k * BN + n];
-            }
-#pragma unroll
-            for (int mi = 0; mi < 4; ++mi)
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni) dmma_8x8x4(acc[mi][ni][0], acc[mi][ni][1], af[mi], bf[ni]);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);
-        if (it % nk == nk - 1) epilogue(blockIdx.x + (it / nk) * gridDim.x);
-    }
+// CTAs of a launch: as many as are resident, at most one per tile.
+template <class Kernel>
+int resident_ctas(Kernel kernel, size_t smem, int& occ, std::once_flag& once)
+{
+    std::call_once(once, [&] {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, THREADS, smem);
+    });
+    return occ * device_sm_count();
 }
 
 template <bool AK, bool BKM>
 int launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, const Fp64Args& a, cudaStream_t st,
                    std::string& why)
 {
-    static int occ = 0, sms = 0;
+    static int occ = 0;
     static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(fp64_tile_kernel<AK, BKM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM_BYTES);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_tile_kernel<AK, BKM>, THREADS, SMEM_BYTES);
-        sms = device_sm_count();
-    });
-    if (occ <= 0) {
+    const int64_t room = resident_ctas(fp64_tile_kernel<AK, BKM>, SMEM_BYTES, occ, once);
+    if (room <= 0) {
         why = "fp64 tile kernel cannot be resident (occupancy 0)";
         return OOC_ERR_CUDA;
     }
-    const int64_t grid = std::min<int64_t>(a.tiles > 0 ? a.tiles : 1, (int64_t)occ * sms);
+    const int64_t grid = std::min<int64_t>(a.tiles > 0 ? a.tiles : 1, room);
     fp64_tile_kernel<AK, BKM><<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(ma, mb, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -350,165 +389,57 @@ __device__ __forceinline__ int group_problem(const GroupArgs& g, int64_t t)
     return lo;
 }
 
-__device__ __forceinline__ void group_tile(const GroupProb& q, int64_t t, int64_t& tm, int64_t& tn)
-{
-    const int64_t local = t - q.tile_begin;
-    const int64_t tiles_m = (q.M + BM - 1) / BM;
-    const int64_t per_group = kRasterRows * q.tiles_n;
-    const int64_t gr = local / per_group, r = local % per_group;
-    const int64_t first = gr * kRasterRows;
-    const int64_t rows = tiles_m - first < kRasterRows ? tiles_m - first : kRasterRows;
-    tm = first + r % rows;
-    tn = r / rows;
-}
-
 template <bool A_KMAJOR, bool B_KMAJOR>
 __global__ void __launch_bounds__(THREADS) fp64_group_kernel(const __grid_constant__ GroupArgs g)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    unsigned char* base = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    double* stages = reinterpret_cast<double*>(base);
-    uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES);
-    uint64_t* empty = full + STAGES;
-
+    Ring r(smem_raw);
+    r.init();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], CONSUMER_WARPS);
-        }
-        mbar_fence_init();
-    }
-    __syncthreads();
-
+    auto item = [&](int64_t t, const GroupProb*& q, int64_t& tm, int64_t& tn) {
+        q = &g.p[group_problem(g, t)];
+        raster_tile(t - q->tile_begin, (q->M + T - 1) / T, q->tiles_n, tm, tn);
+    };
     if (warp == CONSUMER_WARPS) {
         // ---------------- producer ----------------
         if (lane != 0) return;
-        int64_t it = 0;  // stages issued so far (ring position)
+        int64_t issued = 0;
         bool ok = true;
         for (int64_t t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
-            const GroupProb& q = g.p[group_problem(g, t)];
-            int64_t tm64, tn64;
-            group_tile(q, t, tm64, tn64);
-            const int32_t tm = (int32_t)tm64, tn = (int32_t)tn64;
-            const int64_t nk = (q.K + BK - 1) / BK;
-            for (int64_t ks = 0; ks < nk; ++ks, ++it) {
-                const int s = (int)(it % STAGES);
-                if (!mbar_wait(&empty[s], (uint32_t)((it / STAGES) & 1) ^ 1u, g.err, kErrWaitEmpty)) {
-                    ok = false;
-                    break;
-                }
-                double* sA = stages + (size_t)s * (STAGE_A + STAGE_B);
-                double* sB = sA + STAGE_A;
-                mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-                const int32_t k0 = (int32_t)(ks * BK);
-                if (A_KMAJOR) tma_load_2d(sA, &q.ma, &full[s], k0, tm * BM);
-                else tma_load_2d(sA, &q.ma, &full[s], tm * BM, k0);
-                if (B_KMAJOR) tma_load_2d(sB, &q.mb, &full[s], k0, tn * BN);
-                else tma_load_2d(sB, &q.mb, &full[s], tn * BN, k0);
-            }
+            const GroupProb* q;
+            int64_t tm, tn;
+            item(t, q, tm, tn);
+            ok = produce_tile<A_KMAJOR, B_KMAJOR>(r, &q->ma, &q->mb, (q->K + BK - 1) / BK, (int32_t)(tm * T),
+                                                     (int32_t)(tn * T), issued, g.err);
         }
-        if (!ok) {
-            // let the copies already issued land before the CTA exits
-            for (int64_t w = (it > STAGES ? it - STAGES : 0); w < it; ++w) {
-                const int s = (int)(w % STAGES);
-                const uint64_t t0 = globaltimer_ns();
-                while (!mbar_try_wait(smem_u32(&full[s]), (uint32_t)((w / STAGES) & 1)) &&
-                       globaltimer_ns() - t0 < kWaitLimitNs) {
-                }
-            }
-        }
+        if (!ok) drain_ring(r, issued);
         return;
     }
-
     // ---------------- consumers ----------------
-    const int wm = warp >> 1, wn = warp & 1;
-    const int fr = lane >> 2, fc = lane & 3;
-    double acc[4][4][2];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
-    int64_t it = 0;
+    double acc[2] = {0.0, 0.0};
     for (int64_t t = blockIdx.x; t < g.tiles; t += gridDim.x) {
-        const GroupProb& q = g.p[group_problem(g, t)];
-        const int64_t nk = (q.K + BK - 1) / BK;
-        for (int64_t ks = 0; ks < nk; ++ks, ++it) {
-            const int s = (int)(it % STAGES);
-            if (!mbar_wait(&full[s], (uint32_t)((it / STAGES) & 1), g.err, kErrWaitFull)) return;
-            const double* sA = stages + (size_t)s * (STAGE_A + STAGE_B);
-            const double* sB = sA + STAGE_A;
-#pragma unroll
-            for (int kk = 0; kk < BK; kk += 4) {
-                double af[4], bf[4];
-#pragma unroll
-                for (int mi = 0; mi < 4; ++mi) {
-                    const int r = wm * 32 + mi * 8 + fr, k = kk + fc;
-                    af[mi] = A_KMAJOR ? sA[r * BK + k] : sA[k * BM + r];
-                }
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni) {
-                    const int n = wn * 32 + ni * 8 + fr, k = kk + fc;
-                    bf[ni] = B_KMAJOR ? sB[n * BK + k] : sB[k * BN + n];
-                }
-#pragma unroll
-                for (int mi = 0; mi < 4; ++mi)
-#pragma unroll
-                    for (int ni = 0; ni < 4; ++ni) dmma_8x8x4(acc[mi][ni][0], acc[mi][ni][1], af[mi], bf[ni]);
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
-        }
-        // epilogue of item t: C = alpha acc + beta C (K == 0: beta C)
+        const GroupProb* q;
         int64_t tm, tn;
-        group_tile(q, t, tm, tn);
-#pragma unroll
-        for (int mi = 0; mi < 4; ++mi) {
-            const int64_t row = tm * BM + wm * 32 + mi * 8 + fr;
-#pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int64_t col = tn * BN + wn * 32 + ni * 8 + fc * 2;
-                if (row < q.M) {
-                    double* c = q.C + row * q.ldc + col;
-                    if (col + 1 < q.N) {
-                        double2 v;
-                        v.x = q.alpha * acc[mi][ni][0];
-                        v.y = q.alpha * acc[mi][ni][1];
-                        if (q.read_c) {
-                            const double2 o = *reinterpret_cast<const double2*>(c);
-                            v.x += q.beta * o.x;
-                            v.y += q.beta * o.y;
-                        }
-                        *reinterpret_cast<double2*>(c) = v;
-                    } else if (col < q.N) {
-                        double v = q.alpha * acc[mi][ni][0];
-                        if (q.read_c) v += q.beta * c[0];
-                        c[0] = v;
-                    }
-                }
-                acc[mi][ni][0] = acc[mi][ni][1] = 0.0;
-            }
-        }
+        item(t, q, tm, tn);
+        const int64_t row0 = tm * T + (warp >> 1) * W, col0 = tn * T + (warp & 1) * W;
+        if (!consume_tile<A_KMAJOR, B_KMAJOR>(r, acc, (q->K + BK - 1) / BK, q->K, row0 < q->M && col0 < q->N, g.err))
+            return;
+        store_tile<false>(acc, row0, col0, q->M, q->N, q->alpha, q->beta, q->read_c, q->C, q->ldc,
+                             [](int64_t, int64_t) { return true; });
     }
 }
 
 template <bool AK, bool BKM>
 int launch_group_variant(const GroupArgs& a, cudaStream_t st, std::string& why)
 {
-    static int occ = 0, sms = 0;
+    static int occ = 0;
     static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(fp64_group_kernel<AK, BKM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM_BYTES);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fp64_group_kernel<AK, BKM>, THREADS, SMEM_BYTES);
-        sms = device_sm_count();
-    });
-    if (occ <= 0) {
+    const int64_t room = resident_ctas(fp64_group_kernel<AK, BKM>, SMEM_BYTES, occ, once);
+    if (room <= 0) {
         why = "fp64 group kernel cannot be resident (occupancy 0)";
         return OOC_ERR_CUDA;
     }
-    const int64_t grid = std::min<int64_t>(a.tiles > 0 ? a.tiles : 1, (int64_t)occ * sms);
+    const int64_t grid = std::min<int64_t>(a.tiles > 0 ? a.tiles : 1, room);
     fp64_group_kernel<AK, BKM><<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -518,6 +449,16 @@ int launch_group_variant(const GroupArgs& a, cudaStream_t st, std::string& why)
     return OOC_OK;
 }
 
+// Tensor map of one operand: K-major (rows x K) or K down the stored rows, in
+// boxes of T rows by BK of K.
+int operand_map(CUtensorMap* map, bool kmajor, const double* X, int64_t rows, int64_t K, int64_t ld, std::string& why)
+{
+    return kmajor ? encode_map_2d(map, 0, X, (uint64_t)K, (uint64_t)rows, (uint64_t)ld, BK, T, 0, why)
+                  : encode_map_2d(map, 0, X, (uint64_t)rows, (uint64_t)K, (uint64_t)ld, T, BK, 0, why);
+}
+
+int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
 }  // namespace
 
 int launch_fp64_tile(bool a_kmajor, bool b_kmajor, int64_t M, int64_t N, int64_t K, double alpha,
@@ -526,30 +467,24 @@ int launch_fp64_tile(bool a_kmajor, bool b_kmajor, int64_t M, int64_t N, int64_t
                      int64_t tri_off)
 {
     if (M <= 0 || N <= 0) return OOC_OK;
-    static_assert(BM == BN, "the triangular tile map assumes square tiles");
     CUtensorMap ma, mbm;
     std::memset(&ma, 0, sizeof(ma));
     std::memset(&mbm, 0, sizeof(mbm));
     if (K > 0) {
-        int rc = a_kmajor ? encode_map_2d(&ma, 0, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BK, BM, 0, why)
-                          : encode_map_2d(&ma, 0, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM, BK, 0, why);
-        if (rc != OOC_OK) return rc;
-        rc = b_kmajor ? encode_map_2d(&mbm, 0, B, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, BK, BN, 0, why)
-                      : encode_map_2d(&mbm, 0, B, (uint64_t)N, (uint64_t)K, (uint64_t)ldb, BN, BK, 0, why);
+        int rc = operand_map(&ma, a_kmajor, A, M, K, lda, why);
+        if (rc == OOC_OK) rc = operand_map(&mbm, b_kmajor, B, N, K, ldb, why);
         if (rc != OOC_OK) return rc;
     }
     Fp64Args a;
     a.M = M; a.N = N; a.K = K;
-    a.tiles_n = (N + BN - 1) / BN;
-    a.tiles = ((M + BM - 1) / BM) * a.tiles_n;
+    a.tiles_n = cdiv(N, T);
+    a.tiles = cdiv(M, T) * a.tiles_n;
     a.alpha = alpha; a.beta = beta; a.read_c = read_c ? 1 : 0;
     a.C = C; a.ldc = ldc; a.err = err;
     a.tri = tri; a.tri_off = tri_off;
-    a.tt = tri_tiles(tri, tri_off, (M + BM - 1) / BM, a.tiles_n, BM);
-    if (tri) {
-        a.tiles = tri_prefix(a.tt, a.tt.tiles_m);
-        if (a.tiles == 0) return OOC_OK;  // nothing of C is updated
-    }
+    a.tt = tri_tiles(tri, tri_off, cdiv(M, T), a.tiles_n, T);
+    if (tri) a.tiles = tri_prefix(a.tt, a.tt.tiles_m);
+    if (a.tiles == 0) return OOC_OK;  // nothing of C is updated
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (a_kmajor && b_kmajor) return launch_variant<true, true>(ma, mbm, a, st, why);
     if (a_kmajor && !b_kmajor) return launch_variant<true, false>(ma, mbm, a, st, why);
@@ -576,19 +511,16 @@ int launch_fp64_group(bool a_kmajor, bool b_kmajor, const Fp64GroupSpec* probs, 
         if (s.M <= 0 || s.N <= 0) continue;
         GroupProb& q = a.p[n];
         if (s.K > 0) {
-            int rc = a_kmajor ? encode_map_2d(&q.ma, 0, s.A, (uint64_t)s.K, (uint64_t)s.M, (uint64_t)s.lda, BK, BM, 0, why)
-                              : encode_map_2d(&q.ma, 0, s.A, (uint64_t)s.M, (uint64_t)s.K, (uint64_t)s.lda, BM, BK, 0, why);
-            if (rc != OOC_OK) return rc;
-            rc = b_kmajor ? encode_map_2d(&q.mb, 0, s.B, (uint64_t)s.K, (uint64_t)s.N, (uint64_t)s.ldb, BK, BN, 0, why)
-                          : encode_map_2d(&q.mb, 0, s.B, (uint64_t)s.N, (uint64_t)s.K, (uint64_t)s.ldb, BN, BK, 0, why);
+            int rc = operand_map(&q.ma, a_kmajor, s.A, s.M, s.K, s.lda, why);
+            if (rc == OOC_OK) rc = operand_map(&q.mb, b_kmajor, s.B, s.N, s.K, s.ldb, why);
             if (rc != OOC_OK) return rc;
         }
         q.C = s.C; q.ldc = s.ldc;
         q.M = s.M; q.N = s.N; q.K = s.K;
-        q.tiles_n = (s.N + BN - 1) / BN;
+        q.tiles_n = cdiv(s.N, T);
         q.tile_begin = tiles;
         q.alpha = s.alpha; q.beta = s.beta; q.read_c = s.read_c ? 1 : 0;
-        tiles += ((s.M + BM - 1) / BM) * q.tiles_n;
+        tiles += cdiv(s.M, T) * q.tiles_n;
         ++n;
     }
     if (tiles_out) *tiles_out = tiles;
