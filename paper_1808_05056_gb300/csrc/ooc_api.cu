@@ -139,36 +139,13 @@ int encode_map_3d_bf16(void* map_out, const void* base, uint64_t inner, uint64_t
     return OOC_OK;
 }
 
-// The Ozaki groups of the tensor-core kernel: digit products (s, t) with
-// s + t <= S + 1, two consecutive t per group so that the group loads the A
-// plane s once; each product's exact FP32 sum is weighted 2^(-beta (s + t)).
-// Groups sharing a pair of B planes run back to back (t outer, s inner): the
-// tiles in flight then re-read those B planes from L2 rather than DRAM.
-void ozaki_groups(TcProblem& P, int S)
-{
-    int n = 0;
-    for (int t1 = 1; t1 <= S; t1 += 2)
-        for (int s1 = 1; s1 <= S + 1 - t1; ++s1) {
-            TcGroupSpec& g = P.groups[n++];
-            const bool two = t1 + 1 <= S + 1 - s1;
-            g.na = 1; g.nb = two ? 2 : 1; g.np = two ? 2 : 1;
-            g.aplane[0] = s1 - 1;
-            g.bplane[0] = t1 - 1; g.bplane[1] = two ? t1 : 0;
-            g.pa[0] = 0; g.pb[0] = 0;
-            g.pa[1] = 0; g.pb[1] = 1;
-            g.scale_exp = -kOzakiBeta * (s1 + t1);
-            g.scale_exp2 = -kOzakiBeta * (s1 + t1 + 1);
-        }
-    P.ngroups = n;
-}
-
 namespace {
 size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 int64_t up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 size_t side_bytes(int64_t rows, int64_t k_pad, int S)
 {
     const int64_t rp = up(std::max<int64_t>(rows, 1), 128);
-    return al256((size_t)S * rp * k_pad * 2) + al256((size_t)rp * 4) + al256((size_t)rp * 8);
+    return al256((size_t)ozaki_planes(S) * rp * k_pad * 2) + al256((size_t)rp * 4) + al256((size_t)rp * 8);
 }
 }  // namespace
 
@@ -195,6 +172,7 @@ int ozaki_gemm_device(bool a_kmajor, bool b_kmajor, int64_t M, int64_t N, int64_
         return OOC_ERR_BUDGET;
     }
     const int64_t k_pad = up(K, 64);
+    const int planes = ozaki_planes(S);
     char* base = static_cast<char*>(scratch);
     struct Side {
         const double* X;
@@ -208,34 +186,31 @@ int ozaki_gemm_device(bool a_kmajor, bool b_kmajor, int64_t M, int64_t N, int64_
     side[1] = {B, N, b_kmajor ? ldb : 1, b_kmajor ? 1 : ldb, nullptr, nullptr, nullptr, up(N, 128)};
     for (auto& sd : side) {
         sd.planes = base;
-        base += al256((size_t)S * sd.rows_pad * k_pad * 2);
+        base += al256((size_t)planes * sd.rows_pad * k_pad * 2);
         sd.exps = reinterpret_cast<int*>(base);
         base += al256((size_t)sd.rows_pad * 4);
         sd.rowmax = reinterpret_cast<unsigned long long*>(base);
         base += al256((size_t)sd.rows_pad * 8);
         const int rc = launch_split_ozaki(sd.X, sd.sr, sd.sk, (int)sd.rows, (int)K, (int)sd.rows_pad, (int)k_pad,
-                                          S, kOzakiBeta, sd.planes, sd.exps, sd.rowmax, stream, why);
+                                          planes, sd.planes, sd.exps, sd.rowmax, stream, why);
         if (rc) return rc;
     }
-    TcProblem P;
+    OzakiProblem P;
     P.M = M; P.N = N; P.k_pad = k_pad;
-    P.chunk = kOzakiChunk;
-    P.a_planes = side[0].planes; P.a_rows_pad = side[0].rows_pad; P.a_nplanes = S;
-    P.b_planes = side[1].planes; P.b_rows_pad = side[1].rows_pad; P.b_nplanes = S;
-    ozaki_groups(P, S);
+    P.planes = planes;
+    P.a_planes = side[0].planes; P.a_rows_pad = side[0].rows_pad;
+    P.b_planes = side[1].planes; P.b_rows_pad = side[1].rows_pad;
     P.row_exp = side[0].exps;
     P.col_exp = side[1].exps;
     P.alpha = alpha;
     P.beta = beta;
     P.read_c = read_c;
-    P.c_fp32 = false;
     P.C = C;
     P.ldc = ldc;
     P.err = err;
-    P.kblock = 64;
     P.tri = tri;
     P.tri_off = tri_off;
-    return launch_tc_terms(P, stream, why);
+    return launch_ozaki_tiles(P, stream, why);
 }
 
 }  // namespace ooc
@@ -424,7 +399,6 @@ int split_slot(const Plan& p, Exec& x, int src_slot, int dst_slot, bool is_a, in
                std::string& why)
 {
     const bool ozaki = p.form == OOC_FORM_OZAKI;
-    const int S = split_planes(p);
     const int64_t k_pad = split_k_pad(p);
     const int64_t rpad = split_rows_pad(is_a ? p.mb : p.nb);
     void* st = x.smap[kStreamCompute];
@@ -435,11 +409,11 @@ int split_slot(const Plan& p, Exec& x, int src_slot, int dst_slot, bool is_a, in
     const int64_t ld = is_a ? p.lda_dev : p.ldb_dev;
     const int64_t sr = kmajor ? ld : 1, sk = kmajor ? 1 : ld;
     const char* src = x.base + slot_offset(p, src_slot);
-    x.launches += ozaki ? (K > 0 ? 3 : 2) : 1;
+    x.launches += ozaki && K > 0 ? 2 : 1;
     if (ozaki) {
         auto* rowmax = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(exps) + ((rpad * 4 + 255) / 256) * 256);
         return launch_split_ozaki(reinterpret_cast<const double*>(src), sr, sk, (int)nrows, (int)K, (int)rpad,
-                                  (int)k_pad, S, kOzakiBeta, planes, exps, rowmax, st, why);
+                                  (int)k_pad, split_planes(p), planes, exps, rowmax, st, why);
     }
     return launch_split_bf16x3(reinterpret_cast<const float*>(src), sr, sk, (int)nrows, (int)K, (int)rpad, (int)k_pad,
                                planes, st, why);
@@ -455,7 +429,6 @@ int launch_split_tile(const Plan& p, const Op& op, Exec& x, const Operands& o, i
         return OOC_ERR_INVALID_ARG;
     }
     const bool ozaki = p.form == OOC_FORM_OZAKI;
-    const int S = split_planes(p);
     const int64_t rows = p.rows_of(op.i), cols = p.cols_of(op.j), K = p.K > 0 ? p.k_of(op.kc) : 0;  // this chunk
     const int64_t k_pad = split_k_pad(p);
     const int64_t ra_pad = split_rows_pad(p.mb), rb_pad = split_rows_pad(p.nb);
@@ -473,38 +446,36 @@ int launch_split_tile(const Plan& p, const Op& op, Exec& x, const Operands& o, i
         planes[q] = aux;
         exps[q] = reinterpret_cast<int*>(aux + split_planes_bytes(p, sides[q].is_a ? p.mb : p.nb));
     }
-    TcProblem P;
-    P.M = rows; P.N = cols; P.k_pad = K > 0 ? k_pad : 0;
-    P.chunk = ozaki ? kOzakiChunk : kBf16x3Chunk;
-    P.a_planes = planes[0]; P.a_rows_pad = ra_pad; P.a_nplanes = S;
-    P.b_planes = planes[1]; P.b_rows_pad = rb_pad; P.b_nplanes = S;
+    const double beta = op.first ? o.beta : 1.0;
+    const bool read_c = !op.first || o.beta != 0.0, masked = p.block_class(op.i, op.j) == 2;
+    auto common = [&](auto& P) {
+        P.M = rows; P.N = cols; P.k_pad = K > 0 ? k_pad : 0;
+        P.a_planes = planes[0]; P.a_rows_pad = ra_pad;
+        P.b_planes = planes[1]; P.b_rows_pad = rb_pad;
+        P.read_c = read_c;
+        P.ldc = p.ldc_dev;
+        P.err = err;
+        P.tri = masked ? p.tri : 0;
+        P.tri_off = masked ? p.block_off(op.i, op.j) : 0;
+    };
+    ++x.launches;
+    char* C = x.base + slot_offset(p, sc);
     if (ozaki) {
-        ozaki_groups(P, S);
+        OzakiProblem P;
+        common(P);
+        P.planes = split_planes(p);
         P.row_exp = exps[0];
         P.col_exp = exps[1];
-    } else {
-        TcGroupSpec& g = P.groups[0];
-        g.na = 3; g.nb = 3; g.np = 6;
-        for (int i = 0; i < 3; ++i) { g.aplane[i] = i; g.bplane[i] = i; }
-        const int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};  // hh hm mh hl mm lh
-        for (int i = 0; i < 6; ++i) { g.pa[i] = pa[i]; g.pb[i] = pb[i]; }
-        P.ngroups = 1;
-        P.df32 = true;
+        P.alpha = o.alpha; P.beta = beta;
+        P.C = reinterpret_cast<double*>(C);
+        return launch_ozaki_tiles(P, x.smap[kStreamCompute], why);
     }
-    P.alpha = o.alpha;
-    P.beta = op.first ? o.beta : 1.0;
-    P.read_c = !op.first || o.beta != 0.0;
-    P.c_fp32 = p.es == 4;
-    P.C = x.base + slot_offset(p, sc);
-    P.ldc = p.ldc_dev;
-    P.err = err;
-    P.kblock = 64;
-    if (p.block_class(op.i, op.j) == 2) {
-        P.tri = p.tri;
-        P.tri_off = p.block_off(op.i, op.j);
-    }
-    ++x.launches;
-    return launch_tc_terms(P, x.smap[kStreamCompute], why);
+    // ooc_sgemm's alpha and beta are FP32
+    TcProblem P;
+    common(P);
+    P.alpha = (float)o.alpha; P.beta = (float)beta;
+    P.C = reinterpret_cast<float*>(C);
+    return launch_bf16x3_tiles(P, x.smap[kStreamCompute], why);
 }
 
 int launch_tile(const Plan& p, const Op& op, Exec& x, const Operands& o, std::string& why)

@@ -241,73 +241,69 @@ constexpr int kGroupMax = 64;
 int launch_fp64_group(bool a_kmajor, bool b_kmajor, const Fp64GroupSpec* probs, int count, int* err, void* stream,
                       std::string& why, int64_t* tiles_out = nullptr);
 
-// --- tensor-core split-product forms (tc_gemm.cu) -------------------------
-// A group: pairs (A plane, B plane) accumulated into one FP32 TMEM accumulator
-// and added into FP64 with weight 2^scale_exp after every K chunk.
-struct TcGroupSpec {
-    int na = 0, nb = 0, np = 0;
-    int aplane[4] = {0, 0, 0, 0}, bplane[4] = {0, 0, 0, 0};  // planes loaded per K block
-    int pa[6] = {0, 0, 0, 0, 0, 0}, pb[6] = {0, 0, 0, 0, 0, 0};  // pair -> loaded A / B index
-    int scale_exp = 0;   // weight of pair 0's accumulator
-    int scale_exp2 = 0;  // weight of the second accumulator (exact form: pair 1)
-};
-
+// --- BF16x3 form (tc_gemm.cu) ---------------------------------------------
 struct TcProblem {
     int64_t M = 0, N = 0, k_pad = 0;  // C block rows / cols, padded K (multiple of 64)
-    int chunk = 0;                     // K elements per FP64 flush (multiple of 64)
-    const void* a_planes = nullptr;    // [a_nplanes][a_rows_pad][k_pad] bf16
+    const void* a_planes = nullptr;    // [3][a_rows_pad][k_pad] bf16
     int64_t a_rows_pad = 0;
-    int a_nplanes = 0;
-    const void* b_planes = nullptr;    // [b_nplanes][b_rows_pad][k_pad] bf16 (rows = C columns)
+    const void* b_planes = nullptr;    // [3][b_rows_pad][k_pad] bf16 (rows = C columns)
     int64_t b_rows_pad = 0;
-    int b_nplanes = 0;
-    int ngroups = 0;
-    TcGroupSpec groups[64];
-    double alpha = 1.0, beta = 0.0;
-    bool read_c = false, c_fp32 = false;
-    void* C = nullptr;
+    float alpha = 1.0f, beta = 0.0f;
+    bool read_c = false;
+    float* C = nullptr;
     int64_t ldc = 0;
-    const int* row_exp = nullptr;      // per-row power-of-two scale (Ozaki), nullable
-    const int* col_exp = nullptr;
     int* err = nullptr;
-    bool df32 = false;                 // two accumulators per group, double-float drain (BF16x3)
-    int kblock = 64;                   // K block per pipeline stage: 64 or 32
     int tri = 0;                       // epilogue mask as in launch_fp64_tile
     int64_t tri_off = 0;
 };
+int launch_bf16x3_tiles(const TcProblem& P, void* stream, std::string& why);
+int launch_split_bf16x3(const float* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad,
+                        void* planes, void* stream, std::string& why);
 
-int tc_max_groups();
-void ozaki_groups(TcProblem& P, int S);
-// C = alpha op(A) op(B) + beta C on device FP64 operands in the Ozaki form (S
-// digit planes per operand in `scratch`, at least ozaki_device_scratch bytes);
-// operand conventions as launch_fp64_tile.
+// --- Ozaki form (ozaki_gemm.cu) --------------------------------------------
+struct OzakiProblem {
+    int64_t M = 0, N = 0, k_pad = 0;  // C block rows / cols, padded K (multiple of 64)
+    int planes = 0;                    // 8-bit digits per operand (ozaki_planes)
+    const void* a_planes = nullptr;    // [planes][a_rows_pad][k_pad] bf16
+    int64_t a_rows_pad = 0;
+    const void* b_planes = nullptr;    // [planes][b_rows_pad][k_pad] bf16 (rows = C columns)
+    int64_t b_rows_pad = 0;
+    const int* row_exp = nullptr;      // power-of-two scale of each row / column
+    const int* col_exp = nullptr;
+    double alpha = 1.0, beta = 0.0;
+    bool read_c = false;
+    double* C = nullptr;
+    int64_t ldc = 0;
+    int* err = nullptr;
+    int tri = 0;                       // epilogue mask as in launch_fp64_tile
+    int64_t tri_off = 0;
+};
+int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why);
+// `planes` digit planes of an operand and its row exponents (two kernels; one when K == 0)
+int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad, int planes,
+                       void* plane_data, int* rowexp, unsigned long long* rowmax, void* stream, std::string& why);
+
+// C = alpha op(A) op(B) + beta C on device FP64 operands in the Ozaki form (the
+// digit planes of S slices per operand in `scratch`, at least
+// ozaki_device_scratch bytes); operand conventions as launch_fp64_tile.
 size_t ozaki_device_scratch(int64_t M, int64_t N, int64_t K, int S);
 int ozaki_gemm_device(bool a_kmajor, bool b_kmajor, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
                       int64_t lda, const double* B, int64_t ldb, double beta, bool read_c, double* C, int64_t ldc,
                       int S, void* scratch, size_t scratch_bytes, int* err, void* stream, std::string& why, int tri = 0,
                       int64_t tri_off = 0);
-int launch_tc_terms(const TcProblem& P, void* stream, std::string& why);
-int launch_split_bf16x3(const float* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad,
-                        void* planes, void* stream, std::string& why);
-int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad, int S,
-                       int beta, void* planes, int* rowexp, unsigned long long* rowmax, void* stream,
-                       std::string& why);
 int encode_map_3d_bf16(void* map_out, const void* base, uint64_t inner, uint64_t rows, uint64_t planes,
                        uint32_t box_inner, uint32_t box_rows, std::string& why);
 
-// Ozaki digit width and the largest K chunk whose digit products sum exactly in FP32
-constexpr int kOzakiBeta = 6;
-// digits per operand: 8 (48 bits) for the GEMM entry points unless opts->slices
-// asks otherwise; 9 (54 bits, FP64's 53-bit significand covered) for the
-// updates inside the factorizations, whose factors must track FP64's
+// Ozaki slices: opts->slices counts the operands' accuracy in slices of 6 bits --
+// 8 (48 bits) for the GEMM entry points unless the caller asks otherwise; 9 (54
+// bits, FP64's 53-bit significand covered) for the updates inside the
+// factorizations, whose factors must track FP64's.  The kernels hold that many
+// bits in balanced digits of 8 (one bit goes to the sign and comes back by
+// rounding to nearest), so S slices take 3/4 S planes.
 constexpr int kOzakiSlicesGemm = 8;
 constexpr int kOzakiSlicesFactor = 9;
 constexpr int kOzakiMaxSlices = 10;
-constexpr int kOzakiChunk = 4096;
-// BF16x3: K between drains of the leading product's round-toward-zero FP32
-// accumulator (32 accumulations of up to one ulp each: 2^-18 of sum |x||y|)
-constexpr int kBf16x3Chunk = 512;
-
+constexpr int ozaki_planes(int S) { return (3 * S + 3) / 4; }
 int device_sm_count();
 void set_error(const std::string& msg);
 

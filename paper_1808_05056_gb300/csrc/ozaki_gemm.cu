@@ -1,0 +1,830 @@
+// The FP64-accurate Ozaki form on the 5th-generation tensor cores (sm_103a): the
+// compute stage of the out-of-core pipeline for OOC_FORM_OZAKI, after Ozaki, Ogita,
+// Oishi and Rump's error-free splitting of matrix products.
+//
+// Digits.  Every row of A (column of B) is scaled by a power of two 2^e so that its
+// largest entry is below 1 in magnitude; the value, rounded to a fixed-point number
+// of 8 S bits, is cut into S balanced digits of 8 bits, x = 2^(e+1) sum_s d_s 2^(-8 s)
+// with d_s in [-128, 128], each exact in bf16.  Products of digit planes accumulate
+// exactly in FP32 over at most 1024 products of two digits (1024 x 128^2 = 2^24), and
+// the products with s + t <= S + 1 are added with their weight 2^(-8 (s + t)).
+// Eight balanced bits per digit carry what digits of 6 truncated bits (|d| <= 63,
+// the width an exact sum over 4096 needs) carry in 4/3 of the planes: 6 planes and 21
+// products where 8 and 36 were needed, 7 and 28 for 9 and 45.  Rounding to nearest
+// leaves no bias, and the largest dropped product shrinks from 63^2 2^-6(S6+2) to
+// 2^14 2^-(8(S+2)-2), so the error bound of the 6-bit digits holds with room.
+//
+// Sums.  The exact FP32 sums go into one 64-bit fixed-point integer per output (unit
+// 2^-frac, see frac_bits): convert, then one wide multiply-add -- 3 instructions on
+// the integer and conversion pipes.  In FP64 the same drain is bound by the FP64 pipe
+// (1.75 additions a clock and SM: 9400 clocks per 128 x 128 sum, which takes the
+// tensor cores 4096 clocks to make).  Integer sums are exact whatever their order, so
+// the result does not depend on how a tile's work is cut (cut_stages).
+//
+// Kernel shape: tile 128 x 128, 64 of K per stage, 18 warps.
+//   warp 0      TMA producer: the bf16 tiles of one A plane and of two neighbouring B
+//               planes (48 KiB, 128-byte swizzle) into a ring of four stages;
+//   warp 1      allocates all 512 TMEM columns and issues tcgen05.mma: the two B plane
+//               tiles lie back to back, so one N = 256 instruction makes both products
+//               (it reads A once for both: 96 bytes of shared memory a clock instead of
+//               the 128 of two N = 128 ones, which leaves room for the TMA writes);
+//   warps 2-17  drain: finished sums into the 64-bit integers in registers, 32
+//               columns of one row per thread; after the tile's last sum they write
+//               alpha 2^(e_i + f_j) sum + beta C, each store covering 8 rows x 4
+//               consecutive columns (4 x 4 transposes by shuffles).
+// TMEM: two buffers of two 128-column accumulators (neighbouring diagonals s + t).
+//
+// Order of the products: diagonals in pairs (d, d + 1); a group is one A plane s with
+// the B planes d - s and d - s + 1, and one single product (A plane d, B plane 1)
+// completes the pair.  When K is short the groups of a pair share one accumulator
+// pair (their sum is still exact); when it is long each group has its own, drained
+// every 1024 of K.  The host takes whichever drains less often (plan_units).
+//
+// Clusters: when a launch has fewer tiles than SMs, the CTAs of a cluster share each
+// tile.  Each takes a contiguous share of the tile's stages, puts its 64-bit partial
+// sums in shared memory, and the cluster adds them through distributed shared memory.
+// Cluster barriers sit in loops that every thread walks whatever happens, so a CTA
+// whose bounded wait gave up still arrives.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <mutex>
+#include <string>
+
+#include "ooc_internal.hpp"
+#include "tc_common.cuh"
+
+namespace ooc {
+
+namespace {
+
+constexpr int BM = 128, BN = 128, BK = 64;
+constexpr int DIGIT = 8;                              // bits per digit
+constexpr int EXACT_KBLOCKS = 1024 / BK;              // K blocks x products whose FP32 sum stays exact
+constexpr uint32_t TILE_BYTES = BM * BK * 2u;         // one plane tile: 128 rows x 64 bf16 (16 KiB)
+constexpr uint32_t STAGE_BYTES = 3 * TILE_BYTES;      // A plane, two B planes
+constexpr int STAGES = 4;
+constexpr uint32_t RING_BYTES = STAGES * STAGE_BYTES;
+constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + 256;
+constexpr int EPI_WARPS = 16;                         // 4 per TMEM lane quadrant, 32 columns each
+constexpr int THREADS = (2 + EPI_WARPS) * 32;
+constexpr int KSTEPS = BK / 16;
+constexpr int MAX_PLANES = 8;
+constexpr int MAX_GROUPS = 28;                        // 8 planes: 16 double and 4 single groups
+constexpr int MAX_UNITS = MAX_GROUPS;
+constexpr int MAX_CLUSTER = 8;
+static_assert(RING_BYTES >= (uint32_t)BM * BN * 8, "the ring holds a tile of 64-bit partial sums");
+
+// One group: A plane a with B planes b and b + 1 (nb == 2), or with plane b alone, whose
+// product goes into the second accumulator.
+struct Group {
+    int8_t a, b, nb, pad;
+};
+
+// A unit shares one accumulator pair: `ngroups` groups from `first`, drained every
+// `chunk` K blocks.  The two accumulators' weights as a factor applied in FP32 (a
+// power of two; rounds to an integer when it is below one) and a left shift.
+struct Unit {
+    int16_t first, ngroups, chunk, pad;
+    float scale[2];
+    int32_t shift[2];
+};
+
+struct Args {
+    int M, N;
+    int kb0, kblocks;      // K blocks [kb0, kb0 + kblocks) of the planes
+    int tiles_m, tiles_n, tiles;
+    int nunits;
+    int cluster;           // CTAs that share a tile
+    int cut[MAX_CLUSTER + 1];  // CTA r of a cluster takes stages [cut[r], cut[r + 1]) of a tile
+    int frac;              // the integers' unit is 2^-frac
+    double alpha, beta;
+    int read_c;
+    double* C;
+    int64_t ldc;
+    const int* row_exp;
+    const int* col_exp;
+    int* err;
+    int tri;               // 0 full update, 1 lower (col - row <= tri_off), 2 upper (col - row >= tri_off)
+    int64_t tri_off;
+    Unit unit[MAX_UNITS];
+    Group group[MAX_GROUPS];
+};
+
+// Tile order: groups of kRasterRows tile rows, column-major inside a group, so that
+// the tiles in flight at once span few rows and few columns and share their A and B
+// plane tiles in L2.
+constexpr int kRasterRows = 8;
+__device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, int& tm, int& tn)
+{
+    const int per_group = kRasterRows * tiles_n;
+    const int g = tile / per_group, r = tile % per_group;
+    const int first = g * kRasterRows;
+    const int rows = min(tiles_m - first, kRasterRows);
+    tm = first + r % rows;
+    tn = r / rows;
+}
+
+struct Ring {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++s == n) { s = 0; ph ^= 1u; }
+    }
+};
+
+// The stages of a tile that this CTA takes, walked in order by every role: each call
+// of fn(unit, group0, kb0, nk, lo, hi) is one drain -- the stages [lo, hi) of the
+// ngroups x nk block of (group, K block) pairs of one unit and one K chunk.
+template <class Fn>
+__device__ __forceinline__ bool walk(const Args& p, int begin, int end, Fn fn)
+{
+    int pos = 0;
+    for (int u = 0; u < p.nunits; ++u) {
+        const Unit& un = p.unit[u];
+        for (int k0 = 0; k0 < p.kblocks; k0 += un.chunk) {
+            const int nk = min((int)un.chunk, p.kblocks - k0);
+            const int n = un.ngroups * nk;
+            const int lo = max(begin - pos, 0), hi = min(end - pos, n);
+            pos += n;
+            if (lo < hi && !fn(un, k0, nk, lo, hi)) return false;
+            if (pos >= end) return true;
+        }
+    }
+    return true;
+}
+
+// 4 x 4 transpose inside each group of 4 lanes: lane 4g + r holds row r of its
+// group's block in v[0..3] on entry and column r on exit.  Each butterfly stage
+// m swaps the off-diagonal m x m sub-blocks: the lane without bit m trades its
+// elements with bit m set for its partner's elements without it.
+__device__ __forceinline__ void transpose4(double (&v)[4], int lane)
+{
+#pragma unroll
+    for (int m = 2; m >= 1; m >>= 1) {
+        const bool upper = (lane & m) != 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (e & m) continue;
+            const double send = upper ? v[e] : v[e | m];
+            const double got = __shfl_xor_sync(0xffffffffu, send, m);
+            if (upper) v[e] = got;
+            else v[e | m] = got;
+        }
+    }
+}
+
+// t * 2^e, rounded once (to nearest, ties to even) from the 64-bit integer, with
+// integer operations: a conversion and a scaling on the FP64 pipe would take 9400
+// clocks each per tile.  Results outside the normal range go through ldexp.
+__device__ __forceinline__ double fixed_to_f64(long long t, int e)
+{
+    if (t == 0) return 0.0;
+    const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+    const int lz = __clzll((long long)a);
+    const int be = 1023 + 63 - lz + e;  // biased exponent before rounding
+    if (be < 1 || be > 2045) return ldexp((double)t, e);
+    const unsigned long long n = a << lz;          // bit 63 set
+    unsigned long long m = n >> 11;                // 53 bits
+    const unsigned rem = (unsigned)n & 0x7FFu;
+    if (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ++m;
+    // the implicit bit of m (and a carry out of the rounding) adds to the exponent field
+    const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + m;
+    return __longlong_as_double((long long)(bits | (t < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// 64-bit load from the same shared-memory address of CTA `rank` of the cluster
+__device__ __forceinline__ long long ld_cluster(uint32_t addr, uint32_t rank)
+{
+    uint32_t remote;
+    long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(remote) : "memory");
+    return v;
+}
+
+__global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                                const __grid_constant__ CUtensorMap tmB,
+                                                                const __grid_constant__ Args p)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                           ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(ring + RING_BYTES);
+    uint64_t* empty = full + STAGES;
+    uint64_t* acc_full = empty + STAGES;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* done = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, 512);
+        tmem_relinquish();
+    }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], EPI_WARPS);
+        }
+        mbar_init(done, 1);
+        mbar_fence_init();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+
+    const int rank = (int)blockIdx.x % p.cluster;
+    const int first = (int)blockIdx.x / p.cluster, stride = (int)gridDim.x / p.cluster;
+    const int begin = p.cut[rank], end = p.cut[rank + 1];
+
+    Ring r, b;               // stage ring (producer, MMA), accumulator buffers (MMA, drain)
+    uint32_t issued = 0;     // producer: stages issued
+    bool ok = true;
+    const uint32_t idesc2 = idesc_bf16_f32(BM, 2 * BN), idesc1 = idesc_bf16_f32(BM, BN);
+    if (warp == 0 && lane == 0) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+
+    for (int tile = first; tile < p.tiles; tile += stride) {
+        int tm, tn;
+        tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+        if (warp == 0) {
+            // -------------------------------------------- TMA producer
+            if (lane == 0 && ok) {
+                const int arow = tm * BM, brow = tn * BN;
+                ok = walk(p, begin, end, [&](const Unit& un, int k0, int nk, int lo, int hi) {
+                    int gi = lo / nk, kb = lo - gi * nk;
+                    for (int i = lo; i < hi; ++i) {
+                        const Group g = p.group[un.first + gi];
+                        if (!mbar_wait(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) return false;
+                        unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
+                        mbar_arrive_expect_tx(&full[r.s], (1 + g.nb) * TILE_BYTES);
+                        const int x = (p.kb0 + k0 + kb) * BK;
+                        tma_load_3d(st, &tmA, &full[r.s], x, arow, g.a);
+                        tma_load_3d(st + TILE_BYTES, &tmB, &full[r.s], x, brow, g.b);
+                        if (g.nb == 2) tma_load_3d(st + 2 * TILE_BYTES, &tmB, &full[r.s], x, brow, g.b + 1);
+                        r.next(STAGES);
+                        ++issued;
+                        if (++kb == nk) { kb = 0; ++gi; }
+                    }
+                    return true;
+                });
+                if (!ok) {
+                    // let the copies already issued land before the CTA goes on
+                    const uint32_t n = min(issued, (uint32_t)STAGES);
+                    for (uint32_t q = 0; q < n; ++q) {
+                        int s = r.s - 1 - (int)q;
+                        uint32_t ph = r.ph;
+                        if (s < 0) { s += STAGES; ph ^= 1u; }
+                        const uint64_t t0 = globaltimer_ns();
+                        while (!mbar_try_wait(smem_u32(&full[s]), ph) && globaltimer_ns() - t0 < kWaitLimitNs) {
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+        } else if (warp == 1) {
+            // -------------------------------------------- MMA issuer
+            if (lane == 0 && ok) {
+                ok = walk(p, begin, end, [&](const Unit& un, int, int nk, int lo, int hi) {
+                    if (!mbar_wait(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) return false;
+                    tc_fence_after();
+                    const uint32_t d = tmem_base + (uint32_t)b.s * 2 * BN;
+                    int gi = lo / nk, left = nk - (lo - gi * nk);
+                    bool two = p.group[un.first + gi].nb == 2;
+                    uint32_t acc = 0;
+                    for (int i = lo; i < hi; ++i) {
+                        if (!mbar_wait(&full[r.s], r.ph, p.err, kErrWaitFull)) return false;
+                        tc_fence_after();
+                        const uint64_t da = sw128_kmajor_desc(smem_u32(ring + (size_t)r.s * STAGE_BYTES));
+                        const uint64_t db = da + (TILE_BYTES >> 4);
+                        if (two) {
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)
+                                tc_mma_bf16(d, da + 2 * k, db + 2 * k, idesc2, k > 0 ? 1u : acc);
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)
+                                tc_mma_bf16(d + BN, da + 2 * k, db + 2 * k, idesc1, k > 0 ? 1u : acc);
+                        }
+                        acc = 1u;
+                        tc_commit(&empty[r.s]);
+                        r.next(STAGES);
+                        if (--left == 0) {
+                            left = nk;
+                            ++gi;
+                            if (i + 1 < hi) two = p.group[un.first + gi].nb == 2;
+                        }
+                    }
+                    tc_commit(&acc_full[b.s]);
+                    b.next(2);
+                    return true;
+                });
+            }
+            __syncwarp();
+        } else {
+            // -------------------------------------------- drain and epilogue
+            const int q4 = warp & 3;                // TMEM lane quadrant this warp may access
+            const int quarter = (warp - 2) >> 2;    // column quarter of the tile
+            const int row_in_tile = q4 * 32 + lane;
+            const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
+            long long acc[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) acc[j] = 0;
+            if (ok)
+                ok = walk(p, begin, end, [&](const Unit& un, int, int nk, int lo, int) {
+                    // every lane gives up together (the warp shuffles and syncs below need all 32)
+                    if (!__all_sync(0xffffffffu, mbar_wait_backoff(&acc_full[b.s], b.ph, p.err, kErrWaitMma)))
+                        return false;
+                    tc_fence_after();
+                    const uint32_t t0 = tmem_base + lane_off + (uint32_t)(b.s * 2 * BN + quarter * 32);
+                    // the pair's single product comes last: alone, it leaves the first accumulator unused
+                    const int q0 = p.group[un.first + lo / nk].nb == 2 ? 0 : 1;
+#pragma unroll 1
+                    for (int q = q0; q < 2; ++q) {
+                        const float sc = un.scale[q];
+                        const int sh = un.shift[q], mul = 1 << (sh & 31);
+#pragma unroll
+                        for (int cc = 0; cc < 2; ++cc) {
+                            uint32_t v[16];
+                            tmem_ld_32x32b_x16(t0 + q * BN + cc * 16, v);
+                            tmem_wait_ld();
+                            if (sh < 31) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j)
+                                    acc[cc * 16 + j] += (long long)__float2int_rn(__uint_as_float(v[j]) * sc) * mul;
+                            } else {
+                                // a shift of 32 or more reaches the high word only
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) {
+                                    const unsigned hi = (unsigned)__float2int_rn(__uint_as_float(v[j]) * sc) * mul;
+                                    acc[cc * 16 + j] += (long long)((unsigned long long)hi << 32);
+                                }
+                            }
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[b.s]);
+                    b.next(2);
+                    return true;
+                });
+            // the tile's result, 4 columns at a time: each lane forms its own row's values,
+            // transpose4 hands lane 4g + j column j of rows 4g .. 4g + 3, and each store then
+            // covers 8 rows x 4 consecutive columns of C (whole 32-byte sectors)
+            const int64_t row_me = (int64_t)tm * BM + row_in_tile;
+            const int re = (p.row_exp && row_me < p.M ? p.row_exp[row_me] : 0) + 2 - p.frac;  // no exponents when K == 0
+            auto emit = [&](int pass, const long long (&t)[4]) {
+                const int64_t c0 = (int64_t)tn * BN + quarter * 32 + pass * 4;
+                double v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int ce = p.col_exp && c0 + j < p.N ? p.col_exp[c0 + j] : 0;
+                    const double x = fixed_to_f64(t[j], re + ce);
+                    v[j] = p.alpha == 1.0 ? x : p.alpha * x;
+                }
+                transpose4(v, lane);
+                const int64_t col = c0 + (lane & 3), row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
+                if (col >= p.N) return;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t row = row0 + i;
+                    const bool keep = p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off);
+                    if (row < p.M && keep) {
+                        double* c = p.C + row * p.ldc + col;
+                        *c = p.read_c ? fma(p.beta, *c, v[i]) : v[i];
+                    }
+                }
+            };
+            long long* part = reinterpret_cast<long long*>(ring);  // [column][row]
+            if (p.cluster == 1) {
+                if (ok) {
+#pragma unroll
+                    for (int pass = 0; pass < 8; ++pass) {
+                        const long long t[4] = {acc[pass * 4], acc[pass * 4 + 1], acc[pass * 4 + 2], acc[pass * 4 + 3]};
+                        emit(pass, t);
+                    }
+                }
+            } else {
+                // the tile's stages are consumed: its ring carries the partial sums
+                if (ok) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) part[(quarter * 32 + j) * BM + row_in_tile] = acc[j];
+                }
+                cluster_sync();
+                if (ok) {
+                    for (int pass = rank; pass < 8; pass += p.cluster) {
+                        long long t[4] = {0, 0, 0, 0};
+                        const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
+                        for (int q = 0; q < p.cluster; ++q) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) t[j] += ld_cluster(at + j * BM * 8, q);
+                        }
+                        emit(pass, t);
+                    }
+                }
+                // the next tile's copies come after these reads and writes of the ring
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                cluster_sync();
+            }
+        }
+        if (warp < 2 && p.cluster > 1) {
+            cluster_sync();
+            cluster_sync();
+        }
+    }
+    if (warp == 1 && lane == 0) {
+        // every MMA issued so far has completed before TMEM is released
+        tc_commit(done);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(smem_u32(done), 0u) && globaltimer_ns() - t0 < kWaitLimitNs) {
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, 512);
+    }
+}
+
+// ---------------------------------------------------------------- splits --
+// Operand views: element (r, k) of a slot is X[r * sr + k * sk] with either
+// sk == 1 (K-major rows) or sr == 1 (K runs down the stored rows).  Planes are
+// K-major [rows_pad x k_pad] bf16, zero outside rows x K.
+
+constexpr int ST = 64;      // split tile: 64 rows x 64 K
+constexpr int MAX_K = 2048; // K per block of the row-maximum kernel (K-major)
+
+__device__ __forceinline__ unsigned long long abs_bits(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// max |x| over each row (as the bit pattern of a non-negative double, which orders
+// like its value); rowmax must start at zero.  One row and MAX_K of K per block.
+__global__ void __launch_bounds__(256) rowmax_rows_kernel(const double* __restrict__ X, int64_t sr, int K,
+                                                          unsigned long long* __restrict__ rowmax)
+{
+    __shared__ unsigned long long wm[8];
+    const double* x = X + (int64_t)blockIdx.x * sr;
+    unsigned long long m = 0;
+    for (int64_t b = (int64_t)blockIdx.y * MAX_K; b < K; b += (int64_t)gridDim.y * MAX_K) {
+        const int64_t k1 = min((int64_t)K, b + MAX_K);
+#pragma unroll 8
+        for (int64_t k = b + threadIdx.x; k < k1; k += 256) m = max(m, abs_bits(__ldg(x + k)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) m = max(m, wm[w]);
+        if (m) atomicMax(&rowmax[blockIdx.x], m);
+    }
+}
+
+// The same with K down the stored rows: 64 rows and 256 of K per block, one row and
+// 64 of K per thread.
+__global__ void __launch_bounds__(256) rowmax_cols_kernel(const double* __restrict__ X, int64_t sk, int rows, int K,
+                                                          unsigned long long* __restrict__ rowmax)
+{
+    __shared__ unsigned long long t[4][ST];
+    const int c = threadIdx.x & 63, q = threadIdx.x >> 6;
+    const int r = blockIdx.y * ST + c;
+    const int64_t k0 = (int64_t)blockIdx.x * 256, k1 = min((int64_t)K, k0 + 256);
+    unsigned long long m = 0;
+    if (r < rows) {
+#pragma unroll 8
+        for (int64_t k = k0 + q; k < k1; k += 4) m = max(m, abs_bits(__ldg(X + k * sk + r)));
+    }
+    t[q][c] = m;
+    __syncthreads();
+    if (q == 0 && r < rows) {
+        m = max(max(t[0][c], t[1][c]), max(t[2][c], t[3][c]));
+        if (m) atomicMax(&rowmax[r], m);
+    }
+}
+
+// exponent e with max|x| < 2^e (0 for an all-zero row)
+__device__ __forceinline__ int exponent_of(unsigned long long rowmax)
+{
+    if (!rowmax) return 0;
+    const int biased = (int)((rowmax >> 52) & 0x7FF);
+    return (biased ? biased - 1023 : -1022) + 1;
+}
+
+// The fixed-point value x 2^(8 S - 1 - e), rounded to nearest.  |x| < 2^e, so it is at
+// most 2^(8 S - 1) in magnitude; for S = 8 it has no bits to round off at that size
+// and stays below 2^63.
+__device__ __forceinline__ long long fixed_point(double x, int e, int S)
+{
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const int biased = (int)((bits >> 52) & 0x7FF);
+    unsigned long long mant = bits & ((1ull << 52) - 1ull);
+    if (biased) mant |= 1ull << 52;
+    const int ex = biased ? biased - 1023 : -1022;  // |x| = mant * 2^(ex - 52)
+    const int shift = ex - 52 + DIGIT * S - 1 - e;
+    unsigned long long F;
+    if (shift >= 0) F = mant << shift;              // at most DIGIT S - 54 for entries of this row
+    else F = shift > -64 ? (mant + (1ull << (-shift - 1))) >> -shift : 0ull;
+    return (bits >> 63) ? -(long long)F : (long long)F;
+}
+
+// S balanced digits of each element (most significant first): 64 rows x 64 K per
+// block, 8 consecutive K per thread and step, one 16-byte store per plane.
+__global__ void __launch_bounds__(256) split_kernel(const double* __restrict__ X, int64_t sr, int64_t sk, int rows,
+                                                    int K, int rows_pad, int k_pad,
+                                                    const unsigned long long* __restrict__ rowmax, int S,
+                                                    __nv_bfloat16* __restrict__ planes, int* __restrict__ rowexp)
+{
+    __shared__ double t[ST][ST + 1];  // [k][row], operands with K down the stored rows
+    const int r0 = blockIdx.y * ST, k0 = blockIdx.x * ST;
+    if (sk != 1) {
+        const int c = threadIdx.x & 63;
+        for (int i = threadIdx.x >> 6; i < ST; i += 4)
+            t[i][c] = (r0 + c < rows && k0 + i < K) ? __ldg(X + (int64_t)(k0 + i) * sk + r0 + c) : 0.0;
+        __syncthreads();
+    }
+    const size_t plane = (size_t)rows_pad * k_pad;
+    const int g = threadIdx.x & 7;
+    for (int i = threadIdx.x >> 3; i < ST; i += 32) {
+        const int r = r0 + i, k = k0 + g * 8;
+        if (r >= rows_pad || k >= k_pad) continue;
+        const int e = r < rows ? exponent_of(rowmax[r]) : 0;
+        if (k == 0) rowexp[r] = e;
+        long long F[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            double x;
+            if (sk != 1) x = t[g * 8 + j][i];
+            else x = (r < rows && k + j < K) ? __ldg(X + (int64_t)r * sr + k + j) : 0.0;
+            F[j] = fixed_point(x, e, S);
+        }
+        const size_t o = (size_t)r * k_pad + k;
+        for (int s = S - 1; s >= 0; --s) {
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                int d[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // the low 8 bits as a signed digit, the rest carried on; the top digit is what is left
+                    d[h] = s > 0 ? (int)(signed char)(F[j + h] & 0xFF) : (int)F[j + h];
+                    F[j + h] = (F[j + h] - d[h]) >> DIGIT;
+                }
+                const __nv_bfloat162 b = __floats2bfloat162_rn((float)d[0], (float)d[1]);
+                w[j / 2] = *reinterpret_cast<const uint32_t*>(&b);
+            }
+            *reinterpret_cast<uint4*>(planes + (size_t)s * plane + o) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+
+int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Groups and units of a launch (kernel comment, "Order of the products") for S planes
+// and `kblocks` K blocks, and each accumulator's weight: a sum of digit products
+// with s + t = m counts 2^(frac - 8 m) units.
+void plan_units(Args& a, int S)
+{
+    int ng = 0, nu = 0;
+    auto weigh = [&](Unit& u, int q, int m) {
+        // a left shift of the converted sum (below 2^24 in magnitude); 31 would overflow
+        // the multiplier, so the odd power goes into the conversion; below 0: rounded off
+        int sh = a.frac - DIGIT * m;
+        float sc = 1.0f;
+        if (sh < 0) { sc = std::ldexp(1.0f, sh); sh = 0; }
+        else if (sh == 31) { sc = 2.0f; sh = 30; }
+        u.scale[q] = sc;
+        u.shift[q] = sh;
+    };
+    auto add_unit = [&](int first, int n, int chunk, int d) {
+        Unit& u = a.unit[nu++];
+        u.first = (int16_t)first;
+        u.ngroups = (int16_t)n;
+        u.chunk = (int16_t)std::max(1, chunk);
+        weigh(u, 0, d);
+        weigh(u, 1, d + 1);
+    };
+    // diagonals 2 .. S + 1 in pairs (d, d + 1); an odd number of them leaves 2 to itself, a
+    // single product, which a pair (1, 2) describes
+    for (int d = S % 2 ? 1 : 2; d <= S; d += 2) {
+        const int first = ng;
+        for (int s = 1; s < d; ++s) a.group[ng++] = Group{(int8_t)(s - 1), (int8_t)(d - s - 1), 2, 0};
+        a.group[ng++] = Group{(int8_t)(d - 1), 0, 1, 0};
+        const int shared = EXACT_KBLOCKS / d;  // the second accumulator adds d products
+        if (cdiv(a.kblocks, shared) <= d * cdiv(a.kblocks, EXACT_KBLOCKS)) add_unit(first, d, shared, d);
+        else
+            for (int g = first; g < ng; ++g) add_unit(g, 1, EXACT_KBLOCKS, d);
+    }
+    a.nunits = nu;
+}
+
+// Cost of a stage in clocks: the MMAs of one K block of a double or single group (at
+// the rate shared memory lets through) -- only ratios matter here.
+int stage_cost(const Group& g) { return g.nb == 2 ? 2 : 1; }
+
+int64_t tile_cost(const Args& a)
+{
+    int64_t n = 0;
+    for (int u = 0; u < a.nunits; ++u)
+        for (int g = 0; g < a.unit[u].ngroups; ++g) n += stage_cost(a.group[a.unit[u].first + g]);
+    return n * a.kblocks;
+}
+
+// Cut a tile's stages (in walk()'s order) into `cluster` shares of about equal cost; returns
+// the largest.  Sums that are rounded to the integers' unit are cut at drains only, so that
+// what is rounded, and with it the result, does not depend on the cut.
+int64_t cut_stages(Args& a, int cluster, int planes)
+{
+    const bool anywhere = a.frac >= DIGIT * (planes + 1);
+    const int64_t total = tile_cost(a);
+    int64_t cost = 0, largest = 0, begun = 0;
+    int pos = 0, next = 1;
+    a.cut[0] = 0;
+    auto cut = [&](int at, int64_t cost_at) {
+        a.cut[next++] = at;
+        largest = std::max(largest, cost_at - begun);
+        begun = cost_at;
+    };
+    for (int u = 0; u < a.nunits; ++u)
+        for (int k0 = 0; k0 < a.kblocks; k0 += a.unit[u].chunk) {
+            const int nk = std::min<int>(a.unit[u].chunk, a.kblocks - k0);
+            int64_t drain = 0;
+            for (int g = 0; g < a.unit[u].ngroups; ++g) drain += (int64_t)stage_cost(a.group[a.unit[u].first + g]) * nk;
+            while (!anywhere && next < cluster && cost + drain / 2 >= total * next / cluster) cut(pos, cost);
+            for (int g = 0; g < a.unit[u].ngroups; ++g) {
+                const int64_t c = stage_cost(a.group[a.unit[u].first + g]);
+                while (anywhere && next < cluster && cost + c * nk >= total * next / cluster) {
+                    const int64_t n = std::min<int64_t>(nk, (total * next / cluster - cost + c - 1) / c);
+                    cut(pos + (int)n, cost + c * n);
+                }
+                cost += c * nk;
+                pos += nk;
+            }
+        }
+    while (next < cluster) cut(pos, cost);
+    largest = std::max(largest, cost - begun);
+    while (next <= MAX_CLUSTER) a.cut[next++] = pos;
+    return largest;
+}
+
+// Clusters of `n` CTAs of this kernel that the device holds at once (0: none).
+int clusters_at_once(int n)
+{
+    static int count[MAX_CLUSTER + 1] = {0};
+    static std::once_flag once;
+    std::call_once(once, [] {
+        if (cudaFuncSetAttribute(ozaki_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        count[1] = device_sm_count();
+        for (int c = 2; c <= MAX_CLUSTER; c *= 2) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            cfg.gridDim = dim3((unsigned)c);
+            cfg.blockDim = dim3(THREADS);
+            cfg.dynamicSmemBytes = SMEM_BYTES;
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)c;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&count[c], ozaki_tile_kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                count[c] = 0;
+            }
+        }
+    });
+    return count[n];
+}
+
+// CTAs per tile: the size whose busiest cluster finishes first.  The CTAs of a cluster share
+// a tile's stages; the exchange of their partial sums costs about as much as kExchange
+// stages.  Leaves the chosen size and its cuts in `a`.
+constexpr int64_t kExchange = 16;
+void choose_cluster(Args& a, int planes)
+{
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
+        const int n = clusters_at_once(c);
+        if (n <= 0) continue;
+        const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c, planes) + (c > 1 ? kExchange : 0));
+        if (t < cost) { cost = t; best = c; }
+    }
+    a.cluster = best;
+    cut_stages(a, best, planes);
+}
+
+}  // namespace
+
+int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad, int S,
+                       void* planes, int* rowexp, unsigned long long* rowmax, void* stream, std::string& why)
+{
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (cudaMemsetAsync(rowmax, 0, sizeof(unsigned long long) * (size_t)rows_pad, st) != cudaSuccess) {
+        why = "rowmax clear";
+        return OOC_ERR_CUDA;
+    }
+    if (K > 0 && rows > 0) {
+        if (sk == 1)
+            rowmax_rows_kernel<<<dim3((unsigned)rows, (unsigned)std::min<int64_t>(cdiv(K, MAX_K), 65535)), 256, 0,
+                                 st>>>(X, sr, K, rowmax);
+        else
+            rowmax_cols_kernel<<<dim3((unsigned)cdiv(K, 256), (unsigned)cdiv(rows, ST)), 256, 0, st>>>(X, sk, rows, K,
+                                                                                                       rowmax);
+    }
+    split_kernel<<<dim3((unsigned)cdiv(k_pad, ST), (unsigned)cdiv(rows_pad, ST)), 256, 0, st>>>(
+        X, sr, sk, rows, K, rows_pad, k_pad, rowmax, S, static_cast<__nv_bfloat16*>(planes), rowexp);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { why = std::string("split_ozaki: ") + cudaGetErrorString(e); return OOC_ERR_CUDA; }
+    return OOC_OK;
+}
+
+int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
+{
+    if (P.M <= 0 || P.N <= 0) return OOC_OK;
+    if (P.planes < 1 || P.planes > MAX_PLANES) { why = "digit plane count out of range"; return OOC_ERR_INVALID_ARG; }
+    if (P.k_pad % BK) { why = "K padding not a multiple of the K block"; return OOC_ERR_INVALID_ARG; }
+    if (clusters_at_once(1) <= 0) { why = "ozaki tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
+    CUtensorMap ma, mb;
+    std::memset(&ma, 0, sizeof(ma));
+    std::memset(&mb, 0, sizeof(mb));
+    if (P.k_pad > 0) {  // K == 0 runs the epilogue only (C = beta * C)
+        int rc = encode_map_3d_bf16(&ma, P.a_planes, (uint64_t)P.k_pad, (uint64_t)P.a_rows_pad, (uint64_t)P.planes,
+                                    BK, BM, why);
+        if (rc) return rc;
+        rc = encode_map_3d_bf16(&mb, P.b_planes, (uint64_t)P.k_pad, (uint64_t)P.b_rows_pad, (uint64_t)P.planes, BK,
+                                BN, why);
+        if (rc) return rc;
+    }
+    Args a;
+    std::memset(&a, 0, sizeof(a));
+    a.M = (int)P.M; a.N = (int)P.N;
+    a.tiles_m = (int)cdiv(P.M, BM);
+    a.tiles_n = (int)cdiv(P.N, BN);
+    a.tiles = a.tiles_m * a.tiles_n;
+    a.alpha = P.alpha;
+    a.C = P.C; a.ldc = P.ldc;
+    a.row_exp = P.row_exp; a.col_exp = P.col_exp;
+    a.err = P.err;
+    a.tri = P.tri; a.tri_off = P.tri_off;
+    // The integers' unit: |sum| <= (128 / 255)^2 K < 0.253 K, so 2^(64 - ceil(log2 K)) units stay
+    // below 2^62.02.  Sums too fine for it are rounded to it; a longer K goes in stretches of
+    // kStretch (each added into C in FP64) so that the unit stays at or below 2^-46, under what
+    // the dropped products cost.
+    constexpr int64_t kStretch = 1 << 18;
+    const int64_t kb_total = P.k_pad / BK, kb_step = kStretch / BK;
+    for (int64_t kb0 = 0; kb0 == 0 || kb0 < kb_total; kb0 += kb_step) {
+        a.kb0 = (int)kb0;
+        a.kblocks = (int)std::min(kb_step, kb_total - kb0);
+        a.beta = kb0 == 0 ? P.beta : 1.0;
+        a.read_c = kb0 == 0 ? (P.read_c ? 1 : 0) : 1;
+        int lg = 6;
+        while (((int64_t)1 << lg) < (int64_t)a.kblocks * BK) ++lg;
+        a.frac = 64 - lg;
+        plan_units(a, P.planes);
+        choose_cluster(a, P.planes);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        cfg.gridDim = dim3((unsigned)(std::min(a.tiles, clusters_at_once(a.cluster)) * a.cluster));
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = SMEM_BYTES;
+        cfg.stream = static_cast<cudaStream_t>(stream);
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)a.cluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel, ma, mb, a);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            why = std::string("ozaki tile launch: ") + cudaGetErrorString(e);
+            return OOC_ERR_CUDA;
+        }
+    }
+    return OOC_OK;
+}
+
+}  // namespace ooc

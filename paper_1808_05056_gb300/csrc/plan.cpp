@@ -66,11 +66,12 @@ FormModel form_model(int form, int es, int64_t K, int slices_opt)
         // copies beside tensor-core kernels share HBM and the power budget: 65536^3 with 309 GB
         // H2D (1.46 s at the link rate) ran 2.84 s steps on 2.45 s of kernel-stream time
         f.overlap_cost = 0.27;
-    } else {  // Ozaki (measured 1.39-1.40 PFLOP/s bf16)
+    } else {  // Ozaki
         int s = slices_opt > 0 ? slices_opt : kOzakiSlicesGemm;
         f.tile_m = 128; f.tile_n = 128; f.ctas_per_sm = 1;
         f.slices = s; f.products = s * (s + 1) / 2;
-        f.rate = 1.38e15 / f.products;
+        const int planes = ozaki_planes(s);
+        f.rate = 1.38e15 / (planes * (planes + 1) / 2);
         f.overlap_cost = 0.27;
     }
     (void)es; (void)K;
@@ -79,7 +80,7 @@ FormModel form_model(int form, int es, int64_t K, int slices_opt)
 
 }  // namespace
 
-int split_planes(const Plan& p) { return p.form == OOC_FORM_BF16X3 ? 3 : p.slices; }
+int split_planes(const Plan& p) { return p.form == OOC_FORM_BF16X3 ? 3 : ozaki_planes(p.slices); }
 int64_t split_rows_pad(int64_t rows) { return round_up(std::max<int64_t>(rows, 1), 128); }
 int64_t split_k_pad(const Plan& p) { return round_up(p.kb, 64); }
 size_t split_planes_bytes(const Plan& p, int64_t rows)
