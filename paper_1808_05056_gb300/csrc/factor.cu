@@ -36,62 +36,95 @@ namespace {
 
 constexpr int kSmall = 64;     // order of the triangular blocks the small kernels take
 
-// Solve Tm x = alpha p for nvec vectors p of n <= 64 elements, where
-// Tm[r][c] = T[c][r] if t_trans else T[r][c], lower or upper triangular (only
-// that triangle of the stored T is read), unit diagonal (not read) or not.
-// Element e of vector v lives at P[e * es + v * vs].  kVecs right-hand sides
-// per CTA, one per thread (the launcher picks 128, 64 or 32 so that the grid
-// still fills the SMs).
-template <int kVecs>
-__global__ void __launch_bounds__(kVecs) trsm_small_kernel(const double* __restrict__ T, int64_t ldt, int n,
-                                                           int t_trans, int lower, int unit, double* P, int64_t es,
-                                                           int64_t vs, int64_t nvec, double alpha)
+// x = s / d from the reciprocal `inv` of d (Markstein's correction: the residual of
+// the rounded product is exact in a fused multiply-add, and adding it back rounds to
+// the quotient): three instructions on the FP64 pipe, which a division would hold for
+// about twenty.  `inv` is NaN where the correction could leave the normal range
+// (reciprocal_of); a quotient near the ends of it goes through the division too.
+__device__ __forceinline__ double quotient(double s, double d, double inv)
 {
-    // dynamic shared memory (above the 48 KB static limit): the block, then the vectors
-    extern __shared__ double smem_f64[];
-    double (*Ts)[kSmall + 1] = reinterpret_cast<double (*)[kSmall + 1]>(smem_f64);
-    double (*Xs)[kSmall + 1] = reinterpret_cast<double (*)[kSmall + 1]>(smem_f64 + kSmall * (kSmall + 1));
+    const double q = s * inv;
+    const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 0x7FFu;
+    if (e - 64u < 0x780u) return fma(fma(-q, d, s), inv, q);
+    if ((__double_as_longlong(s) << 1) == 0 && inv == inv) return q;  // zero over a regular divisor
+    return s / d;
+}
+
+__device__ __forceinline__ double reciprocal_of(double d)
+{
+    const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
+    return e - 64u < 0x780u ? 1.0 / d : __longlong_as_double(0x7FF8000000000000ll);
+}
+
+// Solve Tm x = p for nvec vectors p of n <= 64 elements, where Tm[r][c] = T[c][r] if
+// t_trans else T[r][c], lower or upper triangular (only that triangle of the stored T
+// is used), unit diagonal (not used) or not.  Element e of vector v lives at
+// P[e * es + v * vs].
+//
+// FP64 instructions are what this kernel is made of (one every 19 clocks and SM,
+// whatever the number of active lanes), so it counts them: L lanes share a vector,
+// each with 64 / L of its elements in registers, and after element r is known every
+// lane subtracts its column r from what it still has to solve.  A warp spends 192
+// instructions on 64 quotients and 32 (64 / L + 1) on the updates for its 32 / L
+// vectors: few lanes per vector cost the fewest instructions in all, many lanes
+// spread few vectors over the chip (the launcher picks L).  An upper system is solved
+// as a lower one with the elements taken backwards.
+constexpr int kTrsmThreads = 128;
+template <int L>
+__global__ void __launch_bounds__(kTrsmThreads) trsm_small_kernel(const double* __restrict__ T, int64_t ldt, int n,
+                                                                  int t_trans, int lower, int unit, double* P,
+                                                                  int64_t es, int64_t vs, int64_t nvec)
+{
+    constexpr int R = kSmall / L, LD = kSmall + 1;
+    __shared__ double Tc[kSmall * LD];  // [column][row] of the lower system, zero elsewhere
+    __shared__ double dg[kSmall], inv[kSmall];
     const int tid = threadIdx.x;
-    const int64_t v0 = (int64_t)blockIdx.x * kVecs;
-    for (int idx = tid; idx < n * n; idx += blockDim.x) {
-        const int r = idx / n, c = idx % n;
+#pragma unroll 8
+    for (int idx = tid; idx < kSmall * kSmall; idx += kTrsmThreads) {
+        const int sr = idx >> 6, sc = idx & 63;  // stored row and column: columns fastest for coalescing
+        int r = t_trans ? sc : sr, c = t_trans ? sr : sc;
+        const bool in = sr < n && sc < n;
+        if (!lower && in) { r = n - 1 - r; c = n - 1 - c; }
         double t = 0.0;
-        if (r == c) t = unit ? 1.0 : T[(int64_t)r * ldt + c];
-        else if (lower ? c < r : c > r) t = t_trans ? T[(int64_t)c * ldt + r] : T[(int64_t)r * ldt + c];
-        Ts[r][c] = t;
-    }
-    // stage the vectors, the unit-stride index fastest for coalescing
-    const bool v_fast = vs == 1;
-    for (int idx = tid; idx < n * kVecs; idx += blockDim.x) {
-        const int e = v_fast ? idx / kVecs : idx % n;
-        const int v = v_fast ? idx % kVecs : idx / n;
-        if (v0 + v < nvec) Xs[v][e] = P[(int64_t)e * es + (v0 + v) * vs];
-    }
-    __syncthreads();
-    if (v0 + tid < nvec) {
-        // one right-hand side per thread; four partial sums break the dependent FMA chain
-        double* x = Xs[tid];
-        for (int q = 0; q < n; ++q) {
-            const int r = lower ? q : n - 1 - q;
-            const int c0 = lower ? 0 : r + 1, c1 = lower ? r : n;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int c = c0;
-            for (; c + 3 < c1; c += 4) {
-                s0 = fma(Ts[r][c], x[c], s0);
-                s1 = fma(Ts[r][c + 1], x[c + 1], s1);
-                s2 = fma(Ts[r][c + 2], x[c + 2], s2);
-                s3 = fma(Ts[r][c + 3], x[c + 3], s3);
-            }
-            for (; c < c1; ++c) s0 = fma(Ts[r][c], x[c], s0);
-            const double s = alpha * x[r] - ((s0 + s1) + (s2 + s3));
-            x[r] = unit ? s : s / Ts[r][r];
+        if (in && (r > c || (r == c && !unit))) t = T[(int64_t)sr * ldt + sc];
+        Tc[c * LD + r] = t;
+        if (r == c) {
+            dg[r] = t;
+            inv[r] = unit || !in ? 1.0 : reciprocal_of(t);
         }
     }
+    const int warp = tid >> 5, lane = tid & 31, l = lane & (L - 1);
+    const int64_t v = ((int64_t)blockIdx.x * (kTrsmThreads / 32) + warp) * (32 / L) + lane / L;
+    double x[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int i = j * L + l, e = lower ? i : n - 1 - i;
+        x[j] = i < n && v < nvec ? P[e * es + v * vs] : 0.0;
+    }
     __syncthreads();
-    for (int idx = tid; idx < n * kVecs; idx += blockDim.x) {
-        const int e = v_fast ? idx / kVecs : idx % n;
-        const int v = v_fast ? idx % kVecs : idx / n;
-        if (v0 + v < nvec) P[(int64_t)e * es + (v0 + v) * vs] = Xs[v][e];
+#pragma unroll
+    for (int jr = 0; jr < R; ++jr) {
+        const int lr_end = min(L, n - jr * L);
+#pragma unroll 1
+        for (int lr = 0; lr < lr_end; ++lr) {
+            const int r = jr * L + lr;
+            const double q = unit ? x[jr] : quotient(x[jr], dg[r], inv[r]);
+            const double xr = __shfl_sync(0xffffffffu, q, lr, L);
+            const double* t = Tc + r * LD + l;
+            if (L > 1) {
+                const double u = fma(-t[jr * L], xr, x[jr]);
+                x[jr] = l > lr ? u : (l == lr ? q : x[jr]);
+            } else {
+                x[jr] = q;
+            }
+#pragma unroll
+            for (int j = jr + 1; j < R; ++j) x[j] = fma(-t[j * L], xr, x[j]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int i = j * L + l, e = lower ? i : n - 1 - i;
+        if (i < n && v < nvec) P[e * es + v * vs] = x[j];
     }
 }
 
@@ -356,28 +389,41 @@ __global__ void scale_kernel(double* P, int64_t ld, int64_t rows, int64_t cols, 
     }
 }
 
-template <int kVecs>
-constexpr size_t trsm_smem() { return (size_t)(kSmall + kVecs) * (kSmall + 1) * sizeof(double); }
-
-template <int kVecs>
-int launch_trsm_small(const double* T, int64_t ldt, int n, bool t_trans, bool lower, bool unit, double* P,
-                      int64_t es, int64_t vs, int64_t nv, cudaStream_t st, std::string& why)
+template <int L>
+int launch_trsm_lanes(const double* T, int64_t ldt, int n, bool t_trans, bool lower, bool unit, double* P, int64_t es,
+                      int64_t vs, int64_t nv, cudaStream_t st, std::string& why)
 {
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        trsm_small_kernel<kVecs>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem<kVecs>());
-    if (attr != cudaSuccess) {
-        why = std::string("trsm_small_kernel shared memory: ") + cudaGetErrorString(attr);
-        return OOC_ERR_CUDA;
-    }
-    const int64_t grid = (nv + kVecs - 1) / kVecs;
-    trsm_small_kernel<kVecs><<<(unsigned)grid, kVecs, trsm_smem<kVecs>(), st>>>(
-        T, ldt, n, t_trans ? 1 : 0, lower ? 1 : 0, unit ? 1 : 0, P, es, vs, nv, 1.0);
+    const int64_t per_cta = kTrsmThreads / L;
+    trsm_small_kernel<L><<<(unsigned)((nv + per_cta - 1) / per_cta), kTrsmThreads, 0, st>>>(
+        T, ldt, n, t_trans ? 1 : 0, lower ? 1 : 0, unit ? 1 : 0, P, es, vs, nv);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         why = std::string("trsm_small_kernel: ") + cudaGetErrorString(e);
         return OOC_ERR_CUDA;
     }
     return OOC_OK;
+}
+
+// Lanes per vector: the count whose busiest SM has the fewest FP64 instructions to issue
+// (its CTAs times the instructions of a warp).
+int launch_trsm_small(const double* T, int64_t ldt, int n, bool t_trans, bool lower, bool unit, double* P, int64_t es,
+                      int64_t vs, int64_t nv, cudaStream_t st, std::string& why)
+{
+    const int64_t sms = device_sm_count();
+    int best = 32;
+    int64_t cost = INT64_MAX;
+    for (int L = 32; L >= 2; L /= 2) {
+        const int64_t ctas = (nv * L + kTrsmThreads - 1) / kTrsmThreads;
+        const int64_t c = (ctas + sms - 1) / sms * (192 + 32 * (kSmall / L + 1));
+        if (c < cost) { cost = c; best = L; }
+    }
+    switch (best) {
+    case 32: return launch_trsm_lanes<32>(T, ldt, n, t_trans, lower, unit, P, es, vs, nv, st, why);
+    case 16: return launch_trsm_lanes<16>(T, ldt, n, t_trans, lower, unit, P, es, vs, nv, st, why);
+    case 8: return launch_trsm_lanes<8>(T, ldt, n, t_trans, lower, unit, P, es, vs, nv, st, why);
+    case 4: return launch_trsm_lanes<4>(T, ldt, n, t_trans, lower, unit, P, es, vs, nv, st, why);
+    default: return launch_trsm_lanes<2>(T, ldt, n, t_trans, lower, unit, P, es, vs, nv, st, why);
+    }
 }
 
 int check_launch(const char* what, std::string& why)
@@ -448,14 +494,8 @@ int incore_trsm(bool left, bool op_lower, const double* T, int64_t ldt, bool t_t
         const bool tm_lower = left ? op_lower : !op_lower;
         const bool tm_trans = left ? t_trans : !t_trans;
         const int64_t es = left ? ldp : 1, vs = left ? 1 : ldp;
-        // the most right-hand sides per CTA (more warps per SM) that still gives two CTAs per SM
-        const int64_t want = 2 * (int64_t)device_sm_count();
         ++d.launches;
-        if ((nv + 127) / 128 >= want)
-            return launch_trsm_small<128>(T, ldt, (int)n, tm_trans, tm_lower, unit, P, es, vs, nv, d.st, why);
-        if ((nv + 63) / 64 >= want)
-            return launch_trsm_small<64>(T, ldt, (int)n, tm_trans, tm_lower, unit, P, es, vs, nv, d.st, why);
-        return launch_trsm_small<32>(T, ldt, (int)n, tm_trans, tm_lower, unit, P, es, vs, nv, d.st, why);
+        return launch_trsm_small(T, ldt, (int)n, tm_trans, tm_lower, unit, P, es, vs, nv, d.st, why);
     }
     const int64_t n1 = split_point(n), n2 = n - n1;
     const double* T11 = T;
