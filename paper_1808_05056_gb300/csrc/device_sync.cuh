@@ -127,6 +127,23 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* map)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// Barrier of a thread-block cluster; every thread of every CTA arrives.  It has no time
+// limit: callers keep it in code that all of them reach whatever a bounded wait returned.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// 64-bit load from the same shared-memory address of CTA `rank` of the cluster
+__device__ __forceinline__ long long ld_cluster(uint32_t addr, uint32_t rank)
+{
+    uint32_t remote;
+    long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(remote) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ bool launch_failed(const int* err)
 {
     return *reinterpret_cast<const volatile int*>(err) != 0;

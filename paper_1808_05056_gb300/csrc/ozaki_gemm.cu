@@ -52,7 +52,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <string>
 
 #include "ooc_internal.hpp"
@@ -115,29 +114,6 @@ struct Args {
     Group group[MAX_GROUPS];
 };
 
-// Tile order: groups of kRasterRows tile rows, column-major inside a group, so that
-// the tiles in flight at once span few rows and few columns and share their A and B
-// plane tiles in L2.
-constexpr int kRasterRows = 8;
-__device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, int& tm, int& tn)
-{
-    const int per_group = kRasterRows * tiles_n;
-    const int g = tile / per_group, r = tile % per_group;
-    const int first = g * kRasterRows;
-    const int rows = min(tiles_m - first, kRasterRows);
-    tm = first + r % rows;
-    tn = r / rows;
-}
-
-struct Ring {
-    int s = 0;
-    uint32_t ph = 0;
-    __device__ __forceinline__ void next(int n)
-    {
-        if (++s == n) { s = 0; ph ^= 1u; }
-    }
-};
-
 // The stages of a tile that this CTA takes, walked in order by every role: each call
 // of fn(unit, group0, kb0, nk, lo, hi) is one drain -- the stages [lo, hi) of the
 // ngroups x nk block of (group, K block) pairs of one unit and one K chunk.
@@ -159,26 +135,6 @@ __device__ __forceinline__ bool walk(const Args& p, int begin, int end, Fn fn)
     return true;
 }
 
-// 4 x 4 transpose inside each group of 4 lanes: lane 4g + r holds row r of its
-// group's block in v[0..3] on entry and column r on exit.  Each butterfly stage
-// m swaps the off-diagonal m x m sub-blocks: the lane without bit m trades its
-// elements with bit m set for its partner's elements without it.
-__device__ __forceinline__ void transpose4(double (&v)[4], int lane)
-{
-#pragma unroll
-    for (int m = 2; m >= 1; m >>= 1) {
-        const bool upper = (lane & m) != 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (e & m) continue;
-            const double send = upper ? v[e] : v[e | m];
-            const double got = __shfl_xor_sync(0xffffffffu, send, m);
-            if (upper) v[e] = got;
-            else v[e | m] = got;
-        }
-    }
-}
-
 // t * 2^e, rounded once (to nearest, ties to even) from the 64-bit integer, with
 // integer operations: a conversion and a scaling on the FP64 pipe would take 9400
 // clocks each per tile.  Results outside the normal range go through ldexp.
@@ -196,21 +152,6 @@ __device__ __forceinline__ double fixed_to_f64(long long t, int e)
     // the implicit bit of m (and a carry out of the rounding) adds to the exponent field
     const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + m;
     return __longlong_as_double((long long)(bits | (t < 0 ? 0x8000000000000000ull : 0ull)));
-}
-
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// 64-bit load from the same shared-memory address of CTA `rank` of the cluster
-__device__ __forceinline__ long long ld_cluster(uint32_t addr, uint32_t rank)
-{
-    uint32_t remote;
-    long long v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(remote) : "memory");
-    return v;
 }
 
 __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -687,48 +628,16 @@ int64_t cut_stages(Args& a, int cluster, int planes)
     return largest;
 }
 
-// Clusters of `n` CTAs of this kernel that the device holds at once (0: none).
-int clusters_at_once(int n)
-{
-    static int count[MAX_CLUSTER + 1] = {0};
-    static std::once_flag once;
-    std::call_once(once, [] {
-        if (cudaFuncSetAttribute(ozaki_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        count[1] = device_sm_count();
-        for (int c = 2; c <= MAX_CLUSTER; c *= 2) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at[1];
-            cfg.gridDim = dim3((unsigned)c);
-            cfg.blockDim = dim3(THREADS);
-            cfg.dynamicSmemBytes = SMEM_BYTES;
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = (unsigned)c;
-            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&count[c], ozaki_tile_kernel, &cfg) != cudaSuccess) {
-                cudaGetLastError();
-                count[c] = 0;
-            }
-        }
-    });
-    return count[n];
-}
-
 // CTAs per tile: the size whose busiest cluster finishes first.  The CTAs of a cluster share
 // a tile's stages; the exchange of their partial sums costs about as much as kExchange
 // stages.  Leaves the chosen size and its cuts in `a`.
 constexpr int64_t kExchange = 16;
-void choose_cluster(Args& a, int planes)
+void choose_cluster(Args& a, int planes, const ClusterCounts& counts)
 {
     int best = 1;
     int64_t cost = INT64_MAX;
     for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
-        const int n = clusters_at_once(c);
+        const int n = counts.at_once[c];
         if (n <= 0) continue;
         const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c, planes) + (c > 1 ? kExchange : 0));
         if (t < cost) { cost = t; best = c; }
@@ -767,7 +676,8 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     if (P.M <= 0 || P.N <= 0) return OOC_OK;
     if (P.planes < 1 || P.planes > MAX_PLANES) { why = "digit plane count out of range"; return OOC_ERR_INVALID_ARG; }
     if (P.k_pad % BK) { why = "K padding not a multiple of the K block"; return OOC_ERR_INVALID_ARG; }
-    if (clusters_at_once(1) <= 0) { why = "ozaki tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
+    static const ClusterCounts counts = count_clusters((const void*)ozaki_tile_kernel, THREADS, SMEM_BYTES);
+    if (counts.at_once[1] <= 0) { why = "ozaki tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
     CUtensorMap ma, mb;
     std::memset(&ma, 0, sizeof(ma));
     std::memset(&mb, 0, sizeof(mb));
@@ -805,18 +715,11 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
         while (((int64_t)1 << lg) < (int64_t)a.kblocks * BK) ++lg;
         a.frac = 64 - lg;
         plan_units(a, P.planes);
-        choose_cluster(a, P.planes);
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        cfg.gridDim = dim3((unsigned)(std::min(a.tiles, clusters_at_once(a.cluster)) * a.cluster));
-        cfg.blockDim = dim3(THREADS);
-        cfg.dynamicSmemBytes = SMEM_BYTES;
-        cfg.stream = static_cast<cudaStream_t>(stream);
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)a.cluster;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
+        choose_cluster(a, P.planes, counts);
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, SMEM_BYTES,
+                       static_cast<cudaStream_t>(stream));
         const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel, ma, mb, a);
         if (e != cudaSuccess) {
             cudaGetLastError();

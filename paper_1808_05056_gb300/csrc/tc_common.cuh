@@ -12,8 +12,10 @@
 #pragma once
 #include <cstdint>
 #include <cuda.h>
+#include <cuda_runtime.h>
 
 #include "device_sync.cuh"
+#include "ooc_internal.hpp"
 
 namespace ooc {
 
@@ -138,6 +140,92 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
         " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
+}
+
+// --- shared by the tile kernels of both forms ------------------------------
+// Tile order: groups of kRasterRows tile rows, column-major inside a group, so that
+// the tiles in flight at once span few rows and few columns and share their A and B
+// plane tiles in L2.
+constexpr int kRasterRows = 8;
+__device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, int& tm, int& tn)
+{
+    const int per_group = kRasterRows * tiles_n;
+    const int g = tile / per_group, r = tile % per_group;
+    const int first = g * kRasterRows;
+    const int rows = min(tiles_m - first, kRasterRows);
+    tm = first + r % rows;
+    tn = r / rows;
+}
+
+// ring position: slot and pass parity, advanced without division
+struct Ring {
+    int s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++s == n) { s = 0; ph ^= 1u; }
+    }
+};
+
+// 4 x 4 transpose inside each group of 4 lanes: lane 4g + r holds row r of its
+// group's block in v[0..3] on entry and column r on exit.  Each butterfly stage
+// m swaps the off-diagonal m x m sub-blocks: the lane without bit m trades its
+// elements with bit m set for its partner's elements without it.
+__device__ __forceinline__ void transpose4(double (&v)[4], int lane)
+{
+#pragma unroll
+    for (int m = 2; m >= 1; m >>= 1) {
+        const bool upper = (lane & m) != 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (e & m) continue;
+            const double send = upper ? v[e] : v[e | m];
+            const double got = __shfl_xor_sync(0xffffffffu, send, m);
+            if (upper) v[e] = got;
+            else v[e | m] = got;
+        }
+    }
+}
+
+// How many clusters of 1, 2, 4 and 8 CTAs of a kernel the device holds at once (0: none);
+// sets the kernel's shared-memory limit.
+struct ClusterCounts {
+    int at_once[9] = {0};
+};
+
+inline void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, int clusters, int threads,
+                           size_t smem, cudaStream_t st)
+{
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * cluster));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+inline ClusterCounts count_clusters(const void* kernel, int threads, size_t smem)
+{
+    ClusterCounts n;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return n;
+    }
+    n.at_once[1] = device_sm_count();
+    for (int c = 2; c <= 8; c *= 2) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        cluster_config(cfg, at, c, 1, threads, smem, nullptr);
+        if (cudaOccupancyMaxActiveClusters(&n.at_once[c], kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n.at_once[c] = 0;
+        }
+    }
+    return n;
 }
 
 }  // namespace ooc

@@ -13,35 +13,43 @@
 // sub-partitions): draining hh every 128 of K took enough of that thread's issue
 // slots to cost a fifth of the tensor-core rate.
 //
-// Kernel shape: persistent CTAs, one per SM, tile 128 x 128.
+// Kernel shape: tile 128 x 128, 18 warps, persistent CTAs (one per SM).
 //   warp 0      TMA producer: for each K block of 64 loads the three plane tiles of
 //               A and of B (96 KiB, 128-byte swizzle) into a ring of two stages;
-//   warp 1      allocates all 512 TMEM columns and issues tcgen05.mma (M=128,
-//               N=128, K=16), committing stage releases and accumulator-full
-//               events to mbarriers;
+//   warp 1      allocates all 512 TMEM columns and issues tcgen05.mma, committing
+//               stage releases and accumulator-full events to mbarriers;
 //   warps 2-17  epilogue: drain finished accumulators with tcgen05.ld into packed
 //               double-float FP32 registers, 32 columns of one row per thread,
 //               release them, and after the last chunk write alpha * acc + beta *
 //               C_old, each store covering 8 rows x 4 consecutive columns (4 x 4
 //               transposes by shuffles inside groups of 4 lanes).
-// TMEM: three buffers for hh and one accumulator for the small products.
 //
-// The single issuing thread keeps its per-stage work to the MMAs themselves
-// (descriptor offsets are constants, ring positions advance without division): at
-// 64 cycles per 128 x 128 x 16 MMA, anything more starves the tensor pipe.  For the
-// same reason the ring releases whole stages: finer slots (one 16 KiB plane tile
-// each, with a wait and a release per tile) ran at half the rate.  CTA pairs
-// (cta_group::2, 256 x 128 tiles with half of each B tile per CTA) were measured
-// slower on GB300 (1216 vs 1384 bf16 TFLOP/s) and are not built.  Every wait is
-// bounded (device_sync.cuh); the epilogue warps wait with a sleep between tries so
-// that they leave the issue slots to the TMA and MMA threads.
+// Instructions: the B planes h and m lie back to back in a stage, so one N = 256
+// instruction multiplies an A plane by both; h l and l h take N = 128 ones.  Four
+// instructions per 16 of K instead of six, and 104 bytes of operands read from shared
+// memory per clock instead of 128, which leaves room for the TMA writes.
+// TMEM: leading accumulators X0 and X1 used in turn, with two small-product ones, Y0
+// and Y1, between them (columns X0 Y0 Y1 X1).  h x (h, m) fills X0 and Y0 in one chunk;
+// in the next the stage holds the planes in the order (m, h) and the same instruction
+// fills Y1 and X1.  m x (h, m) fills both Y.
+//
+// Clusters: when a launch has fewer tiles than SMs, the CTAs of a cluster share each
+// tile's K blocks and add their double-float partial sums, in rank order, through
+// distributed shared memory.  Cluster barriers sit in loops that every thread walks
+// whatever happens, so a CTA whose bounded wait gave up still arrives.
+//
+// The ring releases whole stages: finer slots (one 16 KiB plane tile each, with a wait
+// and a release per tile) ran at half the rate.  CTA pairs (cta_group::2, 256 x 128
+// tiles with half of each B tile per CTA) were measured slower (1216 vs 1384 bf16
+// TFLOP/s) and are not built.  Every wait is bounded (device_sync.cuh); the epilogue
+// warps wait with a sleep between tries so that they leave the issue slots to the TMA
+// and MMA threads.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 #include <string>
 
 #include "ooc_internal.hpp"
@@ -59,19 +67,21 @@ constexpr uint32_t RING_BYTES = STAGES * STAGE_BYTES;
 constexpr int EPI_WARPS = 16;                         // 4 per TMEM lane quadrant, 32 columns each
 constexpr int THREADS = (2 + EPI_WARPS) * 32;
 constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + 1024;
-constexpr int NBUF = 3;                               // TMEM buffers of the leading product
-constexpr int PRODUCTS = 6;
 constexpr int KSTEPS = BK / 16;
 // K blocks between drains of the leading product's round-toward-zero accumulator (512:
 // 32 accumulations of up to one ulp each, 2^-18 of sum |x||y|) and chunks between
 // drains of the small products' (2048 of K)
 constexpr int CHUNK_KBLOCKS = 512 / BK;
 constexpr int SMALL_EVERY = 4;
-constexpr uint32_t kSmallCol = 384;                   // TMEM column of the small-product accumulator
+// TMEM columns: X0 Y0 Y1 X1
+constexpr uint32_t kX0 = 0, kY0 = BN, kY1 = 2 * BN, kX1 = 3 * BN;
+constexpr int MAX_CLUSTER = 8;
+static_assert(RING_BYTES >= (uint32_t)BM * BN * 8, "the ring holds a tile of double-float partial sums");
 
 struct TcArgs {
     int M, N;
-    int kblocks, nchunks;
+    int kblocks;
+    int cluster;      // CTAs that share a tile's K blocks
     int tiles_m, tiles_n, tiles;
     float alpha, beta;
     int read_c;
@@ -81,20 +91,6 @@ struct TcArgs {
     int tri;          // 0 full update, 1 lower (col - row <= tri_off), 2 upper (col - row >= tri_off)
     int64_t tri_off;
 };
-
-// Tile order: groups of kRasterRows tile rows, column-major inside a group, so
-// that the tiles in flight at once span few rows and few columns and share
-// their A and B plane tiles in L2.
-constexpr int kRasterRows = 8;
-__device__ __forceinline__ void tile_coords(int tile, int tiles_m, int tiles_n, int& tm, int& tn)
-{
-    const int per_group = kRasterRows * tiles_n;
-    const int g = tile / per_group, r = tile % per_group;
-    const int first = g * kRasterRows;
-    const int rows = min(tiles_m - first, kRasterRows);
-    tm = first + r % rows;
-    tn = r / rows;
-}
 
 // Packed pairs of FP32 values (element 2j in the low half): Blackwell's f32x2
 // arithmetic does two of the drain's additions per instruction.
@@ -113,63 +109,40 @@ __device__ __forceinline__ uint64_t f2sub(uint64_t a, uint64_t b)
 __device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 __device__ __forceinline__ float unpack2(uint64_t v, int j) { return __uint_as_float((uint32_t)(v >> (32 * j))); }
 
-// ring position: slot and pass parity, advanced without division
-struct Ring {
-    int s = 0;
-    uint32_t ph = 0;
-    __device__ __forceinline__ void next(int n)
-    {
-        if (++s == n) { s = 0; ph ^= 1u; }
-    }
-};
-
-// 4 x 4 transpose inside each group of 4 lanes: lane 4g + r holds row r of its
-// group's block in v[0..3] on entry and column r on exit.  Each butterfly stage
-// m swaps the off-diagonal m x m sub-blocks: the lane without bit m trades its
-// elements with bit m set for its partner's elements without it.
-__device__ __forceinline__ void transpose4(double (&v)[4], int lane)
-{
-#pragma unroll
-    for (int m = 2; m >= 1; m >>= 1) {
-        const bool upper = (lane & m) != 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (e & m) continue;
-            const double send = upper ? v[e] : v[e | m];
-            const double got = __shfl_xor_sync(0xffffffffu, send, m);
-            if (upper) v[e] = got;
-            else v[e | m] = got;
-        }
-    }
-}
-
-// Drains of the small-product accumulator: every SMALL_EVERY chunks and at the last
+// Drains of the small-product accumulators: every SMALL_EVERY chunks and at the last
 // chunk of a tile (both the MMA issuer and the epilogue use this)
 __device__ __forceinline__ bool small_drain_after(int c, int nchunks)
 {
     return c == nchunks - 1 || (c % SMALL_EVERY) == SMALL_EVERY - 1;
 }
 
+// (hi, lo) += (h, l): the sum of the leading parts exactly (TwoSum), its error with the rest
+__device__ __forceinline__ void add_double_float(float& hi, float& lo, float h, float l)
+{
+    const float s = __fadd_rn(hi, h), bp = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(l, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(h, bp))));
+    hi = s;
+}
+
 __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                  const __grid_constant__ CUtensorMap tmB,
                                                                  const __grid_constant__ TcArgs p)
 {
-    constexpr uint32_t kTmemCols = 512;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(ring + RING_BYTES);
     uint64_t* empty = full + STAGES;
     uint64_t* acc_full = empty + STAGES;
-    uint64_t* acc_empty = acc_full + NBUF;
-    uint64_t* small_full = acc_empty + NBUF;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* small_full = acc_empty + 2;
     uint64_t* small_empty = small_full + 1;
-    uint64_t* drain = small_empty + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    uint64_t* done = small_empty + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 1) {
-        tmem_alloc(tmem_slot, kTmemCols);
+        tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
     }
     if (threadIdx.x == 0) {
@@ -177,13 +150,13 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < NBUF; ++b) {
+        for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], EPI_WARPS);
         }
         mbar_init(small_full, 1);
         mbar_init(small_empty, EPI_WARPS);
-        mbar_init(drain, 1);
+        mbar_init(done, 1);
         mbar_fence_init();
     }
     tc_fence_before();
@@ -191,95 +164,115 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int64_t my_tiles =
-        p.tiles > (int)blockIdx.x ? (p.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int rank = (int)blockIdx.x % p.cluster;
+    const int first = (int)blockIdx.x / p.cluster, stride = (int)gridDim.x / p.cluster;
+    const int kb0 = (int)((int64_t)p.kblocks * rank / p.cluster), kb1 = (int)((int64_t)p.kblocks * (rank + 1) / p.cluster);
+    const int nchunks = (kb1 - kb0 + CHUNK_KBLOCKS - 1) / CHUNK_KBLOCKS;
 
-    if (warp == 0) {
-        // ------------------------------------------------ TMA producer
-        if (lane == 0) {
-            tma_prefetch_desc(&tmA);
-            tma_prefetch_desc(&tmB);
-            Ring r;
-            uint32_t issued = 0;
-            bool ok = true;
-            for (int64_t tl = 0; tl < my_tiles && ok; ++tl) {
-                const int tile = (int)blockIdx.x + (int)tl * (int)gridDim.x;
-                int tm, tn;
-                tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
-                const int arow = tm * BM, brow = tn * BN;
-                for (int kb = 0; kb < p.kblocks; ++kb) {
-                    if (!mbar_wait(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) { ok = false; break; }
-                    unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
-                    mbar_arrive_expect_tx(&full[r.s], STAGE_BYTES);
-                    for (int a = 0; a < 3; ++a) tma_load_3d(st + a * A_TILE, &tmA, &full[r.s], kb * BK, arow, a);
-                    for (int b = 0; b < 3; ++b) tma_load_3d(st + (3 + b) * A_TILE, &tmB, &full[r.s], kb * BK, brow, b);
-                    r.next(STAGES);
-                    ++issued;
+    Ring r, b;                   // stage ring (producer, MMA); leading accumulators in turn (producer, MMA, epilogue)
+    uint32_t issued = 0;         // producer: stages issued
+    uint32_t small_drains = 0;   // drains of the small accumulators so far (MMA, epilogue)
+    bool small_pending = false;  // MMA: one not yet released by the epilogue
+    bool ok = true;
+    const uint32_t idesc2 = idesc_bf16_f32(BM, 2 * BN), idesc1 = idesc_bf16_f32(BM, BN);
+    if (warp == 0 && lane == 0) {
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+
+    for (int tile = first; tile < p.tiles; tile += stride) {
+        int tm, tn;
+        tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
+        if (warp == 0) {
+            // -------------------------------------------- TMA producer
+            if (lane == 0 && ok) {
+                for (int c = 0; c < nchunks && ok; ++c) {
+                    const int end = min(kb1, kb0 + (c + 1) * CHUNK_KBLOCKS);
+                    for (int kb = kb0 + c * CHUNK_KBLOCKS; kb < end; ++kb) {
+                        if (!mbar_wait(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) { ok = false; break; }
+                        unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
+                        mbar_arrive_expect_tx(&full[r.s], STAGE_BYTES);
+                        for (int a = 0; a < 3; ++a)
+                            tma_load_3d(st + a * A_TILE, &tmA, &full[r.s], kb * BK, tm * BM, a);
+                        // B planes (h, m, l) beside X0, (m, h, l) beside X1
+                        tma_load_3d(st + 3 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, b.s);
+                        tma_load_3d(st + 4 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 1 - b.s);
+                        tma_load_3d(st + 5 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 2);
+                        r.next(STAGES);
+                        ++issued;
+                    }
+                    b.next(2);
                 }
-            }
-            if (!ok) {
-                // let the copies already issued land before the CTA exits
-                const uint32_t n = min(issued, (uint32_t)STAGES);
-                for (uint32_t q = 0; q < n; ++q) {
-                    int s = r.s - 1 - (int)q;
-                    uint32_t ph = r.ph;
-                    while (s < 0) { s += STAGES; ph ^= 1u; }
-                    const uint64_t t0 = globaltimer_ns();
-                    while (!mbar_try_wait(smem_u32(&full[s]), ph) && globaltimer_ns() - t0 < kWaitLimitNs) {
+                if (!ok) {
+                    // let the copies already issued land before the CTA goes on
+                    const uint32_t n = min(issued, (uint32_t)STAGES);
+                    for (uint32_t q = 0; q < n; ++q) {
+                        int s = r.s - 1 - (int)q;
+                        uint32_t ph = r.ph;
+                        if (s < 0) { s += STAGES; ph ^= 1u; }
+                        const uint64_t t0 = globaltimer_ns();
+                        while (!mbar_try_wait(smem_u32(&full[s]), ph) && globaltimer_ns() - t0 < kWaitLimitNs) {
+                        }
                     }
                 }
             }
-        }
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32(BM, BN);
-            Ring r, b;
-            uint32_t small_drains = 0;   // small-accumulator drains committed so far
-            bool small_pending = false;  // a drain committed and not yet released by the epilogue
-            bool ok = true;
-            // products hh hm mh hl mm lh: the stage's A and B plane of each
-            constexpr int pa[PRODUCTS] = {0, 0, 1, 0, 1, 2}, pb[PRODUCTS] = {0, 1, 0, 2, 1, 0};
-            for (int64_t tl = 0; tl < my_tiles && ok; ++tl) {
-                uint32_t small_acc = 0;  // accumulate flag of the small-product accumulator
-                for (int c = 0; c < p.nchunks && ok; ++c) {
-                    const int kb0 = c * CHUNK_KBLOCKS, kb1 = min(p.kblocks, kb0 + CHUNK_KBLOCKS);
+            __syncwarp();
+        } else if (warp == 1) {
+            // -------------------------------------------- MMA issuer
+            if (lane == 0 && ok) {
+                uint32_t small_acc = 0;  // accumulate flag of the small-product accumulators
+                for (int c = 0; c < nchunks && ok; ++c) {
+                    const int end = min(kb1, kb0 + (c + 1) * CHUNK_KBLOCKS);
                     if (!mbar_wait(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) { ok = false; break; }
+                    if (small_pending) {
+                        // the epilogue has read the small accumulators before they restart
+                        if (!mbar_wait(small_empty, (small_drains - 1) & 1u, p.err, kErrWaitAcc)) { ok = false; break; }
+                        small_pending = false;
+                    }
                     tc_fence_after();
-                    const uint32_t d0 = tmem_base + (uint32_t)b.s * BN;
-                    uint32_t acc0 = 0;
-                    for (int kb = kb0; kb < kb1; ++kb) {
+                    // h x (h, m) -> (X0, Y0) or h x (m, h) -> (Y1, X1)
+                    const uint32_t dh = tmem_base + (b.s ? kY1 : kX0), dy = tmem_base + kY0;
+                    const uint32_t dlead = tmem_base + (b.s ? kX1 : kX0), dsmall = tmem_base + (b.s ? kY1 : kY0);
+                    const uint32_t bh = (uint32_t)(3 + b.s) * (A_TILE >> 4);  // plane h of B
+                    bool fresh = true;
+                    for (int kb = kb0 + c * CHUNK_KBLOCKS; kb < end; ++kb) {
                         if (!mbar_wait(&full[r.s], r.ph, p.err, kErrWaitFull)) { ok = false; break; }
                         tc_fence_after();
-                        const uint64_t dst = sw128_kmajor_desc(smem_u32(ring + (size_t)r.s * STAGE_BYTES));
-                        if (small_pending) {
-                            // the epilogue has read the small accumulator before it restarts
-                            if (!mbar_wait(small_empty, (small_drains - 1) & 1u, p.err, kErrWaitAcc)) {
-                                ok = false;
-                                break;
-                            }
-                            tc_fence_after();
-                            small_pending = false;
-                        }
+                        const uint64_t A = sw128_kmajor_desc(smem_u32(ring + (size_t)r.s * STAGE_BYTES));
+                        constexpr uint32_t T = A_TILE >> 4;
+                        // both small accumulators start with m x (h, m)
 #pragma unroll
-                        for (int q = 0; q < PRODUCTS; ++q) {
-                            // hh into buffer d0, the others into the small accumulator
-                            const uint32_t d = q == 0 ? d0 : tmem_base + kSmallCol;
-                            uint32_t& flag = q == 0 ? acc0 : small_acc;
-                            const uint64_t da = dst + (((uint32_t)pa[q] * A_TILE) >> 4);
-                            const uint64_t db = dst + (((uint32_t)(3 + pb[q]) * A_TILE) >> 4);
+                        for (int k = 0; k < KSTEPS; ++k)
+                            tc_mma_bf16(dy, A + T + 2 * k, A + 3 * T + 2 * k, idesc2, k > 0 ? 1u : small_acc);
+                        small_acc = 1u;
+                        if (fresh) {
+                            // the chunk's first h x h restarts the leading accumulator, which an
+                            // N = 256 instruction cannot do without restarting its neighbour
 #pragma unroll
                             for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(d, da + 2 * k, db + 2 * k, idesc, k > 0 ? 1u : flag);
-                            flag = 1u;
+                                tc_mma_bf16(dlead, A + 2 * k, A + bh + 2 * k, idesc1, k > 0 ? 1u : 0u);
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)
+                                tc_mma_bf16(dsmall, A + 2 * k, A + (7 * T - bh) + 2 * k, idesc1, 1u);
+                            fresh = false;
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)
+                                tc_mma_bf16(dh, A + 2 * k, A + 3 * T + 2 * k, idesc2, 1u);
                         }
+#pragma unroll
+                        for (int k = 0; k < KSTEPS; ++k)  // h x l
+                            tc_mma_bf16(dy, A + 2 * k, A + 5 * T + 2 * k, idesc1, 1u);
+#pragma unroll
+                        for (int k = 0; k < KSTEPS; ++k)  // l x h
+                            tc_mma_bf16(dy, A + 2 * T + 2 * k, A + bh + 2 * k, idesc1, 1u);
                         tc_commit(&empty[r.s]);
                         r.next(STAGES);
                     }
                     if (!ok) break;
                     tc_commit(&acc_full[b.s]);
-                    b.next(NBUF);
-                    if (small_drain_after(c, p.nchunks)) {
+                    b.next(2);
+                    if (small_drain_after(c, nchunks)) {
                         tc_commit(small_full);
                         ++small_drains;
                         small_pending = true;
@@ -287,35 +280,24 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     }
                 }
             }
-            // every MMA issued so far has completed before TMEM is released
-            tc_commit(drain);
-            const uint64_t t0 = globaltimer_ns();
-            while (!mbar_try_wait(smem_u32(drain), 0u) && globaltimer_ns() - t0 < kWaitLimitNs) {
-            }
-        }
-    } else {
-        // ------------------------------------------------ epilogue warps
-        const int q4 = warp & 3;                 // TMEM lane quadrant this warp may access
-        const int quarter = (warp - 2) >> 2;    // column quarter of the tile
-        const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
-        uint64_t hi2[16], lo2[16];  // a packed double-float (hi, lo) per output
+            __syncwarp();
+        } else {
+            // -------------------------------------------- epilogue warps
+            const int q4 = warp & 3;                 // TMEM lane quadrant this warp may access
+            const int quarter = (warp - 2) >> 2;    // column quarter of the tile
+            const int row_in_tile = q4 * 32 + lane;
+            const uint32_t lane_off = ((uint32_t)(q4 * 32) << 16) + (uint32_t)(quarter * 32);
+            uint64_t hi2[16], lo2[16];  // a packed double-float (hi, lo) per output
 #pragma unroll
-        for (int j = 0; j < 16; ++j) hi2[j] = lo2[j] = 0ull;
-        Ring b;
-        uint32_t small_drains = 0;
-        bool ok = true;
-        for (int64_t tl = 0; tl < my_tiles && ok; ++tl) {
-            const int tile = (int)blockIdx.x + (int)tl * (int)gridDim.x;
-            int tm, tn;
-            tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
-            for (int c = 0; c < p.nchunks && ok; ++c) {
+            for (int j = 0; j < 16; ++j) hi2[j] = lo2[j] = 0ull;
+            for (int c = 0; c < nchunks && ok; ++c) {
                 // every lane gives up together (the warp shuffles and syncs below need all 32)
                 if (!__all_sync(0xffffffffu, mbar_wait_backoff(&acc_full[b.s], b.ph, p.err, kErrWaitMma))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t t0 = tmem_base + lane_off + (uint32_t)b.s * BN + (uint32_t)(quarter * 32);
+                const uint32_t t0 = tmem_base + lane_off + (b.s ? kX1 : kX0);
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) {
                     uint32_t v[8];
@@ -336,8 +318,8 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[b.s]);
-                b.next(NBUF);
-                if (small_drain_after(c, p.nchunks)) {
+                b.next(2);
+                if (small_drain_after(c, nchunks)) {
                     // the small products (2^-8 of hh and below) go straight into lo
                     if (!__all_sync(0xffffffffu,
                                     mbar_wait_backoff(small_full, small_drains & 1u, p.err, kErrWaitMma))) {
@@ -345,15 +327,14 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t ts = tmem_base + lane_off + kSmallCol + (uint32_t)(quarter * 32);
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
+                    for (int cc = 0; cc < 8; ++cc) {
                         uint32_t v[8];
-                        tmem_ld_32x32b_x8(ts + cc * 8, v);
+                        tmem_ld_32x32b_x8(tmem_base + lane_off + (cc < 4 ? kY0 : kY1) + (cc & 3) * 8, v);
                         tmem_wait_ld();
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            lo2[cc * 4 + j] = f2add(lo2[cc * 4 + j], pack2(v[2 * j], v[2 * j + 1]));
+                            lo2[(cc & 3) * 4 + j] = f2add(lo2[(cc & 3) * 4 + j], pack2(v[2 * j], v[2 * j + 1]));
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -361,64 +342,107 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     ++small_drains;
                 }
             }
-            if (!ok) break;
-            // final epilogue of this tile, 4 columns at a time: each lane forms its own row's
-            // values, transpose4 hands lane 4g + j column j of rows 4g .. 4g + 3, and each store
-            // then covers 8 rows x 4 consecutive columns of C.  alpha * (hi + lo) + beta * C_old
-            // in FP32 double-float steps (TwoSum, products split with fma), rounded once at the
+            // the tile's result, 4 columns at a time: each lane forms its own row's values,
+            // transpose4 hands lane 4g + j column j of rows 4g .. 4g + 3, and each store then
+            // covers 8 rows x 4 consecutive columns of C.  alpha * (hi + lo) + beta * C_old in
+            // FP32 double-float steps (TwoSum, products split with fma), rounded once at the
             // end: on this part the FP64 pipe would take ~18 us per tile for it, holding the
             // accumulators the MMAs wait for
-            const int64_t row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
-#pragma unroll
-            for (int pass = 0; pass < 8; ++pass) {
+            auto emit = [&](int pass, const float (&h)[4], const float (&l)[4]) {
                 const int64_t c0 = (int64_t)tn * BN + quarter * 32 + pass * 4;
                 double v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int jj = pass * 4 + j;
                     // (ph, pl) = alpha * (hi + lo), packed
-                    const float hi = unpack2(hi2[jj >> 1], jj & 1), lo = unpack2(lo2[jj >> 1], jj & 1);
-                    const float sh = __fadd_rn(hi, lo), bp = __fsub_rn(sh, hi);
-                    const float sl = __fadd_rn(__fsub_rn(hi, __fsub_rn(sh, bp)), __fsub_rn(lo, bp));
+                    const float sh = __fadd_rn(h[j], l[j]), bp = __fsub_rn(sh, h[j]);
+                    const float sl = __fadd_rn(__fsub_rn(h[j], __fsub_rn(sh, bp)), __fsub_rn(l[j], bp));
                     const float ph = __fmul_rn(p.alpha, sh);
                     const float pl = __fmaf_rn(p.alpha, sl, __fmaf_rn(p.alpha, sh, -ph));
                     v[j] = __longlong_as_double((long long)pack2(__float_as_uint(ph), __float_as_uint(pl)));
                 }
                 transpose4(v, lane);
-                const int64_t col = c0 + (lane & 3);
-                if (col < p.N) {
+                const int64_t col = c0 + (lane & 3), row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
+                if (col >= p.N) return;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int64_t row = row0 + i;
-                        const bool keep =
-                            p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off);
-                        if (row < p.M && keep) {
-                            const uint64_t b = (uint64_t)__double_as_longlong(v[i]);
-                            const float ph = unpack2(b, 0), pl = unpack2(b, 1);
-                            float* cp = p.C + row * p.ldc + col;
-                            if (p.read_c) {
-                                // beta * c = qh + ql and ph + qh = th + tl exactly; one rounding left
-                                const float c = *cp;
-                                const float qh = __fmul_rn(p.beta, c), ql = __fmaf_rn(p.beta, c, -qh);
-                                const float th = __fadd_rn(ph, qh), bq = __fsub_rn(th, ph);
-                                const float tl = __fadd_rn(__fsub_rn(ph, __fsub_rn(th, bq)), __fsub_rn(qh, bq));
-                                *cp = __fadd_rn(th, __fadd_rn(tl, __fadd_rn(pl, ql)));
-                            } else {
-                                *cp = __fadd_rn(ph, pl);
-                            }
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t row = row0 + i;
+                    const bool keep = p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off);
+                    if (row < p.M && keep) {
+                        const uint64_t w = (uint64_t)__double_as_longlong(v[i]);
+                        const float ph = unpack2(w, 0), pl = unpack2(w, 1);
+                        float* cp = p.C + row * p.ldc + col;
+                        if (p.read_c) {
+                            // beta * c = qh + ql and ph + qh = th + tl exactly; one rounding left
+                            const float old = *cp;
+                            const float qh = __fmul_rn(p.beta, old), ql = __fmaf_rn(p.beta, old, -qh);
+                            const float th = __fadd_rn(ph, qh), bq = __fsub_rn(th, ph);
+                            const float tl = __fadd_rn(__fsub_rn(ph, __fsub_rn(th, bq)), __fsub_rn(qh, bq));
+                            *cp = __fadd_rn(th, __fadd_rn(tl, __fadd_rn(pl, ql)));
+                        } else {
+                            *cp = __fadd_rn(ph, pl);
                         }
                     }
                 }
-            }
+            };
+            if (p.cluster == 1) {
+                if (ok) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) hi2[j] = lo2[j] = 0ull;
+                    for (int pass = 0; pass < 8; ++pass) {
+                        float h[4], l[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            h[j] = unpack2(hi2[pass * 2 + (j >> 1)], j & 1);
+                            l[j] = unpack2(lo2[pass * 2 + (j >> 1)], j & 1);
+                        }
+                        emit(pass, h, l);
+                    }
+                }
+            } else {
+                // the tile's stages are consumed: its ring carries the partial sums, [column][row]
+                uint64_t* part = reinterpret_cast<uint64_t*>(ring);
+                if (ok) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        part[(quarter * 32 + j) * BM + row_in_tile] =
+                            pack2(__float_as_uint(unpack2(hi2[j >> 1], j & 1)), __float_as_uint(unpack2(lo2[j >> 1], j & 1)));
+                }
+                cluster_sync();
+                if (ok) {
+                    for (int pass = rank; pass < 8; pass += p.cluster) {
+                        float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+                        const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
+                        for (int q = 0; q < p.cluster; ++q) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint64_t w = (uint64_t)ld_cluster(at + j * BM * 8, q);
+                                add_double_float(h[j], l[j], unpack2(w, 0), unpack2(w, 1));
+                            }
+                        }
+                        emit(pass, h, l);
+                    }
+                }
+                // the next tile's copies come after these reads and writes of the ring
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                cluster_sync();
+            }
+        }
+        if (warp < 2 && p.cluster > 1) {
+            cluster_sync();
+            cluster_sync();
+        }
+    }
+    if (warp == 1 && lane == 0) {
+        // every MMA issued so far has completed before TMEM is released
+        tc_commit(done);
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(smem_u32(done), 0u) && globaltimer_ns() - t0 < kWaitLimitNs) {
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(tmem_base, 512);
     }
 }
 
@@ -512,8 +536,20 @@ __global__ void __launch_bounds__(256) split_bf16x3_rows_kernel(const float* __r
     *reinterpret_cast<uint4*>(planes + 2 * plane + o) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
 
-std::once_flag g_attr_once;
-int g_sms = 0;
+// CTAs per tile: the size whose busiest cluster finishes first, in K blocks; the exchange
+// of the partial sums costs about as much as kExchange of them.
+constexpr int64_t kExchange = 4;
+int cluster_size(const ClusterCounts& n, int64_t tiles, int64_t kblocks)
+{
+    int best = 1;
+    int64_t cost = INT64_MAX;
+    for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
+        if (n.at_once[c] <= 0) continue;
+        const int64_t t = (tiles + n.at_once[c] - 1) / n.at_once[c] * ((kblocks + c - 1) / c + (c > 1 ? kExchange : 0));
+        if (t < cost) { cost = t; best = c; }
+    }
+    return best;
+}
 
 }  // namespace
 
@@ -538,16 +574,13 @@ int launch_split_bf16x3(const float* X, int64_t sr, int64_t sk, int rows, int K,
 int launch_bf16x3_tiles(const TcProblem& P, void* stream, std::string& why)
 {
     if (P.M <= 0 || P.N <= 0) return OOC_OK;
-    std::call_once(g_attr_once, [] {
-        cudaFuncSetAttribute(bf16x3_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-        g_sms = device_sm_count();
-    });
+    static const ClusterCounts counts = count_clusters((const void*)bf16x3_tile_kernel, THREADS, SMEM_BYTES);
+    if (counts.at_once[1] <= 0) { why = "bf16x3 tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
     if (P.k_pad % BK) { why = "K padding not a multiple of the K block"; return OOC_ERR_INVALID_ARG; }
     TcArgs a;
     std::memset(&a, 0, sizeof(a));
     a.M = (int)P.M; a.N = (int)P.N;
     a.kblocks = (int)(P.k_pad / BK);
-    a.nchunks = (a.kblocks + CHUNK_KBLOCKS - 1) / CHUNK_KBLOCKS;
     a.tiles_n = (int)((P.N + BN - 1) / BN);
     a.tiles_m = (int)((P.M + BM - 1) / BM);
     a.tiles = a.tiles_m * a.tiles_n;
@@ -565,9 +598,13 @@ int launch_bf16x3_tiles(const TcProblem& P, void* stream, std::string& why)
         rc = encode_map_3d_bf16(&mb, P.b_planes, (uint64_t)P.k_pad, (uint64_t)P.b_rows_pad, 3, BK, BN, why);
         if (rc) return rc;
     }
-    const int grid = std::min(a.tiles, g_sms > 0 ? g_sms : 152);
-    bf16x3_tile_kernel<<<grid, THREADS, SMEM_BYTES, static_cast<cudaStream_t>(stream)>>>(ma, mb, a);
-    cudaError_t e = cudaGetLastError();
+    a.cluster = cluster_size(counts, a.tiles, a.kblocks);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, SMEM_BYTES,
+                   static_cast<cudaStream_t>(stream));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, bf16x3_tile_kernel, ma, mb, a);
+    if (e != cudaSuccess) cudaGetLastError();
     if (e != cudaSuccess) { why = std::string("bf16x3 tile launch: ") + cudaGetErrorString(e); return OOC_ERR_CUDA; }
     return OOC_OK;
 }
