@@ -168,7 +168,8 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
     uint64_t* done = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the shuffle tells the compiler that the warp index is the same in all lanes
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
@@ -198,7 +199,8 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
     uint32_t issued = 0;     // producer: stages issued
     bool ok = true;
     const uint32_t idesc2 = idesc_bf16_f32(BM, 2 * BN), idesc1 = idesc_bf16_f32(BM, BN);
-    if (warp == 0 && lane == 0) {
+    const bool leader = elect_one();  // the lane that issues copies and MMAs
+    if (warp == 0 && leader) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
@@ -208,19 +210,21 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
         tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
         if (warp == 0) {
             // -------------------------------------------- TMA producer
-            if (lane == 0 && ok) {
+            if (ok) {
                 const int arow = tm * BM, brow = tn * BN;
                 ok = walk(p, begin, end, [&](const Unit& un, int k0, int nk, int lo, int hi) {
                     int gi = lo / nk, kb = lo - gi * nk;
                     for (int i = lo; i < hi; ++i) {
                         const Group g = p.group[un.first + gi];
-                        if (!mbar_wait(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) return false;
-                        unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
-                        mbar_arrive_expect_tx(&full[r.s], (1 + g.nb) * TILE_BYTES);
-                        const int x = (p.kb0 + k0 + kb) * BK;
-                        tma_load_3d(st, &tmA, &full[r.s], x, arow, g.a);
-                        tma_load_3d(st + TILE_BYTES, &tmB, &full[r.s], x, brow, g.b);
-                        if (g.nb == 2) tma_load_3d(st + 2 * TILE_BYTES, &tmB, &full[r.s], x, brow, g.b + 1);
+                        if (!wait_warp(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) return false;
+                        if (leader) {
+                            unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
+                            mbar_arrive_expect_tx(&full[r.s], (1 + g.nb) * TILE_BYTES);
+                            const int x = (p.kb0 + k0 + kb) * BK;
+                            tma_load_3d(st, &tmA, &full[r.s], x, arow, g.a);
+                            tma_load_3d(st + TILE_BYTES, &tmB, &full[r.s], x, brow, g.b);
+                            if (g.nb == 2) tma_load_3d(st + 2 * TILE_BYTES, &tmB, &full[r.s], x, brow, g.b + 1);
+                        }
                         r.next(STAGES);
                         ++issued;
                         if (++kb == nk) { kb = 0; ++gi; }
@@ -240,33 +244,29 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     }
                 }
             }
-            __syncwarp();
         } else if (warp == 1) {
             // -------------------------------------------- MMA issuer
-            if (lane == 0 && ok) {
+            if (ok) {
                 ok = walk(p, begin, end, [&](const Unit& un, int, int nk, int lo, int hi) {
-                    if (!mbar_wait(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) return false;
+                    if (!wait_warp(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) return false;
                     tc_fence_after();
                     const uint32_t d = tmem_base + (uint32_t)b.s * 2 * BN;
                     int gi = lo / nk, left = nk - (lo - gi * nk);
                     bool two = p.group[un.first + gi].nb == 2;
                     uint32_t acc = 0;
                     for (int i = lo; i < hi; ++i) {
-                        if (!mbar_wait(&full[r.s], r.ph, p.err, kErrWaitFull)) return false;
+                        if (!wait_warp(&full[r.s], r.ph, p.err, kErrWaitFull)) return false;
                         tc_fence_after();
                         const uint64_t da = sw128_kmajor_desc(smem_u32(ring + (size_t)r.s * STAGE_BYTES));
                         const uint64_t db = da + (TILE_BYTES >> 4);
-                        if (two) {
+                        if (leader) {
+                            const uint32_t dst = two ? d : d + BN, idesc = two ? idesc2 : idesc1;
 #pragma unroll
                             for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(d, da + 2 * k, db + 2 * k, idesc2, k > 0 ? 1u : acc);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(d + BN, da + 2 * k, db + 2 * k, idesc1, k > 0 ? 1u : acc);
+                                tc_mma_bf16(dst, da + 2 * k, db + 2 * k, idesc, k > 0 ? 1u : acc);
+                            tc_commit(&empty[r.s]);
                         }
                         acc = 1u;
-                        tc_commit(&empty[r.s]);
                         r.next(STAGES);
                         if (--left == 0) {
                             left = nk;
@@ -274,12 +274,11 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                             if (i + 1 < hi) two = p.group[un.first + gi].nb == 2;
                         }
                     }
-                    tc_commit(&acc_full[b.s]);
+                    if (leader) tc_commit(&acc_full[b.s]);
                     b.next(2);
                     return true;
                 });
             }
-            __syncwarp();
         } else {
             // -------------------------------------------- drain and epilogue
             const int q4 = warp & 3;                // TMEM lane quadrant this warp may access
@@ -391,7 +390,7 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
             cluster_sync();
         }
     }
-    if (warp == 1 && lane == 0) {
+    if (warp == 1 && leader) {
         // every MMA issued so far has completed before TMEM is released
         tc_commit(done);
         const uint64_t t0 = globaltimer_ns();

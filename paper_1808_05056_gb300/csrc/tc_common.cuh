@@ -89,6 +89,28 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
         : "memory");
 }
 
+// One lane of a converged warp.  The TMA and MMA warps run their loops with all lanes
+// (waits are voted, see wait_warp) and only issue under this lane's flag: the compiler
+// then keeps descriptors and addresses in uniform registers.  With the loop inside an
+// `if (lane == 0)` it moved every operand of every tcgen05.mma there one by one, and the
+// issuing thread took 700 clocks for a stage of 450 clocks of MMAs.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// mbar_wait by a whole warp, with one answer for all lanes
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, int* err, int code)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code)) != 0;
+}
+
 // arrive on an mbarrier once every tcgen05 operation issued so far by this thread completes
 __device__ __forceinline__ void tc_commit(uint64_t* bar)
 {

@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
     uint64_t* done = small_empty + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the shuffle tells the compiler that the warp index is the same in all lanes
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (warp == 1) {
         tmem_alloc(tmem_slot, 512);
         tmem_relinquish();
@@ -175,7 +176,8 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
     bool small_pending = false;  // MMA: one not yet released by the epilogue
     bool ok = true;
     const uint32_t idesc2 = idesc_bf16_f32(BM, 2 * BN), idesc1 = idesc_bf16_f32(BM, BN);
-    if (warp == 0 && lane == 0) {
+    const bool leader = elect_one();  // the lane that issues copies and MMAs
+    if (warp == 0 && leader) {
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
@@ -185,19 +187,21 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
         tile_coords(tile, p.tiles_m, p.tiles_n, tm, tn);
         if (warp == 0) {
             // -------------------------------------------- TMA producer
-            if (lane == 0 && ok) {
+            if (ok) {
                 for (int c = 0; c < nchunks && ok; ++c) {
                     const int end = min(kb1, kb0 + (c + 1) * CHUNK_KBLOCKS);
                     for (int kb = kb0 + c * CHUNK_KBLOCKS; kb < end; ++kb) {
-                        if (!mbar_wait(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) { ok = false; break; }
-                        unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
-                        mbar_arrive_expect_tx(&full[r.s], STAGE_BYTES);
-                        for (int a = 0; a < 3; ++a)
-                            tma_load_3d(st + a * A_TILE, &tmA, &full[r.s], kb * BK, tm * BM, a);
-                        // B planes (h, m, l) beside X0, (m, h, l) beside X1
-                        tma_load_3d(st + 3 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, b.s);
-                        tma_load_3d(st + 4 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 1 - b.s);
-                        tma_load_3d(st + 5 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 2);
+                        if (!wait_warp(&empty[r.s], r.ph ^ 1u, p.err, kErrWaitEmpty)) { ok = false; break; }
+                        if (leader) {
+                            unsigned char* st = ring + (size_t)r.s * STAGE_BYTES;
+                            mbar_arrive_expect_tx(&full[r.s], STAGE_BYTES);
+                            for (int a = 0; a < 3; ++a)
+                                tma_load_3d(st + a * A_TILE, &tmA, &full[r.s], kb * BK, tm * BM, a);
+                            // B planes (h, m, l) beside X0, (m, h, l) beside X1
+                            tma_load_3d(st + 3 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, b.s);
+                            tma_load_3d(st + 4 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 1 - b.s);
+                            tma_load_3d(st + 5 * A_TILE, &tmB, &full[r.s], kb * BK, tn * BN, 2);
+                        }
                         r.next(STAGES);
                         ++issued;
                     }
@@ -216,17 +220,16 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     }
                 }
             }
-            __syncwarp();
         } else if (warp == 1) {
             // -------------------------------------------- MMA issuer
-            if (lane == 0 && ok) {
+            if (ok) {
                 uint32_t small_acc = 0;  // accumulate flag of the small-product accumulators
                 for (int c = 0; c < nchunks && ok; ++c) {
                     const int end = min(kb1, kb0 + (c + 1) * CHUNK_KBLOCKS);
-                    if (!mbar_wait(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) { ok = false; break; }
+                    if (!wait_warp(&acc_empty[b.s], b.ph ^ 1u, p.err, kErrWaitAcc)) { ok = false; break; }
                     if (small_pending) {
                         // the epilogue has read the small accumulators before they restart
-                        if (!mbar_wait(small_empty, (small_drains - 1) & 1u, p.err, kErrWaitAcc)) { ok = false; break; }
+                        if (!wait_warp(small_empty, (small_drains - 1) & 1u, p.err, kErrWaitAcc)) { ok = false; break; }
                         small_pending = false;
                     }
                     tc_fence_after();
@@ -236,51 +239,52 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     const uint32_t bh = (uint32_t)(3 + b.s) * (A_TILE >> 4);  // plane h of B
                     bool fresh = true;
                     for (int kb = kb0 + c * CHUNK_KBLOCKS; kb < end; ++kb) {
-                        if (!mbar_wait(&full[r.s], r.ph, p.err, kErrWaitFull)) { ok = false; break; }
+                        if (!wait_warp(&full[r.s], r.ph, p.err, kErrWaitFull)) { ok = false; break; }
                         tc_fence_after();
                         const uint64_t A = sw128_kmajor_desc(smem_u32(ring + (size_t)r.s * STAGE_BYTES));
                         constexpr uint32_t T = A_TILE >> 4;
-                        // both small accumulators start with m x (h, m)
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k)
-                            tc_mma_bf16(dy, A + T + 2 * k, A + 3 * T + 2 * k, idesc2, k > 0 ? 1u : small_acc);
-                        small_acc = 1u;
-                        if (fresh) {
-                            // the chunk's first h x h restarts the leading accumulator, which an
-                            // N = 256 instruction cannot do without restarting its neighbour
+                        if (leader) {
+                            // both small accumulators start with m x (h, m)
 #pragma unroll
                             for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(dlead, A + 2 * k, A + bh + 2 * k, idesc1, k > 0 ? 1u : 0u);
+                                tc_mma_bf16(dy, A + T + 2 * k, A + 3 * T + 2 * k, idesc2, k > 0 ? 1u : small_acc);
+                            if (fresh) {
+                                // the chunk's first h x h restarts the leading accumulator, which an
+                                // N = 256 instruction cannot do without restarting its neighbour
 #pragma unroll
-                            for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(dsmall, A + 2 * k, A + (7 * T - bh) + 2 * k, idesc1, 1u);
-                            fresh = false;
-                        } else {
+                                for (int k = 0; k < KSTEPS; ++k)
+                                    tc_mma_bf16(dlead, A + 2 * k, A + bh + 2 * k, idesc1, k > 0 ? 1u : 0u);
 #pragma unroll
-                            for (int k = 0; k < KSTEPS; ++k)
-                                tc_mma_bf16(dh, A + 2 * k, A + 3 * T + 2 * k, idesc2, 1u);
+                                for (int k = 0; k < KSTEPS; ++k)
+                                    tc_mma_bf16(dsmall, A + 2 * k, A + (7 * T - bh) + 2 * k, idesc1, 1u);
+                            } else {
+#pragma unroll
+                                for (int k = 0; k < KSTEPS; ++k)
+                                    tc_mma_bf16(dh, A + 2 * k, A + 3 * T + 2 * k, idesc2, 1u);
+                            }
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)  // h x l
+                                tc_mma_bf16(dy, A + 2 * k, A + 5 * T + 2 * k, idesc1, 1u);
+#pragma unroll
+                            for (int k = 0; k < KSTEPS; ++k)  // l x h
+                                tc_mma_bf16(dy, A + 2 * T + 2 * k, A + bh + 2 * k, idesc1, 1u);
+                            tc_commit(&empty[r.s]);
                         }
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k)  // h x l
-                            tc_mma_bf16(dy, A + 2 * k, A + 5 * T + 2 * k, idesc1, 1u);
-#pragma unroll
-                        for (int k = 0; k < KSTEPS; ++k)  // l x h
-                            tc_mma_bf16(dy, A + 2 * T + 2 * k, A + bh + 2 * k, idesc1, 1u);
-                        tc_commit(&empty[r.s]);
+                        small_acc = 1u;
+                        fresh = false;
                         r.next(STAGES);
                     }
                     if (!ok) break;
-                    tc_commit(&acc_full[b.s]);
+                    if (leader) tc_commit(&acc_full[b.s]);
                     b.next(2);
                     if (small_drain_after(c, nchunks)) {
-                        tc_commit(small_full);
+                        if (leader) tc_commit(small_full);
                         ++small_drains;
                         small_pending = true;
                         small_acc = 0;
                     }
                 }
             }
-            __syncwarp();
         } else {
             // -------------------------------------------- epilogue warps
             const int q4 = warp & 3;                 // TMEM lane quadrant this warp may access
@@ -431,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
             cluster_sync();
         }
     }
-    if (warp == 1 && lane == 0) {
+    if (warp == 1 && leader) {
         // every MMA issued so far has completed before TMEM is released
         tc_commit(done);
         const uint64_t t0 = globaltimer_ns();
