@@ -55,11 +55,21 @@ CONFIGS = {
 }
 LEVEL3 = ("syrk", "trsm", "potrf", "getrf")
 # per form: (element dtype name, relative Frobenius tolerance, products per logical product, dtype tag)
-FORMS = {"fp64": ("float64", 1e-13, 1, "f64"), "ozaki": ("float64", 1e-12, 36, "f64 (bf16 digit planes)"),
+FORMS = {"fp64": ("float64", 1e-13, 1, "f64"), "ozaki": ("float64", 1e-12, 21, "f64 (bf16 digit planes)"),
          "bf16x3": ("float32", 1e-6, 6, "f32 (bf16x3 pieces)"), "batched": ("float64", 1e-13, 1, "f64"),
          "syrk": ("float64", 1e-13, 1, "f64"), "trsm": ("float64", 1e-12, 1, "f64"),
-         "potrf": ("float64", 1e-12, 1, "f64"), "getrf": ("float64", 1e-12, 1, "f64"), "summa": ("float64", 1e-12, 36, "f64 (bf16 digit planes)"),
+         "potrf": ("float64", 1e-12, 1, "f64"), "getrf": ("float64", 1e-12, 1, "f64"), "summa": ("float64", 1e-12, 21, "f64 (bf16 digit planes)"),
          "pipe": ("float64", 1e-13, 1, "f64")}
+
+
+def tensor_work(form, st):
+    """(bf16 planes per operand, bf16 products per logical product) that a tensor-core form executes.
+    The Ozaki form's stats count accuracy in slices of 6 bits; its kernels hold S slices in 3/4 S
+    planes of 8-bit digits (csrc/ozaki_gemm.cu) and multiply the pairs s + t <= planes + 1."""
+    if form == "bf16x3":
+        return 3, 6
+    planes = (3 * (st.slices or 8) + 3) // 4
+    return planes, planes * (planes + 1) // 2
 
 
 def batch_shapes(seed, count, lo, hi, cap=64 << 30, es=8):
@@ -79,12 +89,7 @@ NOMINAL_FP64_TF, NOMINAL_BF16_TF = 1.25, 2250.0
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the
 # dominant kernel, from one ncu capture of the configuration's plan (the summary
 # under profiles/ named for the kernel); reported only when a run uses that plan.
-TRAFFIC = {"fp64-32768": {"plan": (2048, 8192, 8192), "bytes": 2.624778e9 + 135.795456e6,
-                          "profile": "profiles/fp64_tile_kernel_traffic_32768.md"},
-           "ozaki-65536": {"plan": (1024, 21888, 16384), "bytes": 11.501296128e9 + 199.416576e6,
-                           "profile": "profiles/tc_terms_kernel_traffic_65536.md"},
-           "bf16x3-65536": {"plan": (1024, 7296, 65536), "bytes": 4.110287616e9 + 27.162880e6,
-                            "profile": "profiles/tc_terms_kernel_traffic_65536.md"}}
+TRAFFIC = {}  # none captured with the present kernels
 
 
 def parse():
@@ -462,20 +467,22 @@ def run_ours(args, w, world, rank, local, pg):
         compute_peak = roof["peak"]
     else:
         peak = pk["bf16_tflops_sustained"]
+        planes, nprod = tensor_work(w["form"], s0)
         # the contraction alone: its launches' event time minus the split kernels before them
-        achieved = flops * s0.products * n_steps / (ker_s - split_s) / 1e12
+        achieved = flops * nprod * n_steps / (ker_s - split_s) / 1e12
         roof = {"bound": "tensor",
-                "kernel": "tc_terms_kernel (tcgen05 bf16 x bf16 -> f32 TMEM, TMA)",
+                "kernel": "%s (tcgen05 bf16 x bf16 -> f32 TMEM, TMA)" % (
+                    "ozaki_tile_kernel" if w["form"] == "ozaki" else "bf16x3_tile_kernel"),
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
                 "split_kernels_s_per_step": split_s / n_steps,
-                "with_split_kernels": flops * s0.products * n_steps / ker_s / 1e12,
-                "traffic_alg_bytes": (s0.slices if w["form"] == "ozaki" else 3) * 2.0 * (s0.mb + s0.nb) * s0.kb +
+                "with_split_kernels": flops * nprod * n_steps / ker_s / 1e12,
+                "traffic_alg_bytes": planes * 2.0 * (s0.mb + s0.nb) * s0.kb +
                                      (2.0 if w["beta"] != 0 else 1.0) * s0.mb * s0.nb * (4 if w["form"] == "bf16x3" else 8),
                 "traffic_source": tr["profile"] if traffic else None,
-                "flop_count": "2*M*N*K x %d bf16 products per logical product" % s0.products,
+                "flop_count": "2*M*N*K x %d bf16 products per logical product" % nprod,
                 "peak_source": "%s bf16 sustained (cuBLAS) %.1f TF" % (pk_src, peak),
                 "logical_tflops": flops * n_steps / (ker_s - split_s) / 1e12, "launches_per_step": s0.steps}
-        compute_peak = peak / s0.products
+        compute_peak = peak / nprod
     t_roof = max(flops / (compute_peak * 1e12), s0.h2d_bytes / (link_h2d * 1e9), s0.d2h_bytes / (link_d2h * 1e9))
     host_gib = (M * K + K * N + M * N) * (4 if w["form"] == "bf16x3" else 8) / 2 ** 30
     line = {
@@ -910,12 +917,12 @@ def run_level3_bench(args, w, world, rank, local, pg):
     pk, pk_src = peaks()
     achieved = flops * args.steps / wall_s / 1e12
     roof = {"bound": "tensor", "kernel": "pipelined out-of-core GEMM updates (%s tile kernel)" % (
-                "tc_terms Ozaki" if args.form == "ozaki" else "fp64_tile"),
+                "ozaki_tile" if args.form == "ozaki" else "fp64_tile"),
             "achieved": achieved, "unit": "TFLOP/s", "traffic": None}
     if args.form != "ozaki":
         roof.update(fp64_roof_fields(pk, pk_src, probe, achieved, (clocks or {}).get("sm_mhz")))
     else:
-        nprod = s0.products or 45
+        nprod = tensor_work("ozaki", s0)[1]
         roof.update({"peak": pk["bf16_tflops_sustained"] / nprod, "frac": achieved / (pk["bf16_tflops_sustained"] / nprod),
                      "peak_source": "%s bf16 sustained %.1f TF / %d Ozaki digit products" % (
                          pk_src, pk["bf16_tflops_sustained"], nprod)})
@@ -1068,7 +1075,7 @@ def run_summa_bench(args, w, world, rank, local, pg):
         "roofline": {"bound": "tensor", "kernel": "tc_terms_kernel (Ozaki, tcgen05)",
                      "achieved": flops * 36 / (st.kernel_seconds - st.split_seconds) / 1e12, "peak": peak,
                      "unit": "TFLOP/s",
-                     "frac": flops * 36 / (st.kernel_seconds - st.split_seconds) / 1e12 / peak, "traffic": None,
+                     "frac": flops * tensor_work("ozaki", st)[1] / (st.kernel_seconds - st.split_seconds) / 1e12 / peak, "traffic": None,
                      "peak_source": "%s bf16 sustained (cuBLAS) %.1f TF" % (pk_src, peak)},
         "session": {"resident_blocks": info["resident_blocks"], "blocks": info["blocks"], "mb": info["mb"],
                     "nb": info["nb"], "h2d_bytes": st.h2d_bytes, "d2h_bytes": st.d2h_bytes},

@@ -71,7 +71,9 @@ extern "C" {
  * mb, nb, kb: C block rows, C block columns and K-chunk length.
  * depth: A-slice buffers (2 or 3); c_buffers: C-block buffers; b_buffers:
  * B-chunk buffers (a whole column of B chunks keeps B resident per column).
- * slices: Ozaki slice count (0 = chosen from the input exponent spread).
+ * slices: accuracy of the Ozaki form's operands in slices of 6 bits of each row's
+ * (column's) largest entry (0: 8 slices in the GEMM calls, 9 in the updates of the
+ * factorizations; 2..10).
  * workspace/workspace_bytes: optional caller-owned device memory for the
  * buffers (see the conventions above).
  */
@@ -101,8 +103,10 @@ typedef struct {
     int64_t blocks;          /* C blocks (h * w)                                     */
     int64_t steps;           /* block x K-chunk steps (tile launches)                */
     int64_t device_bytes;    /* device buffer bytes the plan uses                    */
-    int32_t slices;          /* Ozaki slices / BF16x3 pieces used                    */
-    int32_t products;        /* slice products per tile                              */
+    int32_t slices;          /* Ozaki slices of 6 bits / BF16x3 pieces               */
+    int32_t products;        /* products of such slices, S (S + 1) / 2, / BF16x3's 6
+                                (the Ozaki kernels hold S slices in 3/4 S planes of
+                                8-bit digits and multiply fewer)                     */
     int64_t kernel_launches; /* kernels the call launched (tile + split kernels)    */
     double split_seconds;    /* share of kernel_seconds spent in the split forms'
                                 splitting kernels (0 for FP64 and in graph mode)    */
