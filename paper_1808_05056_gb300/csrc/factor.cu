@@ -25,6 +25,7 @@
 #include <memory>
 #include <string>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "device_sync.cuh"
@@ -133,43 +134,108 @@ __global__ void __launch_bounds__(kTrsmThreads) trsm_small_kernel(const double* 
 // with U^T U = T).  Only that triangle is read and written.  A pivot that is
 // not positive stops the block and records gofs + its column + 1 in *info
 // (first failure wins).
+//
+// One CTA, so the chain of 64 pivots is what it waits for, and that chain is FP64
+// instructions of one warp at 64 clocks each -- 150 when other warps' updates share the
+// pipe, so root and scaling of a column run alone, between two barriers.  The matrix
+// stays in registers (thread (ti, tk) of a 16 x 16 grid holds rows ti + 16 a and columns
+// tk + 16 b).  Root and quotients come from one reciprocal root, corrected to the
+// rounded values (the residuals are exact in fused multiply-adds).
+struct PotrfBlock {
+    double a[4][4];
+    int ti, tk;
+
+    // subtract column j (in col) from this thread's part of the columns of sub-block b
+    template <int b>
+    __device__ __forceinline__ void update(const double* col, int j)
+    {
+        const int k = tk + 16 * b;
+        const double f = k > j ? col[k] : 0.0;
+        if (k <= j) return;
+#pragma unroll
+        for (int r = b; r < 4; ++r) a[r][b] = fma(-col[ti + 16 * r], f, a[r][b]);
+    }
+
+    // root and scaling of column j = 16 b + jj by its 16 owners (a half-warp, lanes `mask`);
+    // j + 1 when the pivot is not positive, else 0
+    template <int b>
+    __device__ __forceinline__ int factor(double* col, int jj, unsigned mask)
+    {
+        const int j = 16 * b + jj;
+        const double d = __shfl_sync(mask, a[b][b], jj, 16);
+        if (!(d > 0.0)) return j + 1;
+        const unsigned e = ((unsigned)__double2hiint(d) >> 20) & 0x7FFu;
+        double root, inv;
+        if (e - 64u < 0x780u) {
+            inv = rsqrt(d);
+            const double g = d * inv;
+            root = fma(fma(-g, g, d), 0.5 * inv, g);
+        } else {
+            root = sqrt(d);
+            inv = __longlong_as_double(0x7FF8000000000000ll);
+        }
+#pragma unroll
+        for (int r = b; r < 4; ++r) {
+            const int i = ti + 16 * r;
+            if (i > j) a[r][b] = quotient(a[r][b], root, inv);
+            else if (i == j) a[r][b] = root;
+            col[i] = a[r][b];
+        }
+        return 0;
+    }
+};
+
 __global__ void __launch_bounds__(256) potrf_small_kernel(double* T, int64_t ldt, int n, int upper, int64_t gofs,
                                                           unsigned long long* info)
 {
-    __shared__ double S[kSmall][kSmall + 1];
-    __shared__ int fail;
+    __shared__ double col[kSmall];
     const int tid = threadIdx.x;
-    for (int idx = tid; idx < n * n; idx += blockDim.x) {
-        const int r = idx / n, c = idx % n;
-        if (c <= r) S[r][c] = upper ? T[(int64_t)c * ldt + r] : T[(int64_t)r * ldt + c];
-    }
-    if (tid == 0) fail = 0;
-    __syncthreads();
-    for (int j = 0; j < n; ++j) {
-        if (tid == 0) {
-            const double d = S[j][j];
-            if (d > 0.0) S[j][j] = sqrt(d);
-            else fail = j + 1;
+    PotrfBlock p;
+    p.ti = tid & 15;
+    p.tk = tid >> 4;
+    const unsigned mask = (tid & 16) ? 0xffff0000u : 0x0000ffffu;
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int i = p.ti + 16 * r, k = p.tk + 16 * c;
+            p.a[r][c] = i == k ? 1.0 : 0.0;  // rows beyond n: the identity
+            if (i < n && k <= i) p.a[r][c] = upper ? T[(int64_t)k * ldt + i] : T[(int64_t)i * ldt + k];
         }
-        __syncthreads();
-        if (fail) break;
-        for (int i = j + 1 + tid; i < n; i += blockDim.x) S[i][j] = S[i][j] / S[j][j];
-        __syncthreads();
-        const int m = n - j - 1;
-        for (int idx = tid; idx < m * m; idx += blockDim.x) {
-            const int i = j + 1 + idx / m, k = j + 1 + idx % m;
-            if (k <= i) S[i][k] -= S[i][j] * S[k][j];
+    int fail = 0;  // first pivot that is not positive (column + 1), on the threads that own it
+    if (p.tk == 0) fail = p.factor<0>(col, 0, mask);
+    bool go = !__syncthreads_or(fail);
+    auto block = [&](auto bc) {
+        constexpr int b = decltype(bc)::value, nx = b < 3 ? b + 1 : 3;
+#pragma unroll 1
+        for (int jj = 0; jj < 16 && go; ++jj) {
+            const int j = 16 * b + jj;
+            if (j + 1 >= n) { go = false; break; }
+            p.update<b>(col, j);
+            if (b + 1 < 4) p.update<(b + 1 < 4 ? b + 1 : 3)>(col, j);
+            if (b + 2 < 4) p.update<(b + 2 < 4 ? b + 2 : 3)>(col, j);
+            if (b + 3 < 4) p.update<(b + 3 < 4 ? b + 3 : 3)>(col, j);
+            __syncthreads();
+            if (jj < 15 && p.tk == jj + 1) fail = p.factor<b>(col, jj + 1, mask);
+            if (jj == 15 && b < 3 && p.tk == 0) fail = p.factor<nx>(col, 0, mask);
+            go = !__syncthreads_or(fail);
         }
-        __syncthreads();
-    }
-    if (tid == 0 && fail) atomicCAS(info, 0ull, (unsigned long long)(gofs + fail));
-    for (int idx = tid; idx < n * n; idx += blockDim.x) {
-        const int r = idx / n, c = idx % n;
-        if (c <= r) {
-            if (upper) T[(int64_t)c * ldt + r] = S[r][c];
-            else T[(int64_t)r * ldt + c] = S[r][c];
+    };
+    block(std::integral_constant<int, 0>{});
+    block(std::integral_constant<int, 1>{});
+    block(std::integral_constant<int, 2>{});
+    block(std::integral_constant<int, 3>{});
+    if (p.ti == 0 && fail) atomicCAS(info, 0ull, (unsigned long long)(gofs + fail));
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int i = p.ti + 16 * r, k = p.tk + 16 * c;
+            if (i < n && k <= i) {
+                if (upper) T[(int64_t)k * ldt + i] = p.a[r][c];
+                else T[(int64_t)i * ldt + k] = p.a[r][c];
+            }
         }
-    }
 }
 
 // ---- LU with partial pivoting ------------------------------------------------
