@@ -18,11 +18,13 @@
 
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <type_traits>
@@ -399,13 +401,14 @@ __global__ void __launch_bounds__(kLuThreads) narrow_lu_kernel(double* P, int64_
         __syncthreads();
         if (zero) continue;
         // own rows below j, one warp per row: multiplier a[j] / pivot, then the rank-1 update
+        const double inv = reciprocal_of(pv);
         for (int64_t i = max(r0, (int64_t)j + 1) + warp; i < r1; i += kLuWarps) {
             const int k0 = lane, k1 = lane + 32;
             double a0 = 0.0, a1 = 0.0;
             if (k0 < nw) a0 = lu_at<kInSmem>(S, P, ldp, r0, i, k0);
             if (k1 < nw) a1 = lu_at<kInSmem>(S, P, ldp, r0, i, k1);
             const double aj = __shfl_sync(0xffffffffu, j < 32 ? a0 : a1, j & 31);
-            const double l = aj / pv;
+            const double l = quotient(aj, pv, inv);
             if (k0 > j && k0 < nw) a0 = fma(-l, prow[k0], a0);
             if (k1 > j && k1 < nw) a1 = fma(-l, prow[k1], a1);
             if (k0 == j) a0 = l;
@@ -422,6 +425,151 @@ __global__ void __launch_bounds__(kLuThreads) narrow_lu_kernel(double* P, int64_
             const int k = (int)(e % nw);
             P[(r0 + r) * ldp + k] = S[r * kLuLd + k];
         }
+    }
+}
+
+// Unblocked LU with partial pivoting of an m x nw panel (nw <= 32), in place, by one
+// cluster of CTAs: CTA g keeps rows [g * rows_per_cta, (g + 1) * rows_per_cta) in its
+// shared memory from the first column to the last, one row per thread and 256 rows.
+//
+// What it waits for is the chain of pivots.  Per column each CTA finds its candidate
+// (largest |a|, smallest row on ties) and writes it,
+// its reciprocal and its row into every CTA's shared memory, as the owner of row j does
+// with row j; after one cluster barrier (about 400 clocks, against microseconds for a
+// barrier through global memory) every warp picks the same winner from its own copy.
+// Nothing else is exchanged, and the interchange, the multipliers and the update touch
+// only a thread's own rows.  The published copies alternate between two buffers by
+// column parity: a slot is rewritten two columns later, after a barrier that every CTA
+// reaches only when it has finished reading it.  Quotients and sums are those of
+// narrow_lu_kernel, which takes the panels too tall for one cluster's shared memory.
+constexpr int kLuClusterCols = 32;
+constexpr int kLuClusterMax = 16;             // CTAs of the cluster (above 8: not portable, sm_103 allows it)
+constexpr int kLuClusterLd = kLuClusterCols + 1;
+constexpr size_t kLuClusterSmem = 190 * 1024;
+
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster(void* p, int rank, long long v)
+{
+    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(void* p, int rank, double v)
+{
+    st_cluster(p, rank, (long long)__double_as_longlong(v));
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// A pivot candidate: the bits of |a| plus one, which order like it (0: nothing
+// comparable), and its row.  Three warp reductions in hardware find the first maximum.
+struct PivotCand {
+    unsigned long long key;
+    int row;
+    __device__ __forceinline__ void take(unsigned long long k, int r)
+    {
+        if (k > key || (k == key && r < row)) { key = k; row = r; }
+    }
+    __device__ __forceinline__ void reduce()
+    {
+        const unsigned hi = (unsigned)(key >> 32), top = __reduce_max_sync(0xffffffffu, hi);
+        const unsigned lo = hi == top ? (unsigned)key : 0u, low = __reduce_max_sync(0xffffffffu, lo);
+        const bool best = hi == top && (unsigned)key == low;
+        row = __reduce_min_sync(0xffffffffu, best ? row : INT_MAX);
+        key = ((unsigned long long)top << 32) | low;
+    }
+};
+
+__global__ void __launch_bounds__(kLuThreads) lu_cluster_kernel(double* P, int64_t ldp, int m, int nw,
+                                                                int rows_per_cta, int64_t* piv,
+                                                                unsigned long long* info, int64_t gofs)
+{
+    extern __shared__ double S[];  // the CTA's rows, stride kLuClusterLd
+    __shared__ double crow[2][kLuClusterMax][kLuClusterCols], jrow[2][kLuClusterCols], cinv[2][kLuClusterMax];
+    __shared__ unsigned long long ckey[2][kLuClusterMax], crow_at[2][kLuClusterMax];
+    __shared__ unsigned long long wkey[2][kLuWarps];
+    __shared__ int wrow[2][kLuWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int G = (int)gridDim.x, rank = (int)blockIdx.x;  // one cluster
+    const int r0 = rank * rows_per_cta, nloc = max(0, min(m - r0, rows_per_cta));
+    for (int e = tid; e < nloc * kLuClusterCols; e += kLuThreads) {
+        const int r = e / kLuClusterCols, k = e % kLuClusterCols;
+        if (k < nw) S[r * kLuClusterLd + k] = P[(int64_t)(r0 + r) * ldp + k];
+    }
+    __syncthreads();
+    cluster_barrier();  // every CTA of the cluster runs before the first write to another's memory
+#pragma unroll 1
+    for (int j = 0; j < nw; ++j) {
+        const int b = j & 1;
+        // local candidate over own rows i >= j, smallest row on ties
+        PivotCand c{0, INT_MAX};
+        for (int r = tid; r < nloc; r += kLuThreads) {
+            const unsigned long long k =
+                (unsigned long long)__double_as_longlong(S[r * kLuClusterLd + j]) & 0x7FFFFFFFFFFFFFFFull;
+            if (r0 + r >= j && k <= 0x7FF0000000000000ull) c.take(k + 1, r0 + r);  // a NaN is never chosen
+        }
+        c.reduce();
+        if (lane == 0) { wkey[b][warp] = c.key; wrow[b][warp] = c.row; }
+        __syncthreads();
+        c = PivotCand{lane < kLuWarps ? wkey[b][lane] : 0, lane < kLuWarps ? wrow[b][lane] : INT_MAX};
+        c.reduce();
+        // publish it and, from its owner, row j: each warp writes to every eighth CTA
+        const double cand = c.key && lane < nw ? S[(c.row - r0) * kLuClusterLd + lane] : 0.0;
+        const double own_j = j >= r0 && j < r0 + nloc && lane < nw ? S[(j - r0) * kLuClusterLd + lane] : 0.0;
+        for (int q = warp; q < G; q += kLuWarps) {
+            if (lane < nw) {
+                st_cluster(&crow[b][rank][lane], q, cand);
+                if (j >= r0 && j < r0 + nloc) st_cluster(&jrow[b][lane], q, own_j);
+            }
+            if (lane == 0) {
+                st_cluster(&ckey[b][rank], q, (long long)c.key);
+                st_cluster(&crow_at[b][rank], q, (long long)c.row);
+            }
+        }
+        if (warp == 0) {
+            const double inv = reciprocal_of(__shfl_sync(0xffffffffu, cand, j));
+            if (lane < G) st_cluster(&cinv[b][rank], lane, inv);
+        }
+        cluster_barrier();
+        // every warp reduces the candidates the same way: the global first maximum
+        c = PivotCand{lane < G ? ckey[b][lane] : 0, lane < G ? (int)crow_at[b][lane] : INT_MAX};
+        c.reduce();
+        const bool found = c.key != 0;
+        const int p = found ? c.row : j, owner = found ? p / rows_per_cta : 0;
+        const double* src = found ? crow[b][owner] : jrow[b];
+        const double pv = src[j], inv = found ? cinv[b][owner] : pv;  // nothing comparable: pv is NaN
+        const bool zero = c.key == 1;
+        if (rank == 0 && tid == 0) {
+            piv[j] = p;
+            if (zero) atomicCAS(info, 0ull, (unsigned long long)(gofs + j + 1));
+        }
+        // own rows: row j becomes the pivot row, row p the old row j; those below j are
+        // scaled and updated
+        for (int r = tid; r < nloc; r += kLuThreads) {
+            const int i = r0 + r;
+            double* row = S + r * kLuClusterLd;
+            if (i < j) continue;
+            if (i == j || i == p) {
+                const double* from = i == j ? src : jrow[b];
+#pragma unroll 8
+                for (int k = 0; k < nw; ++k) row[k] = from[k];
+            }
+            if (i == j || zero) continue;
+            const double l = quotient(row[j], pv, inv);
+            row[j] = l;
+#pragma unroll 4
+            for (int k = j + 1; k < nw; ++k) row[k] = fma(-l, src[k], row[k]);
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < nloc * kLuClusterCols; e += kLuThreads) {
+        const int r = e / kLuClusterCols, k = e % kLuClusterCols;
+        if (k < nw) P[(int64_t)(r0 + r) * ldp + k] = S[r * kLuClusterLd + k];
     }
 }
 
@@ -639,6 +787,50 @@ int launch_laswp(double* P, int64_t ldp, int64_t ncols, const int64_t* piv, int6
     return check_launch("laswp_kernel", why);
 }
 
+void lu_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, size_t smem, cudaStream_t st)
+{
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster);
+    cfg.blockDim = dim3(kLuThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+// CTAs of the cluster that takes an m-row sub-panel (0: too tall): at least 32 rows each,
+// so that a warp's instructions carry 32 rows, and as many CTAs as that leaves -- the
+// update's FP64 work is spread over their SMs.
+int lu_cluster_size(int64_t m)
+{
+    static int largest = 0;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        if (cudaFuncSetAttribute(lu_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kLuClusterSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(lu_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        for (int c = kLuClusterMax; c >= 1 && !largest; c /= 2) {
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute at;
+            lu_cluster_config(cfg, at, c, kLuClusterSmem, nullptr);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, lu_cluster_kernel, &cfg) != cudaSuccess) cudaGetLastError();
+            else if (n > 0) largest = c;
+        }
+    });
+    if (!largest || m > (int64_t)largest * (int64_t)(kLuClusterSmem / (kLuClusterLd * sizeof(double)))) return 0;
+    int c = 1;
+    while (c < largest && (int64_t)c * 32 < m) c *= 2;
+    return c;
+}
+
 // In device memory: LU with partial pivoting of the m x n panel P (m >= n),
 // recursive halving at multiples of 64 (Toledo's recursive LU): factor the
 // left half, interchange the right half's rows, U12 = L11^{-1} A12, A22 -=
@@ -647,7 +839,23 @@ int launch_laswp(double* P, int64_t ldp, int64_t ncols, const int64_t* piv, int6
 // panel's first global column (for info).
 int panel_lu(double* P, int64_t ldp, int64_t m, int64_t n, int64_t* piv, int64_t gofs, Dev& d, std::string& why)
 {
-    if (n <= kSmall) {
+    const int cluster = d.lu_rows_global ? 0 : lu_cluster_size(m);
+    if (cluster && n <= kLuClusterCols) {
+        const int rows = (int)((m + cluster - 1) / cluster);
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        lu_cluster_config(cfg, at, cluster, (size_t)rows * kLuClusterLd * sizeof(double), d.st);
+        const cudaError_t e =
+            cudaLaunchKernelEx(&cfg, lu_cluster_kernel, P, ldp, (int)m, (int)n, rows, piv, d.info, gofs);
+        ++d.launches;
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            why = std::string("lu_cluster_kernel: ") + cudaGetErrorString(e);
+            return OOC_ERR_CUDA;
+        }
+        return OOC_OK;
+    }
+    if (!cluster && n <= kSmall) {
         // rows in shared memory when a co-resident grid's slices fit, else in global memory
         int64_t grid = std::max<int64_t>(1, std::min<int64_t>(d.lu_grid, (m + 31) / 32));
         const int sms = device_sm_count();
@@ -691,7 +899,8 @@ int panel_lu(double* P, int64_t ldp, int64_t m, int64_t n, int64_t* piv, int64_t
         }
         return OOC_OK;
     }
-    const int64_t n1 = split_point(n), n2 = n - n1;
+    // down to one 64-column sub-panel halve at multiples of 64, a 64-column one at 32
+    const int64_t n1 = n > kSmall ? split_point(n) : kLuClusterCols, n2 = n - n1;
     int rc;
     if ((rc = panel_lu(P, ldp, m, n1, piv, gofs, d, why))) return rc;
     if ((rc = launch_laswp(P + n1, ldp, n2, piv, 0, n1, d, why))) return rc;
