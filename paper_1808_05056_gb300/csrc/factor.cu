@@ -573,19 +573,67 @@ __global__ void __launch_bounds__(kLuThreads) lu_cluster_kernel(double* P, int64
     }
 }
 
-// Row interchanges k <-> piv[k] for k in [k0, k1), in order, over columns [0, ncols) of P
-// (one thread per column).
-__global__ void laswp_kernel(double* P, int64_t ldp, int64_t ncols, const int64_t* piv, int64_t k0, int64_t k1)
+// Row interchanges k <-> piv[k] for k in [k0, k1), in order, over columns [0, ncols) of
+// P, as one gather: which original row ends up where is worked out first, so the rows
+// move with independent loads instead of a chain of dependent swaps (a swap waits for
+// two global loads; 64 of them took 40 us).
+//
+// Before swap k row k holds c(k): the value that the latest earlier swap with pivot k
+// put there (its own c), else row k itself.  Swap k puts into row k what row piv[k]
+// holds -- c of the latest earlier swap with that pivot, else row piv[k] itself -- and
+// that is final; a row below k1 ends with c of the last swap with that pivot.  Each CTA
+// finds the earlier swaps by comparison, follows the links to the original rows, then
+// moves a strip of columns through shared memory.  n = k1 - k0 <= kLaswpMax.
+constexpr int kLaswpMax = 512, kLaswpCols = 8, kLaswpThreads = 256;
+__global__ void __launch_bounds__(kLaswpThreads) laswp_kernel(double* P, int64_t ldp, int64_t ncols,
+                                                              const int64_t* __restrict__ piv, int64_t k0, int n)
 {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ncols; c += (int64_t)gridDim.x * blockDim.x)
-        for (int64_t k = k0; k < k1; ++k) {
-            const int64_t p = piv[k];
-            if (p != k) {
-                const double t = P[k * ldp + c];
-                P[k * ldp + c] = P[p * ldp + c];
-                P[p * ldp + c] = t;
-            }
+    extern __shared__ double vals[];   // [2 n][kLaswpCols]: what rows k0 + k and piv[k] end with
+    __shared__ int64_t pv[kLaswpMax];
+    __shared__ int up[kLaswpMax];      // the earlier swap that made c(k); itself: the original row
+    __shared__ int64_t top[kLaswpMax]; // original row that row k0 + k ends with
+    __shared__ int64_t out[kLaswpMax]; // original row that row piv[k] ends with; -1: not decided by swap k
+    for (int k = threadIdx.x; k < n; k += kLaswpThreads) pv[k] = piv[k0 + k];
+    __syncthreads();
+    auto latest = [&](int64_t row, int before) {
+        int q = before - 1;
+        while (q >= 0 && pv[q] != row) --q;
+        return q;
+    };
+    for (int k = threadIdx.x; k < n; k += kLaswpThreads) {
+        const int q = latest(k0 + k, k);
+        up[k] = q >= 0 ? q : k;
+    }
+    __syncthreads();
+    auto origin = [&](int k) {  // original row of c(k)
+        while (up[k] != k) k = up[k];
+        return k0 + k;
+    };
+    for (int k = threadIdx.x; k < n; k += kLaswpThreads) {
+        const int64_t p = pv[k];
+        const int q = p == k0 + k ? k : latest(p, k);
+        top[k] = q >= 0 ? origin(q) : p;
+        bool last = p >= k0 + n;
+        for (int z = k + 1; last && z < n; ++z) last = pv[z] != p;
+        out[k] = last ? origin(k) : -1;
+    }
+    __syncthreads();
+    for (int64_t c0 = (int64_t)blockIdx.x * kLaswpCols; c0 < ncols; c0 += (int64_t)gridDim.x * kLaswpCols) {
+        const int w = (int)min((int64_t)kLaswpCols, ncols - c0);
+        for (int e = threadIdx.x; e < 2 * n * kLaswpCols; e += kLaswpThreads) {
+            const int k = e / kLaswpCols, c = e % kLaswpCols;
+            const int64_t from = k < n ? top[k] : out[k - n];
+            if (c < w && from >= 0) vals[e] = P[from * ldp + c0 + c];
         }
+        __syncthreads();
+        for (int e = threadIdx.x; e < 2 * n * kLaswpCols; e += kLaswpThreads) {
+            const int k = e / kLaswpCols, c = e % kLaswpCols;
+            if (c >= w) continue;
+            if (k < n) P[(k0 + k) * ldp + c0 + c] = vals[e];
+            else if (out[k - n] >= 0) P[pv[k - n] * ldp + c0 + c] = vals[e];
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void add_offset_kernel(int64_t* v, int64_t n, int64_t off)
@@ -781,10 +829,22 @@ int launch_laswp(double* P, int64_t ldp, int64_t ncols, const int64_t* piv, int6
                  std::string& why)
 {
     if (ncols <= 0 || k1 <= k0) return OOC_OK;
-    const int64_t grid = std::min<int64_t>((ncols + 255) / 256, 4096);
-    laswp_kernel<<<(unsigned)grid, 256, 0, d.st>>>(P, ldp, ncols, piv, k0, k1);
-    ++d.launches;
-    return check_launch("laswp_kernel", why);
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        laswp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kLaswpMax * kLaswpCols * (int)sizeof(double));
+    if (attr != cudaSuccess) {
+        why = std::string("laswp_kernel shared memory: ") + cudaGetErrorString(attr);
+        return OOC_ERR_CUDA;
+    }
+    const int64_t grid = std::min<int64_t>((ncols + kLaswpCols - 1) / kLaswpCols, 4096);
+    for (int64_t k = k0; k < k1; k += kLaswpMax) {
+        const int n = (int)std::min<int64_t>(kLaswpMax, k1 - k);
+        laswp_kernel<<<(unsigned)grid, kLaswpThreads, 2 * (size_t)n * kLaswpCols * sizeof(double), d.st>>>(
+            P, ldp, ncols, piv, k, n);
+        ++d.launches;
+        const int rc = check_launch("laswp_kernel", why);
+        if (rc) return rc;
+    }
+    return OOC_OK;
 }
 
 void lu_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, size_t smem, cudaStream_t st)
