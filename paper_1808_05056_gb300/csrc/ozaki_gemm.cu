@@ -15,8 +15,8 @@
 // 2^14 2^-(8(S+2)-2), so the error bound of the 6-bit digits holds with room.
 //
 // Sums.  The exact FP32 sums go into one 64-bit fixed-point integer per output (unit
-// 2^-frac, see frac_bits): convert, then one wide multiply-add -- 3 instructions on
-// the integer and conversion pipes.  In FP64 the same drain is bound by the FP64 pipe
+// 2^-frac): to an integer by packed FP32 additions of large constants (the conversion
+// unit is a quarter as wide as these pipes), then one wide multiply-add.  In FP64 the same drain is bound by the FP64 pipe
 // (1.75 additions a clock and SM: 9400 clocks per 128 x 128 sum, which takes the
 // tensor cores 4096 clocks to make).  Integer sums are exact whatever their order, so
 // the result does not depend on how a tile's work is cut (cut_stages).
@@ -86,7 +86,7 @@ struct Group {
 
 // A unit shares one accumulator pair: `ngroups` groups from `first`, drained every
 // `chunk` K blocks.  The two accumulators' weights as a factor applied in FP32 (a
-// power of two; rounds to an integer when it is below one) and a left shift.
+// power of two, sums are rounded to integers after it) and a left shift.
 struct Unit {
     int16_t first, ngroups, chunk, pad;
     float scale[2];
@@ -102,6 +102,7 @@ struct Args {
     int cut[MAX_CLUSTER + 1];  // CTA r of a cluster takes stages [cut[r], cut[r + 1]) of a tile
     int frac;              // the integers' unit is 2^-frac
     double alpha, beta;
+    int alpha_one;         // 1: alpha is one, -1: minus one (no multiplication on the FP64 pipe)
     int read_c;
     double* C;
     int64_t ldc;
@@ -135,9 +136,45 @@ __device__ __forceinline__ bool walk(const Args& p, int begin, int end, Fn fn)
     return true;
 }
 
+// Packed pairs of FP32 values (element 2j in the low half).
+__device__ __forceinline__ uint64_t f2fma(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2add(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2sub(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t pair(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
+__device__ __forceinline__ uint64_t pair(float x) { return pair(__float_as_uint(x), __float_as_uint(x)); }
+
+// v * sc for two FP32 sums v, |v * sc| <= 2^24, rounded to the nearest integer (ties to
+// even).  Adding 1.5 2^25 rounds to a multiple of 4, h, and leaves h / 4 in the low bits;
+// the rest, exact and at most 2 in magnitude, is rounded by adding 1.5 2^23, and 4 being
+// even the tie rule is that of the whole.
+__device__ __forceinline__ void round_pair(uint64_t v, uint64_t sc, int& i0, int& i1)
+{
+    const uint64_t big = pair(50331648.0f), one = pair(12582912.0f);
+    const uint64_t t = f2fma(v, sc, big);
+    const uint64_t u = f2add(f2fma(v, sc, f2sub(big, t)), one);
+    constexpr uint32_t bias = 0x4C400000u * 4u + 0x4B400000u;  // what the two constants leave
+    i0 = (int)(((uint32_t)t << 2) + (uint32_t)u - bias);
+    i1 = (int)(((uint32_t)(t >> 32) << 2) + (uint32_t)(u >> 32) - bias);
+}
+
 // t * 2^e, rounded once (to nearest, ties to even) from the 64-bit integer, with
-// integer operations: a conversion and a scaling on the FP64 pipe would take 9400
-// clocks each per tile.  Results outside the normal range go through ldexp.
+// integer operations: every instruction per output on the FP64 pipe holds it for 9700
+// clocks a tile, a comparison as much as a conversion, a scaling or a multiplication.  Results outside the normal range go through ldexp.
 __device__ __forceinline__ double fixed_to_f64(long long t, int e)
 {
     if (t == 0) return 0.0;
@@ -299,23 +336,24 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     const int q0 = p.group[un.first + lo / nk].nb == 2 ? 0 : 1;
 #pragma unroll 1
                     for (int q = q0; q < 2; ++q) {
-                        const float sc = un.scale[q];
+                        const uint64_t sc = pair(un.scale[q]);
                         const int sh = un.shift[q], mul = 1 << (sh & 31);
 #pragma unroll
-                        for (int cc = 0; cc < 2; ++cc) {
-                            uint32_t v[16];
-                            tmem_ld_32x32b_x16(t0 + q * BN + cc * 16, v);
+                        for (int cc = 0; cc < 4; ++cc) {
+                            uint32_t v[8];
+                            tmem_ld_32x32b_x8(t0 + q * BN + cc * 8, v);
                             tmem_wait_ld();
-                            if (sh < 31) {
 #pragma unroll
-                                for (int j = 0; j < 16; ++j)
-                                    acc[cc * 16 + j] += (long long)__float2int_rn(__uint_as_float(v[j]) * sc) * mul;
-                            } else {
-                                // a shift of 32 or more reaches the high word only
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    const unsigned hi = (unsigned)__float2int_rn(__uint_as_float(v[j]) * sc) * mul;
-                                    acc[cc * 16 + j] += (long long)((unsigned long long)hi << 32);
+                            for (int j = 0; j < 8; j += 2) {
+                                int s0, s1;
+                                round_pair(pair(v[j], v[j + 1]), sc, s0, s1);
+                                long long &a0 = acc[cc * 8 + j], &a1 = acc[cc * 8 + j + 1];
+                                if (sh < 32) {
+                                    a0 += (long long)s0 * mul;
+                                    a1 += (long long)s1 * mul;
+                                } else {  // reaches the high word only
+                                    a0 += (long long)((unsigned long long)((unsigned)s0 * mul) << 32);
+                                    a1 += (long long)((unsigned long long)((unsigned)s1 * mul) << 32);
                                 }
                             }
                         }
@@ -328,30 +366,45 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                 });
             // the tile's result, 4 columns at a time: each lane forms its own row's values,
             // transpose4 hands lane 4g + j column j of rows 4g .. 4g + 3, and each store then
-            // covers 8 rows x 4 consecutive columns of C (whole 32-byte sectors)
-            const int64_t row_me = (int64_t)tm * BM + row_in_tile;
-            const int re = (p.row_exp && row_me < p.M ? p.row_exp[row_me] : 0) + 2 - p.frac;  // no exponents when K == 0
+            // covers 8 rows x 4 consecutive columns of C (whole 32-byte sectors).  The old values
+            // of a pass are fetched before its conversions, so that they arrive behind them.
+            // One load per lane brings the exponents of its row and of column `lane` of the quarter
+            // (none when K == 0).
+            const int64_t row_me = (int64_t)tm * BM + row_in_tile, col_me = (int64_t)tn * BN + quarter * 32 + lane;
+            const int ce_lane = p.col_exp && col_me < p.N ? p.col_exp[col_me] : 0;
+            const int re = (p.row_exp && row_me < p.M ? p.row_exp[row_me] : 0) + 2 - p.frac;
+            const int row0 = tm * BM + q4 * 32 + (lane & ~3), col0 = tn * BN + quarter * 32 + (lane & 3);
+            double* const c_lane = p.C + (int64_t)row0 * p.ldc + col0;
             auto emit = [&](int pass, const long long (&t)[4]) {
-                const int64_t c0 = (int64_t)tn * BN + quarter * 32 + pass * 4;
+                const int col = col0 + pass * 4;
+                double* const c = c_lane + pass * 4;
+                bool keep[4];
+                double old[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t d = (int64_t)col - (row0 + i);
+                    keep[i] = col < p.N && row0 + i < p.M &&
+                              (p.tri == 0 || (p.tri == 1 ? d <= p.tri_off : d >= p.tri_off));
+                    old[i] = keep[i] && p.read_c ? c[i * p.ldc] : 0.0;
+                }
                 double v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int ce = p.col_exp && c0 + j < p.N ? p.col_exp[c0 + j] : 0;
-                    const double x = fixed_to_f64(t[j], re + ce);
-                    v[j] = p.alpha == 1.0 ? x : p.alpha * x;
+                    v[j] = fixed_to_f64(p.alpha_one < 0 ? -t[j] : t[j],
+                                        re + __shfl_sync(0xffffffffu, ce_lane, pass * 4 + j));
+                }
+                if (p.alpha_one == 0) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] *= p.alpha;
                 }
                 transpose4(v, lane);
-                const int64_t col = c0 + (lane & 3), row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
-                if (col >= p.N) return;
+                if (p.read_c) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int64_t row = row0 + i;
-                    const bool keep = p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off);
-                    if (row < p.M && keep) {
-                        double* c = p.C + row * p.ldc + col;
-                        *c = p.read_c ? fma(p.beta, *c, v[i]) : v[i];
-                    }
+                    for (int i = 0; i < 4; ++i) v[i] = fma(p.beta, old[i], v[i]);
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (keep[i]) c[i * p.ldc] = v[i];
             };
             long long* part = reinterpret_cast<long long*>(ring);  // [column][row]
             if (p.cluster == 1) {
@@ -547,12 +600,12 @@ void plan_units(Args& a, int S)
 {
     int ng = 0, nu = 0;
     auto weigh = [&](Unit& u, int q, int m) {
-        // a left shift of the converted sum (below 2^24 in magnitude); 31 would overflow
-        // the multiplier, so the odd power goes into the conversion; below 0: rounded off
+        // a left shift of the converted sum (at most 2^24 in magnitude); below 0: bits rounded
+        // off in the conversion.  2^31 as a signed multiplier is -2^31, so the sum changes sign
         int sh = a.frac - DIGIT * m;
         float sc = 1.0f;
         if (sh < 0) { sc = std::ldexp(1.0f, sh); sh = 0; }
-        else if (sh == 31) { sc = 2.0f; sh = 30; }
+        else if (sh == 31) sc = -1.0f;
         u.scale[q] = sc;
         u.shift[q] = sh;
     };
@@ -695,6 +748,7 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     a.tiles_n = (int)cdiv(P.N, BN);
     a.tiles = a.tiles_m * a.tiles_n;
     a.alpha = P.alpha;
+    a.alpha_one = P.alpha == 1.0 ? 1 : P.alpha == -1.0 ? -1 : 0;
     a.C = P.C; a.ldc = P.ldc;
     a.row_exp = P.row_exp; a.col_exp = P.col_exp;
     a.err = P.err;
