@@ -409,7 +409,7 @@ int split_slot(const Plan& p, Exec& x, int src_slot, int dst_slot, bool is_a, in
     const int64_t ld = is_a ? p.lda_dev : p.ldb_dev;
     const int64_t sr = kmajor ? ld : 1, sk = kmajor ? 1 : ld;
     const char* src = x.base + slot_offset(p, src_slot);
-    x.launches += ozaki && K > 0 ? 2 : 1;
+    x.launches += ozaki ? split_ozaki_launches(K) : 1;
     if (ozaki) {
         auto* rowmax = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(exps) + ((rpad * 4 + 255) / 256) * 256);
         return launch_split_ozaki(reinterpret_cast<const double*>(src), sr, sk, (int)nrows, (int)K, (int)rpad,

@@ -541,8 +541,33 @@ __device__ __forceinline__ long long fixed_point(double x, int e, int S)
     return (bits >> 63) ? -(long long)F : (long long)F;
 }
 
-// S balanced digits of each element (most significant first): 64 rows x 64 K per
-// block, 8 consecutive K per thread and step, one 16-byte store per plane.
+// S balanced digits (most significant first) of 8 consecutive K of a row: one 16-byte
+// store per plane at element offset o.
+__device__ __forceinline__ void store_digits(const double (&x)[8], int e, int S, __nv_bfloat16* planes, size_t plane,
+                                             size_t o)
+{
+    long long F[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) F[j] = fixed_point(x[j], e, S);
+    for (int s = S - 1; s >= 0; --s) {
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+            int d[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // the low 8 bits as a signed digit, the rest carried on; the top digit is what is left
+                d[h] = s > 0 ? (int)(signed char)(F[j + h] & 0xFF) : (int)F[j + h];
+                F[j + h] = (F[j + h] - d[h]) >> DIGIT;
+            }
+            const __nv_bfloat162 b = __floats2bfloat162_rn((float)d[0], (float)d[1]);
+            w[j / 2] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        *reinterpret_cast<uint4*>(planes + (size_t)s * plane + o) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Digit planes and row exponents from the row maxima: 64 rows x 64 K per block.
 __global__ void __launch_bounds__(256) split_kernel(const double* __restrict__ X, int64_t sr, int64_t sk, int rows,
                                                     int K, int rows_pad, int k_pad,
                                                     const unsigned long long* __restrict__ rowmax, int S,
@@ -556,40 +581,74 @@ __global__ void __launch_bounds__(256) split_kernel(const double* __restrict__ X
             t[i][c] = (r0 + c < rows && k0 + i < K) ? __ldg(X + (int64_t)(k0 + i) * sk + r0 + c) : 0.0;
         __syncthreads();
     }
-    const size_t plane = (size_t)rows_pad * k_pad;
     const int g = threadIdx.x & 7;
     for (int i = threadIdx.x >> 3; i < ST; i += 32) {
         const int r = r0 + i, k = k0 + g * 8;
         if (r >= rows_pad || k >= k_pad) continue;
         const int e = r < rows ? exponent_of(rowmax[r]) : 0;
         if (k == 0) rowexp[r] = e;
-        long long F[8];
+        double x[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            double x;
-            if (sk != 1) x = t[g * 8 + j][i];
-            else x = (r < rows && k + j < K) ? __ldg(X + (int64_t)r * sr + k + j) : 0.0;
-            F[j] = fixed_point(x, e, S);
+            if (sk != 1) x[j] = t[g * 8 + j][i];
+            else x[j] = (r < rows && k + j < K) ? __ldg(X + (int64_t)r * sr + k + j) : 0.0;
         }
-        const size_t o = (size_t)r * k_pad + k;
-        for (int s = S - 1; s >= 0; --s) {
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                int d[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // the low 8 bits as a signed digit, the rest carried on; the top digit is what is left
-                    d[h] = s > 0 ? (int)(signed char)(F[j + h] & 0xFF) : (int)F[j + h];
-                    F[j + h] = (F[j + h] - d[h]) >> DIGIT;
-                }
-                const __nv_bfloat162 b = __floats2bfloat162_rn((float)d[0], (float)d[1]);
-                w[j / 2] = *reinterpret_cast<const uint32_t*>(&b);
-            }
-            *reinterpret_cast<uint4*>(planes + (size_t)s * plane + o) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        store_digits(x, e, S, planes, (size_t)rows_pad * k_pad, (size_t)r * k_pad + k);
     }
 }
+
+// The whole split in one launch, for short K: each block finds the maxima of FR rows over all
+// of K and then cuts them, reading them again from L1 / L2.
+constexpr int FR = 16, FK = 128;
+template <bool kKMajor>
+__global__ void __launch_bounds__(256) split_short_kernel(const double* __restrict__ X, int64_t ld, int rows, int K,
+                                                          int rows_pad, int k_pad, int S,
+                                                          __nv_bfloat16* __restrict__ planes, int* __restrict__ rowexp)
+{
+    __shared__ unsigned long long part[FR][17];
+    __shared__ int ex[FR];
+    __shared__ double t[kKMajor ? 1 : FK][FR + 1];  // [k][row], operands with K down the stored rows
+    const int r0 = blockIdx.x * FR, tid = threadIdx.x;
+    // 16 threads per row: along K when it is contiguous, along the rows when they are
+    const int row = kKMajor ? tid >> 4 : tid & 15, q = kKMajor ? tid & 15 : tid >> 4;
+    auto at = [&](int r, int64_t k) { return __ldg(X + (kKMajor ? (int64_t)r * ld + k : k * ld + r)); };
+    unsigned long long m = 0;
+    if (r0 + row < rows) {
+#pragma unroll 8
+        for (int k = q; k < K; k += 16) m = max(m, abs_bits(at(r0 + row, k)));
+    }
+    part[row][q] = m;
+    __syncthreads();
+    if (tid < FR) {
+        m = part[tid][0];
+#pragma unroll
+        for (int i = 1; i < 16; ++i) m = max(m, part[tid][i]);
+        ex[tid] = exponent_of(m);
+        if (r0 + tid < rows_pad) rowexp[r0 + tid] = ex[tid];
+    }
+    __syncthreads();
+    const int i = tid >> 4, g = tid & 15;  // this thread's row and group of 8 K
+    for (int k0 = 0; k0 < k_pad; k0 += FK) {
+        if (!kKMajor) {
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < FK; u += 16)
+                t[u + q][row] = r0 + row < rows && k0 + u + q < K ? at(r0 + row, k0 + u + q) : 0.0;
+            __syncthreads();
+        }
+        const int r = r0 + i, k = k0 + g * 8;
+        if (r >= rows_pad || k >= k_pad) continue;
+        double x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            x[j] = kKMajor ? (r < rows && k + j < K ? at(r, k + j) : 0.0) : t[kKMajor ? 0 : g * 8 + j][i];
+        store_digits(x, ex[i], S, planes, (size_t)rows_pad * k_pad, (size_t)r * k_pad + k);
+    }
+}
+// K up to which the one-launch split is taken: a block walks K serially, 16 rows at a time,
+// so it pays while that walk is shorter than the clear, the maxima and the cut of the general
+// one (both operands: K 64 43 -> 23 us, 512 81 -> 55, 1024 144 -> 119, but 1900 61 -> 103).
+constexpr int kShortSplit = 1024;
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -700,10 +759,21 @@ void choose_cluster(Args& a, int planes, const ClusterCounts& counts)
 
 }  // namespace
 
+int split_ozaki_launches(int64_t K) { return K > kShortSplit ? 2 : 1; }
+
 int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad, int S,
                        void* planes, int* rowexp, unsigned long long* rowmax, void* stream, std::string& why)
 {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    auto* pl = static_cast<__nv_bfloat16*>(planes);
+    if (K <= kShortSplit) {
+        const unsigned grid = (unsigned)cdiv(rows_pad, FR);
+        if (sk == 1) split_short_kernel<true><<<grid, 256, 0, st>>>(X, sr, rows, K, rows_pad, k_pad, S, pl, rowexp);
+        else split_short_kernel<false><<<grid, 256, 0, st>>>(X, sk, rows, K, rows_pad, k_pad, S, pl, rowexp);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) { why = std::string("split_ozaki: ") + cudaGetErrorString(e); return OOC_ERR_CUDA; }
+        return OOC_OK;
+    }
     if (cudaMemsetAsync(rowmax, 0, sizeof(unsigned long long) * (size_t)rows_pad, st) != cudaSuccess) {
         why = "rowmax clear";
         return OOC_ERR_CUDA;
@@ -717,7 +787,7 @@ int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K,
                                                                                                        rowmax);
     }
     split_kernel<<<dim3((unsigned)cdiv(k_pad, ST), (unsigned)cdiv(rows_pad, ST)), 256, 0, st>>>(
-        X, sr, sk, rows, K, rows_pad, k_pad, rowmax, S, static_cast<__nv_bfloat16*>(planes), rowexp);
+        X, sr, sk, rows, K, rows_pad, k_pad, rowmax, S, pl, rowexp);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { why = std::string("split_ozaki: ") + cudaGetErrorString(e); return OOC_ERR_CUDA; }
     return OOC_OK;
