@@ -40,43 +40,78 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// What the estimate knows of a form's kernels on this device (all measured).
 struct FormModel {
-    int64_t tile_m, tile_n;  // CTA tile of the contraction kernel
+    int64_t tile;            // CTA tile of the contraction kernel (square)
+    int64_t grain;           // block sizes tried are multiples of this
     double rate;             // sustained tile throughput, logical FLOP/s of the whole device
     int ctas_per_sm;
+    int cluster;             // most CTAs that share a tile when a launch has few
+    double exchange;         // seconds that sharing adds to a tile
+    double launch;           // seconds of a launch beyond its tiles, and the least a tile takes
+    double step;             // seconds a step adds to its kernel
+    double split_bytes;      // bytes per element that the split of an operand moves (0: none)
     int products;            // slice products per logical product
     int slices;
-    double overlap_cost;     // share of the hidden copy time a step still loses (measured)
+    double overlap_cost;     // share of the hidden copy time a step still loses
+    bool rows_slow;          // charge copies with short rows beside the pipeline (see estimate)
 };
 
-FormModel form_model(int form, int es, int64_t K, int slices_opt)
+FormModel form_model(int form, int slices_opt, double host_bytes)
 {
     FormModel f{};
+    f.ctas_per_sm = 1;
+    f.cluster = 1;
+    // strided copies with short rows slowed down in pipelines over tens of GiB of host memory;
+    // over less they run at two thirds of the link's rate
+    f.rows_slow = host_bytes > 8.0 * (1ull << 30);
     if (form == OOC_FORM_FP64) {
-        f.tile_m = 64; f.tile_n = 64; f.rate = 1.0e12; f.ctas_per_sm = 3;
+        f.tile = 16; f.grain = 64; f.rate = 1.09e12;
+        // 192 steps of 192 x 1024 x 32: 20.5 us each, of which 13.6 are their tiles at the rate,
+        // and 5.7 us between them
+        f.launch = 6e-6; f.step = 6e-6;
         f.products = 1; f.slices = 1;
-        // no measurable cost: 32768^3 with 180 GB of copies (0.85 s at the link rate) ran 64.16 s
-        // steps on 64.13 s of kernels
-        f.overlap_cost = 0.0;
-    } else if (form == OOC_FORM_BF16X3) {
-        // measured bf16 rate of the tensor-core kernel on whole-K blocks (1.42-1.64 PFLOP/s)
-        f.tile_m = 128; f.tile_n = 128; f.ctas_per_sm = 1;
-        f.products = 6; f.slices = 3;
-        f.rate = 1.4e15 / 6.0;
-        // copies beside tensor-core kernels share HBM and the power budget: 65536^3 with 309 GB
-        // H2D (1.46 s at the link rate) ran 2.84 s steps on 2.45 s of kernel-stream time
-        f.overlap_cost = 0.27;
-    } else {  // Ozaki
-        int s = slices_opt > 0 ? slices_opt : kOzakiSlicesGemm;
-        f.tile_m = 128; f.tile_n = 128; f.ctas_per_sm = 1;
-        f.slices = s; f.products = s * (s + 1) / 2;
-        const int planes = ozaki_planes(s);
-        f.rate = 1.38e15 / (planes * (planes + 1) / 2);
-        f.overlap_cost = 0.27;
+        // no measurable overlap cost: 32768^3 with 180 GB of copies (0.85 s at the link rate) ran
+        // 64.16 s steps on 64.13 s of kernels
+        return f;
     }
-    (void)es; (void)K;
+    f.tile = f.grain = 128;
+    f.cluster = 8;
+    f.step = 6e-6;
+    // copies beside tensor-core kernels share HBM and the power budget: BF16x3 65536^3 with 309 GB
+    // H2D (1.46 s at the link rate) ran 2.84 s steps on 2.45 s of kernel-stream time
+    f.overlap_cost = 0.27;
+    if (form == OOC_FORM_BF16X3) {
+        // 282 TFLOP/s on 1216 tiles of K 8192; one tile of K 4096 26.5 us, 192 of K 64 20 us
+        f.rate = 2.8e14; f.exchange = 5e-6; f.launch = 9e-6;
+        f.products = 6; f.slices = 3;
+        f.split_bytes = 10;
+    } else {
+        // 72 TFLOP/s (21 products) there; one tile of K 4096 57 us, 192 of K 64 49 us
+        const int s = slices_opt > 0 ? slices_opt : kOzakiSlicesGemm;
+        const int planes = ozaki_planes(s);
+        f.rate = 1.5e15 / (planes * (planes + 1) / 2); f.exchange = 4e-6; f.launch = 18e-6;
+        f.slices = s; f.products = s * (s + 1) / 2;
+        f.split_bytes = 8 + 8 + 2 * planes;
+    }
     return f;
 }
+
+// The FP64 estimate by waves of 64 x 64 areas, three to an SM, that large problems are planned
+// with.  Blocks of several such waves keep every SM busy to within a percent, less than either
+// estimate resolves, and this one's choices are the ones their pipelines were measured with
+// (32768^3 in 4 GiB: 2048 x 8192 blocks, 0.999 of the kernel's rate).
+FormModel fp64_waves()
+{
+    FormModel f = form_model(OOC_FORM_FP64, 0, 0.0);
+    f.tile = 64; f.rate = 1.0e12; f.ctas_per_sm = 3;
+    f.launch = 0; f.step = 8e-6;
+    f.rows_slow = true;
+    return f;
+}
+
+// Blocks large enough for that: a wave of areas
+bool whole_waves(const Plan& p, int sms) { return cdiv(p.mb, 64) * cdiv(p.nb, 64) >= 3 * (int64_t)sms; }
 
 }  // namespace
 
@@ -97,7 +132,7 @@ size_t split_aux_bytes(const Plan& p, int64_t rows)
 
 namespace {
 
-void layout(Plan& p, const FormModel& f)
+void layout(Plan& p)
 {
     const int64_t ald = 16;  // 16 elements: 128-byte rows for FP64, 64 for FP32
     const int64_t a_rows = p.ta ? p.kb : p.mb, a_cols = p.ta ? p.mb : p.kb;
@@ -115,7 +150,6 @@ void layout(Plan& p, const FormModel& f)
         p.a_aux = split_aux_bytes(p, p.mb);
         p.b_aux = split_aux_bytes(p, p.nb);
     }
-    (void)f;
     // split forms keep raw staging areas (two for A; one for B when whole-K B slices are
     // loaded once per block column, else two) and planes per slot
     p.staged = p.form != OOC_FORM_FP64;
@@ -230,10 +264,22 @@ bool narrow_rows(const Plan& p, int mat)
     return !contiguous && width * p.es < 64 * 1024;
 }
 
+// One launch of the tile kernel on a rows x cols block, k long.  The busiest SM decides: it
+// takes ceil(tiles / SMs) tiles, or the launch's few tiles are each shared by a cluster.
+double launch_seconds(const FormModel& f, int sms, int64_t rows, int64_t cols, int64_t k)
+{
+    const int64_t tiles = cdiv(rows, f.tile) * cdiv(cols, f.tile), slots = (int64_t)sms * f.ctas_per_sm;
+    const double tile = 2.0 * f.tile * f.tile * k * slots / f.rate;
+    const double floor = f.cluster > 1 ? f.launch : 0.0;  // a tile's drain and epilogue
+    double best = (double)cdiv(tiles, slots) * std::max(tile, floor);
+    for (int c = 2; c <= f.cluster; c *= 2)
+        best = std::min(best, (double)cdiv(tiles, sms / c) * std::max(tile / c + f.exchange, floor));
+    return best + f.launch;
+}
+
 double estimate(const Plan& p, const FormModel& f, int sms, double h2d_gbps, double d2h_gbps)
 {
-    const double slots_total = (double)sms * f.ctas_per_sm;
-    // compute: per step waves x per-tile time, summed over full / ragged blocks
+    // compute: the tiles of each step's launch, summed over full / ragged blocks and K chunks
     double t_comp = 0;
     const int64_t hf = p.M / p.mb, wf = p.N / p.nb;
     const int64_t mr = p.M - hf * p.mb, nr = p.N - wf * p.nb;
@@ -252,16 +298,12 @@ double estimate(const Plan& p, const FormModel& f, int sms, double h2d_gbps, dou
             if (rag_row) parts[rag_col ? 3 : 1].count += 1;
         }
     }
-    const double tile_time_per_k = 2.0 * f.tile_m * f.tile_n * slots_total / f.rate;
     for (auto& pt : parts) {
-        if (pt.count == 0 || pt.rows == 0 || pt.cols == 0) continue;
-        const double tiles = (double)cdiv(pt.rows, f.tile_m) * cdiv(pt.cols, f.tile_n);
-        const double waves = std::ceil(tiles / slots_total);
-        t_comp += pt.count * waves * tile_time_per_k * (double)p.K;
+        if (pt.count == 0 || pt.rows == 0 || pt.cols == 0 || p.K == 0) continue;
+        t_comp += pt.count * ((p.nkc - 1) * launch_seconds(f, sms, pt.rows, pt.cols, p.kb) +
+                              launch_seconds(f, sms, pt.rows, pt.cols, p.K - (p.nkc - 1) * p.kb));
     }
     const double bw_h = h2d_gbps * 1e9, bw_d = d2h_gbps * 1e9;
-    const double t_link = std::max({p.h2d_bytes / bw_h, p.d2h_bytes / bw_d,
-                                    (p.h2d_bytes + p.d2h_bytes) / (0.85 * (bw_h + bw_d))});
     const double es = p.es;
     const double fill = ((double)p.mb * p.kb + (double)p.kb * p.nb * std::min<int64_t>(p.nkc, p.nB)) * es / bw_h;
     const double drain = (double)p.mb * p.nb * es / bw_d;
@@ -271,11 +313,6 @@ double estimate(const Plan& p, const FormModel& f, int sms, double h2d_gbps, dou
     const bool staged_prefetch = p.staged && p.b_prefetch && p.nkc == 1 && p.h >= 2;
     if (p.nB < 2 * p.nkc && p.nkc <= p.nB && !staged_prefetch) bubbles = (double)(p.w - 1) * p.K * p.nb * es / bw_h;
     const double steps = (double)active_blocks(p) * p.nkc;
-    // Strided host copies with short rows (< 64 KiB) run far below the link
-    // rate on this host link and were seen to slow down further as more host
-    // memory is touched; charge them at a quarter of the link rate, outside
-    // the overlap.
-    double narrow = 0;
     const double A = (double)p.M * p.K * es, B = (double)p.K * p.N * es, C = (double)p.M * p.N * es;
     double a_loads = (p.h == 1 && p.nkc <= p.nA) ? A : A * p.w;
     double b_loads = (p.nkc <= p.nB) ? B : B * p.h;
@@ -286,11 +323,21 @@ double estimate(const Plan& p, const FormModel& f, int sms, double h2d_gbps, dou
         b_loads *= c_frac;
         c_moved = p.d2h_bytes * (p.beta_nz ? 2.0 : 1.0);
     }
+    double narrow = 0;
     if (narrow_rows(p, kMatA)) narrow += a_loads;
     if (narrow_rows(p, kMatB)) narrow += b_loads;
     if (narrow_rows(p, kMatC)) narrow += c_moved;
+    // Strided host copies with short rows (< 64 KiB): in pipelines over much host memory they run
+    // far below the link rate and were seen to slow down further as more of it is touched, so they
+    // are charged at a quarter of the link rate, outside the overlap; else they take half again
+    // as long as contiguous ones.
+    const double slow = f.rows_slow ? 0.0 : 0.5 * narrow;
+    const double t_link = std::max({(p.h2d_bytes + slow) / bw_h, p.d2h_bytes / bw_d,
+                                    (p.h2d_bytes + p.d2h_bytes + slow) / (0.85 * (bw_h + bw_d))});
+    if (f.split_bytes > 0)  // the split of every slice loaded, on the compute stream
+        t_comp += (a_loads + b_loads) / es * f.split_bytes / 3e12 + (steps + (double)p.w * p.nkc) * 8e-6;
     return std::max(t_comp, t_link) + f.overlap_cost * std::min(t_comp, t_link) + fill + drain + bubbles +
-           steps * 8e-6 + narrow / (0.25 * bw_h);
+           steps * f.step + (f.rows_slow ? narrow / (0.25 * bw_h) : 0.0);
 }
 
 bool paper_plan(const PlanRequest& rq, Plan& best, std::string& why)
@@ -350,7 +397,9 @@ int make_plan(const PlanRequest& rq, Plan& p, std::string& why)
         why = "opts->slices must be 0 or 2.." + std::to_string(kOzakiMaxSlices);
         return OOC_ERR_INVALID_ARG;
     }
-    const FormModel f = form_model(form, rq.es, rq.K, rq.opts.slices);
+    const double host_bytes = ((double)rq.M * rq.K + (double)rq.K * rq.N + (double)rq.M * rq.N) * rq.es;
+    const FormModel f = form_model(form, rq.opts.slices, host_bytes), waves = fp64_waves();
+    const bool fp64 = form == OOC_FORM_FP64;
     p.slices = f.slices; p.products = f.products;
     const int sms = device_sm_count();
     if (rq.M <= 0 || rq.N <= 0) {
@@ -362,7 +411,7 @@ int make_plan(const PlanRequest& rq, Plan& p, std::string& why)
         if (!paper_plan(rq, p, why)) return OOC_ERR_BUDGET;
         p.paper = true;
         p.h = rq.M / p.mb; p.w = rq.N / p.nb; p.nkc = 1;
-        layout(p, f);
+        layout(p);
         traffic(p);
         p.est_seconds = estimate(p, f, sms, rq.h2d_gbps, rq.d2h_gbps);
         return OOC_OK;
@@ -384,8 +433,8 @@ int make_plan(const PlanRequest& rq, Plan& p, std::string& why)
             if (s < X && std::find(v.begin(), v.end(), s) == v.end()) v.push_back(s);
         return v;
     };
-    const std::vector<int64_t> mbs = sizes(rq.M, f.tile_m, rq.opts.mb);
-    const std::vector<int64_t> nbs = sizes(rq.N, f.tile_n, rq.opts.nb);
+    const std::vector<int64_t> mbs = sizes(rq.M, f.grain, rq.opts.mb);
+    const std::vector<int64_t> nbs = sizes(rq.N, f.grain, rq.opts.nb);
     std::vector<int64_t> kbs, split_chunks;
     if (form != OOC_FORM_FP64) {
         // split forms: whole-K slices (measured fastest on GB300 whenever they fit), else up to 16 K
@@ -413,17 +462,51 @@ int make_plan(const PlanRequest& rq, Plan& p, std::string& why)
         for (int64_t kb = 32; kb >= 16; kb /= 2)
             if (kb < rq.K) kbs.push_back(kb);
     }
-    const std::vector<int> nAs = rq.opts.depth > 0 ? std::vector<int>{rq.opts.depth} : std::vector<int>{2, 3};
-    const std::vector<int> nCs = rq.opts.c_buffers > 0 ? std::vector<int>{rq.opts.c_buffers} : std::vector<int>{2, 3};
-
-    bool found = false;
-    Plan best;
-    double best_t = std::numeric_limits<double>::infinity();
     std::vector<Plan>* keep = collect_;  // candidate collection (plan_candidates)
-    std::vector<Plan> tri_pool;          // triangular updates: candidates awaiting the exact estimate
+    // Longer A and C rings never win by the estimate (it does not see them, save that three A
+    // slots hold a short block row's chunks), so they are only tried when candidates are listed.
+    const std::vector<int> nAs = rq.opts.depth > 0 ? std::vector<int>{rq.opts.depth} : std::vector<int>{2, 3};
+    const std::vector<int> nCs = rq.opts.c_buffers > 0 ? std::vector<int>{rq.opts.c_buffers}
+                                 : keep               ? std::vector<int>{2, 3}
+                                                      : std::vector<int>{2};
+
+    // The fastest plan by each estimate: FP64 is planned by waves first and by the launches' own
+    // balance when that leaves blocks below a wave.
+    struct Choice {
+        bool found = false;
+        Plan plan;
+        double t = std::numeric_limits<double>::infinity();
+        // prefer faster; near-ties go to fewer device bytes
+        void offer(const Plan& c, double est)
+        {
+            if (!found || est < t * (1 - 1e-9) || (est <= t * (1 + 1e-9) && c.device_bytes < plan.device_bytes)) {
+                plan = c;
+                plan.est_seconds = t = est;
+                found = true;
+            }
+        }
+    } best, best_waves;
+    std::vector<double> keep_waves;  // estimates by waves of the kept candidates
+    auto offer = [&](Plan c) {
+        traffic(c);
+        c.est_seconds = estimate(c, f, sms, rq.h2d_gbps, rq.d2h_gbps);
+        const double ew = fp64 ? estimate(c, waves, sms, rq.h2d_gbps, rq.d2h_gbps) : 0.0;
+        if (keep) {
+            keep->push_back(c);
+            keep_waves.push_back(ew);
+        }
+        best.offer(c, c.est_seconds);
+        if (fp64) best_waves.offer(c, ew);
+    };
+    struct Ranked {
+        int64_t mb, nb, kb;
+        int nA, nB, nC;
+        double est, waves;
+    };
+    std::vector<Ranked> tri_pool;  // triangular updates: candidates awaiting the exact estimate
     for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) {
-        if (found || !tri_pool.empty() || split_chunks.empty()) break;
+        if (best.found || !tri_pool.empty() || split_chunks.empty()) break;
         kbs = split_chunks;  // no whole-K split plan fits: stream K in chunks
     }
     for (int64_t kb : kbs) {
@@ -440,52 +523,52 @@ int make_plan(const PlanRequest& rq, Plan& p, std::string& why)
                             c.mb = mb; c.nb = nb; c.kb = kb;
                             c.h = cdiv(rq.M, mb); c.w = cdiv(rq.N, nb); c.nkc = nkc;
                             c.nA = nA; c.nB = nB; c.nC = nC;
+                            if (!keep && rq.opts.depth == 0 && nA == 3 && !(c.h == 1 && nkc == 3)) continue;
                             if (c.nR > c.h * c.w) continue;        // resident blocks need this blocking
                             if (c.nR == c.h * c.w) c.nC = 0;       // every block resident: no C ring
-                            layout(c, f);
+                            layout(c);
                             if (c.device_bytes > rq.budget) continue;
-                            if (c.tri) {
-                                // triangular updates: rank by the full-update estimate first (the exact
-                                // one walks every block column); the best of these are re-ranked below
-                                Plan full = c;
-                                full.tri = 0;
-                                traffic(full);
-                                full.est_seconds = estimate(full, f, sms, rq.h2d_gbps, rq.d2h_gbps);
-                                c.est_seconds = full.est_seconds;
-                                tri_pool.push_back(c);
+                            if (!c.tri) {
+                                offer(c);
                                 continue;
                             }
+                            // triangular updates: rank by the full-update estimates first (the exact
+                            // ones walk every block column); the best of these are re-ranked below
+                            c.tri = 0;
                             traffic(c);
-                            c.est_seconds = estimate(c, f, sms, rq.h2d_gbps, rq.d2h_gbps);
-                            if (keep) keep->push_back(c);
-                            // prefer faster; near-ties go to fewer device bytes
-                            if (!found || c.est_seconds < best_t * (1 - 1e-9) ||
-                                (c.est_seconds <= best_t * (1 + 1e-9) && c.device_bytes < best.device_bytes)) {
-                                best = c; best_t = c.est_seconds; found = true;
-                            }
+                            tri_pool.push_back({mb, nb, kb, c.nA, c.nB, c.nC,
+                                                estimate(c, f, sms, rq.h2d_gbps, rq.d2h_gbps),
+                                                fp64 ? estimate(c, waves, sms, rq.h2d_gbps, rq.d2h_gbps) : 0.0});
                         }
     }
     }
-    if (!tri_pool.empty()) {
-        const size_t top = std::min<size_t>(tri_pool.size(), 48);
+    const size_t top = std::min<size_t>(tri_pool.size(), keep ? 48 : 16);
+    auto rerank = [&](double Ranked::*key) {
         std::partial_sort(tri_pool.begin(), tri_pool.begin() + top, tri_pool.end(),
-                          [](const Plan& a, const Plan& b) { return a.est_seconds < b.est_seconds; });
+                          [&](const Ranked& a, const Ranked& b) { return a.*key < b.*key; });
         for (size_t q = 0; q < top; ++q) {
-            Plan c = tri_pool[q];
-            traffic(c);
-            c.est_seconds = estimate(c, f, sms, rq.h2d_gbps, rq.d2h_gbps);
-            if (keep) keep->push_back(c);
-            if (!found || c.est_seconds < best_t * (1 - 1e-9) ||
-                (c.est_seconds <= best_t * (1 + 1e-9) && c.device_bytes < best.device_bytes)) {
-                best = c; best_t = c.est_seconds; found = true;
-            }
+            const Ranked& r = tri_pool[q];
+            Plan c = p;
+            c.mb = r.mb; c.nb = r.nb; c.kb = r.kb;
+            c.h = cdiv(rq.M, c.mb); c.w = cdiv(rq.N, c.nb); c.nkc = rq.K == 0 ? 1 : cdiv(rq.K, c.kb);
+            c.nA = r.nA; c.nB = r.nB; c.nC = r.nC;
+            layout(c);
+            offer(c);
         }
+    };
+    if (top) rerank(&Ranked::est);
+    if (top && fp64) rerank(&Ranked::waves);
+    // (a session's blocks too: they are kept in HBM, not balanced launch by launch)
+    if (fp64 && best_waves.found && (whole_waves(best_waves.plan, sms) || rq.session_step > 0 || rq.nR > 0)) {
+        best = best_waves;
+        if (keep)
+            for (size_t q = 0; q < keep->size(); ++q) (*keep)[q].est_seconds = keep_waves[q];
     }
-    if (!found) {
+    if (!best.found) {
         why = "budget of " + std::to_string(rq.budget) + " bytes is below the smallest plan";
         return OOC_ERR_BUDGET;
     }
-    p = best;
+    p = best.plan;
     if (!keep && (rq.opts.flags & OOC_PLAN_MODEL) && !rq.tri) {  // the model is trained on full updates
         std::vector<float> params;
         if (costmodel_get(params)) {
@@ -536,14 +619,14 @@ int plan_candidates(const PlanRequest& rq, int max_n, std::vector<Plan>& out, st
 void plan_features(const Plan& p, const PlanRequest& rq, float* f)
 {
     auto lg = [](double x) { return (float)std::log2(std::max(x, 1.0)); };
-    const FormModel fm = form_model(p.form, p.es, p.K, p.slices);
-    const double slots = (double)device_sm_count() * fm.ctas_per_sm;
-    const double tiles = (double)cdiv(p.mb, fm.tile_m) * cdiv(p.nb, fm.tile_n);
-    const double waves = std::ceil(tiles / slots);
+    // how evenly a full block's tiles load the SMs (few tiles shared by clusters count as even)
+    const FormModel fm = form_model(p.form, p.slices, 0.0);
+    const double whole = 2.0 * p.mb * p.nb * (double)p.kb / fm.rate;
+    const double even = whole / std::max(1e-12, launch_seconds(fm, device_sm_count(), p.mb, p.nb, p.kb));
     f[0] = lg((double)p.M) / 16; f[1] = lg((double)p.N) / 16; f[2] = lg((double)std::max<int64_t>(p.K, 1)) / 16;
     f[3] = p.form == OOC_FORM_FP64; f[4] = p.form == OOC_FORM_OZAKI; f[5] = p.form == OOC_FORM_BF16X3;
     f[6] = lg((double)rq.budget) / 40;
-    f[7] = (float)(tiles / (waves * slots));
+    f[7] = (float)std::min(1.0, even);
     f[8] = lg((double)p.mb) / 16; f[9] = lg((double)p.nb) / 16; f[10] = lg((double)p.kb) / 16;
     f[11] = p.nA / 3.0f; f[12] = lg((double)p.nB + 1) / 8;
     f[13] = (narrow_rows(p, kMatA) + narrow_rows(p, kMatB) + narrow_rows(p, kMatC)) / 3.0f;
