@@ -430,18 +430,21 @@ __global__ void __launch_bounds__(kLuThreads) narrow_lu_kernel(double* P, int64_
 
 // Unblocked LU with partial pivoting of an m x nw panel (nw <= 32), in place, by one
 // cluster of CTAs: CTA g keeps rows [g * rows_per_cta, (g + 1) * rows_per_cta) in its
-// shared memory from the first column to the last, one row per thread and 256 rows.
+// shared memory from the first column to the last.
 //
 // What it waits for is the chain of pivots.  Per column each CTA finds its candidate
-// (largest |a|, smallest row on ties) and writes it,
-// its reciprocal and its row into every CTA's shared memory, as the owner of row j does
-// with row j; after one cluster barrier (about 400 clocks, against microseconds for a
-// barrier through global memory) every warp picks the same winner from its own copy.
-// Nothing else is exchanged, and the interchange, the multipliers and the update touch
-// only a thread's own rows.  The published copies alternate between two buffers by
-// column parity: a slot is rewritten two columns later, after a barrier that every CTA
-// reaches only when it has finished reading it.  Quotients and sums are those of
-// narrow_lu_kernel, which takes the panels too tall for one cluster's shared memory.
+// (largest |a|, smallest row on ties) and writes it, its reciprocal and its row into
+// every CTA's shared memory, as the owner of row j does with row j; the writes count
+// themselves off on the receiver's mbarrier, so a CTA waits for data and for nothing else
+// (a cluster barrier in their place, with the fence that orders the writes before it, took
+// a quarter of the column's 6200 clocks).  Then every warp picks the same winner from its
+// own copy, and the interchange, the multipliers and the update touch only a row's own
+// threads: four per row up to 32 rows a CTA, two up to 64, one above, since the update's
+// FP64 instructions need four warps to run at the SM's rate.  The published copies
+// alternate between two buffers by column parity: a CTA writes column j + 2's when it has
+// all of column j + 1's, which its receivers sent after they had read column j's.
+// Quotients and sums are those of narrow_lu_kernel, which takes the panels too tall for one
+// cluster's shared memory.
 constexpr int kLuClusterCols = 32;
 constexpr int kLuClusterMax = 16;             // CTAs of the cluster (above 8: not portable, sm_103 allows it)
 constexpr int kLuClusterLd = kLuClusterCols + 1;
@@ -453,17 +456,13 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster(void* p, int rank, long long v)
+// 8 bytes to the same place of CTA `rank`'s shared memory, counted on its mbarrier `bar`
+__device__ __forceinline__ void st_counted(void* p, uint64_t* bar, int rank, long long v)
 {
-    asm volatile("st.shared::cluster.s64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster(void* p, int rank, double v)
-{
-    st_cluster(p, rank, (long long)__double_as_longlong(v));
-}
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
+                     cluster_addr(p, rank)),
+                 "l"(v), "r"(cluster_addr(bar, rank))
+                 : "memory");
 }
 
 // A pivot candidate: the bits of |a| plus one, which order like it (0: nothing
@@ -487,86 +486,107 @@ struct PivotCand {
 
 __global__ void __launch_bounds__(kLuThreads) lu_cluster_kernel(double* P, int64_t ldp, int m, int nw,
                                                                 int rows_per_cta, int64_t* piv,
-                                                                unsigned long long* info, int64_t gofs)
+                                                                unsigned long long* info, int64_t gofs, int* err)
 {
     extern __shared__ double S[];  // the CTA's rows, stride kLuClusterLd
     __shared__ double crow[2][kLuClusterMax][kLuClusterCols], jrow[2][kLuClusterCols], cinv[2][kLuClusterMax];
     __shared__ unsigned long long ckey[2][kLuClusterMax], crow_at[2][kLuClusterMax];
     __shared__ unsigned long long wkey[2][kLuWarps];
     __shared__ int wrow[2][kLuWarps];
+    __shared__ uint64_t arrived[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int G = (int)gridDim.x, rank = (int)blockIdx.x;  // one cluster
     const int r0 = rank * rows_per_cta, nloc = max(0, min(m - r0, rows_per_cta));
+    const int tpr = rows_per_cta <= 32 ? 4 : rows_per_cta <= 64 ? 2 : 1;  // threads of a row, in one warp
+    const int row0 = tid / tpr, part = tid % tpr, row_step = kLuThreads / tpr;
     for (int e = tid; e < nloc * kLuClusterCols; e += kLuThreads) {
         const int r = e / kLuClusterCols, k = e % kLuClusterCols;
         if (k < nw) S[r * kLuClusterLd + k] = P[(int64_t)(r0 + r) * ldp + k];
     }
+    if (tid == 0) {
+        mbar_init(&arrived[0], 1);
+        mbar_init(&arrived[1], 1);
+        mbar_fence_init();
+    }
     __syncthreads();
-    cluster_barrier();  // every CTA of the cluster runs before the first write to another's memory
+    cluster_sync();  // every CTA of the cluster runs, its mbarriers ready, before the first write to it
+    const uint32_t expected = 8u * (uint32_t)(G * (nw + 3) + nw);
+    bool ok = true;
 #pragma unroll 1
-    for (int j = 0; j < nw; ++j) {
+    for (int j = 0; j < nw && ok; ++j) {
         const int b = j & 1;
         // local candidate over own rows i >= j, smallest row on ties
         PivotCand c{0, INT_MAX};
-        for (int r = tid; r < nloc; r += kLuThreads) {
-            const unsigned long long k =
-                (unsigned long long)__double_as_longlong(S[r * kLuClusterLd + j]) & 0x7FFFFFFFFFFFFFFFull;
-            if (r0 + r >= j && k <= 0x7FF0000000000000ull) c.take(k + 1, r0 + r);  // a NaN is never chosen
-        }
+        if (part == 0)
+            for (int r = row0; r < nloc; r += row_step) {
+                const unsigned long long k =
+                    (unsigned long long)__double_as_longlong(S[r * kLuClusterLd + j]) & 0x7FFFFFFFFFFFFFFFull;
+                if (r0 + r >= j && k <= 0x7FF0000000000000ull) c.take(k + 1, r0 + r);  // a NaN is never chosen
+            }
         c.reduce();
         if (lane == 0) { wkey[b][warp] = c.key; wrow[b][warp] = c.row; }
+        if (tid == 0) mbar_arrive_expect_tx(&arrived[b], expected);
         __syncthreads();
         c = PivotCand{lane < kLuWarps ? wkey[b][lane] : 0, lane < kLuWarps ? wrow[b][lane] : INT_MAX};
         c.reduce();
-        // publish it and, from its owner, row j: each warp writes to every eighth CTA
-        const double cand = c.key && lane < nw ? S[(c.row - r0) * kLuClusterLd + lane] : 0.0;
-        const double own_j = j >= r0 && j < r0 + nloc && lane < nw ? S[(j - r0) * kLuClusterLd + lane] : 0.0;
-        for (int q = warp; q < G; q += kLuWarps) {
-            if (lane < nw) {
-                st_cluster(&crow[b][rank][lane], q, cand);
-                if (j >= r0 && j < r0 + nloc) st_cluster(&jrow[b][lane], q, own_j);
+        // publish it and, from its owner, row j; the last warp takes its reciprocal
+        const double* cand = S + (c.key ? c.row - r0 : 0) * kLuClusterLd;
+        if (warp < kLuWarps - 1) {
+            const bool own_j = j >= r0 && j < r0 + nloc;
+            const long long cv = c.key && lane < nw ? __double_as_longlong(cand[lane]) : 0;
+            const long long jv = own_j && lane < nw ? __double_as_longlong(S[(j - r0) * kLuClusterLd + lane]) : 0;
+            for (int q = warp; q < G; q += kLuWarps - 1) {
+                if (lane < nw) {
+                    st_counted(&crow[b][rank][lane], &arrived[b], q, cv);
+                    if (own_j) st_counted(&jrow[b][lane], &arrived[b], q, jv);
+                }
+                if (lane == 0) {
+                    st_counted(&ckey[b][rank], &arrived[b], q, (long long)c.key);
+                    st_counted(&crow_at[b][rank], &arrived[b], q, (long long)c.row);
+                }
             }
-            if (lane == 0) {
-                st_cluster(&ckey[b][rank], q, (long long)c.key);
-                st_cluster(&crow_at[b][rank], q, (long long)c.row);
-            }
+        } else {
+            const double inv = c.key ? reciprocal_of(cand[j]) : 0.0;
+            if (lane < G) st_counted(&cinv[b][rank], &arrived[b], lane, __double_as_longlong(inv));
         }
-        if (warp == 0) {
-            const double inv = reciprocal_of(__shfl_sync(0xffffffffu, cand, j));
-            if (lane < G) st_cluster(&cinv[b][rank], lane, inv);
-        }
-        cluster_barrier();
+        // the whole CTA gives up together (it meets at barriers)
+        ok = __syncthreads_and(mbar_wait(&arrived[b], (uint32_t)(j >> 1) & 1u, err, kErrGridBarrier)) != 0;
+        if (!ok) break;
         // every warp reduces the candidates the same way: the global first maximum
         c = PivotCand{lane < G ? ckey[b][lane] : 0, lane < G ? (int)crow_at[b][lane] : INT_MAX};
         c.reduce();
-        const bool found = c.key != 0;
+        const bool found = c.key != 0, zero = c.key == 1;
         const int p = found ? c.row : j, owner = found ? p / rows_per_cta : 0;
         const double* src = found ? crow[b][owner] : jrow[b];
         const double pv = src[j], inv = found ? cinv[b][owner] : pv;  // nothing comparable: pv is NaN
-        const bool zero = c.key == 1;
         if (rank == 0 && tid == 0) {
             piv[j] = p;
             if (zero) atomicCAS(info, 0ull, (unsigned long long)(gofs + j + 1));
         }
         // own rows: row j becomes the pivot row, row p the old row j; those below j are
         // scaled and updated
-        for (int r = tid; r < nloc; r += kLuThreads) {
-            const int i = r0 + r;
+        for (int base = 0; base < nloc; base += row_step) {
+            const int r = base + row0, i = r0 + r;
             double* row = S + r * kLuClusterLd;
-            if (i < j) continue;
-            if (i == j || i == p) {
+            const bool mine = r < nloc, below = mine && i > j && !zero;
+            if (mine && (i == j || (i == p && p != j))) {
                 const double* from = i == j ? src : jrow[b];
-#pragma unroll 8
-                for (int k = 0; k < nw; ++k) row[k] = from[k];
-            }
-            if (i == j || zero) continue;
-            const double l = quotient(row[j], pv, inv);
-            row[j] = l;
 #pragma unroll 4
-            for (int k = j + 1; k < nw; ++k) row[k] = fma(-l, src[k], row[k]);
+                for (int k = part; k < nw; k += tpr) row[k] = from[k];
+            }
+            __syncwarp();
+            const double l = below ? quotient(row[j], pv, inv) : 0.0;
+            __syncwarp();
+            if (below) {
+                if (part == 0) row[j] = l;
+#pragma unroll 4
+                for (int k = j + 1 + part; k < nw; k += tpr) row[k] = fma(-l, src[k], row[k]);
+            }
         }
+        __syncwarp();
     }
-    __syncthreads();
+    cluster_sync();  // no CTA leaves while another may still write to it
+    if (!ok) return;
     for (int e = tid; e < nloc * kLuClusterCols; e += kLuThreads) {
         const int r = e / kLuClusterCols, k = e % kLuClusterCols;
         if (k < nw) P[(int64_t)(r0 + r) * ldp + k] = S[r * kLuClusterLd + k];
@@ -906,7 +926,7 @@ int panel_lu(double* P, int64_t ldp, int64_t m, int64_t n, int64_t* piv, int64_t
         cudaLaunchAttribute at;
         lu_cluster_config(cfg, at, cluster, (size_t)rows * kLuClusterLd * sizeof(double), d.st);
         const cudaError_t e =
-            cudaLaunchKernelEx(&cfg, lu_cluster_kernel, P, ldp, (int)m, (int)n, rows, piv, d.info, gofs);
+            cudaLaunchKernelEx(&cfg, lu_cluster_kernel, P, ldp, (int)m, (int)n, rows, piv, d.info, gofs, d.err);
         ++d.launches;
         if (e != cudaSuccess) {
             cudaGetLastError();
