@@ -82,6 +82,14 @@ __global__ void __launch_bounds__(kTrsmThreads) trsm_small_kernel(const double* 
     __shared__ double Tc[kSmall * LD];  // [column][row] of the lower system, zero elsewhere
     __shared__ double dg[kSmall], inv[kSmall];
     const int tid = threadIdx.x;
+    const int warp = tid >> 5, lane = tid & 31, l = lane & (L - 1);
+    const int64_t v = ((int64_t)blockIdx.x * (kTrsmThreads / 32) + warp) * (32 / L) + lane / L;
+    double x[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int i = j * L + l, e = lower ? i : n - 1 - i;
+        x[j] = i < n && v < nvec ? P[e * es + v * vs] : 0.0;
+    }
 #pragma unroll 8
     for (int idx = tid; idx < kSmall * kSmall; idx += kTrsmThreads) {
         const int sr = idx >> 6, sc = idx & 63;  // stored row and column: columns fastest for coalescing
@@ -91,19 +99,11 @@ __global__ void __launch_bounds__(kTrsmThreads) trsm_small_kernel(const double* 
         double t = 0.0;
         if (in && (r > c || (r == c && !unit))) t = T[(int64_t)sr * ldt + sc];
         Tc[c * LD + r] = t;
-        if (r == c) {
-            dg[r] = t;
-            inv[r] = unit || !in ? 1.0 : reciprocal_of(t);
-        }
+        if (r == c) dg[r] = t;
     }
-    const int warp = tid >> 5, lane = tid & 31, l = lane & (L - 1);
-    const int64_t v = ((int64_t)blockIdx.x * (kTrsmThreads / 32) + warp) * (32 / L) + lane / L;
-    double x[R];
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const int i = j * L + l, e = lower ? i : n - 1 - i;
-        x[j] = i < n && v < nvec ? P[e * es + v * vs] : 0.0;
-    }
+    __syncthreads();
+    // the reciprocals by two whole warps: a division holds the pipe the same for one lane or 32
+    if (tid < kSmall) inv[tid] = unit || tid >= n ? 1.0 : reciprocal_of(dg[tid]);
     __syncthreads();
 #pragma unroll
     for (int jr = 0; jr < R; ++jr) {
