@@ -53,6 +53,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 
 #include "ooc_internal.hpp"
 #include "tc_common.cuh"
@@ -172,23 +173,29 @@ __device__ __forceinline__ void round_pair(uint64_t v, uint64_t sc, int& i0, int
     i1 = (int)(((uint32_t)(t >> 32) << 2) + (uint32_t)(u >> 32) - bias);
 }
 
-// t * 2^e, rounded once (to nearest, ties to even) from the 64-bit integer, with
+// Results outside the normal range, rounded by the library.
+__device__ __noinline__ double scaled_slowly(long long t, int e) { return ldexp((double)t, e); }
+
+// t * 2^e, rounded once (to nearest, ties to even) from the 64-bit integer, with 32-bit
 // integer operations: every instruction per output on the FP64 pipe holds it for 9700
-// clocks a tile, a comparison as much as a conversion, a scaling or a multiplication.  Results outside the normal range go through ldexp.
+// clocks a tile, a comparison as much as a conversion, a scaling or a multiplication.
 __device__ __forceinline__ double fixed_to_f64(long long t, int e)
 {
-    if (t == 0) return 0.0;
-    const unsigned long long a = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
-    const int lz = __clzll((long long)a);
-    const int be = 1023 + 63 - lz + e;  // biased exponent before rounding
-    if (be < 1 || be > 2045) return ldexp((double)t, e);
-    const unsigned long long n = a << lz;          // bit 63 set
-    unsigned long long m = n >> 11;                // 53 bits
-    const unsigned rem = (unsigned)n & 0x7FFu;
-    if (rem > 0x400u || (rem == 0x400u && (m & 1ull))) ++m;
-    // the implicit bit of m (and a carry out of the rounding) adds to the exponent field
-    const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + m;
-    return __longlong_as_double((long long)(bits | (t < 0 ? 0x8000000000000000ull : 0ull)));
+    const long long sign = t >> 63;
+    const unsigned long long a = (unsigned long long)((t ^ sign) - sign);
+    const uint32_t h = (uint32_t)(a >> 32), l = (uint32_t)a;
+    const uint32_t top = h ? h : l, next = h ? l : 0u;
+    const int lz = __clz((int)top);
+    const uint32_t x = __funnelshift_l(next, top, lz), y = next << (lz & 31);  // bit 31 of x set (t != 0)
+    const int be = 1023 + 63 - lz - (h ? 0 : 32) + e;  // biased exponent before rounding
+    if ((uint32_t)(be - 1) >= 2045u && top) return scaled_slowly(t, e);
+    const uint32_t ml = __funnelshift_r(y, x, 11);      // the 53 bits of x : y above the 11 dropped ones
+    const uint32_t up = ((y & 0x7FFu) + 0x3FFu + (ml & 1u)) >> 11;
+    // the implicit bit of the mantissa (and a carry out of the rounding) adds to the exponent
+    const uint32_t mh = ((uint32_t)(be - 1) << 20) + (x >> 11);
+    const unsigned long long m = (((unsigned long long)mh << 32) | ml) + up;
+    const uint32_t hi = (uint32_t)(m >> 32) | ((uint32_t)sign & 0x80000000u);
+    return top ? __hiloint2double((int)hi, (int)(uint32_t)m) : 0.0;
 }
 
 __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_constant__ CUtensorMap tmA,
@@ -375,17 +382,25 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
             const int re = (p.row_exp && row_me < p.M ? p.row_exp[row_me] : 0) + 2 - p.frac;
             const int row0 = tm * BM + q4 * 32 + (lane & ~3), col0 = tn * BN + quarter * 32 + (lane & 3);
             double* const c_lane = p.C + (int64_t)row0 * p.ldc + col0;
-            auto emit = [&](int pass, const long long (&t)[4]) {
+            const int rows_left = p.M - row0;
+            // read_c and scale are compile-time: a predicated-off instruction holds the FP64 pipe too
+            auto emit = [&](auto read_c, auto scale, int pass, const long long (&t)[4]) {
                 const int col = col0 + pass * 4;
                 double* const c = c_lane + pass * 4;
                 bool keep[4];
                 double old[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int64_t d = (int64_t)col - (row0 + i);
-                    keep[i] = col < p.N && row0 + i < p.M &&
-                              (p.tri == 0 || (p.tri == 1 ? d <= p.tri_off : d >= p.tri_off));
-                    old[i] = keep[i] && p.read_c ? c[i * p.ldc] : 0.0;
+                for (int i = 0; i < 4; ++i) keep[i] = col < p.N && i < rows_left;
+                if (p.tri) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int64_t d = (int64_t)col - (row0 + i);
+                        keep[i] = keep[i] && (p.tri == 1 ? d <= p.tri_off : d >= p.tri_off);
+                    }
+                }
+                if constexpr (read_c.value) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) old[i] = keep[i] ? c[i * p.ldc] : 0.0;
                 }
                 double v[4];
 #pragma unroll
@@ -393,12 +408,12 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     v[j] = fixed_to_f64(p.alpha_one < 0 ? -t[j] : t[j],
                                         re + __shfl_sync(0xffffffffu, ce_lane, pass * 4 + j));
                 }
-                if (p.alpha_one == 0) {
+                if constexpr (scale.value) {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) v[j] *= p.alpha;
                 }
                 transpose4(v, lane);
-                if (p.read_c) {
+                if constexpr (read_c.value) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) v[i] = fma(p.beta, old[i], v[i]);
                 }
@@ -407,32 +422,45 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     if (keep[i]) c[i * p.ldc] = v[i];
             };
             long long* part = reinterpret_cast<long long*>(ring);  // [column][row]
-            if (p.cluster == 1) {
-                if (ok) {
-#pragma unroll
-                    for (int pass = 0; pass < 8; ++pass) {
-                        const long long t[4] = {acc[pass * 4], acc[pass * 4 + 1], acc[pass * 4 + 2], acc[pass * 4 + 3]};
-                        emit(pass, t);
-                    }
-                }
-            } else {
+            if (p.cluster > 1) {
                 // the tile's stages are consumed: its ring carries the partial sums
                 if (ok) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) part[(quarter * 32 + j) * BM + row_in_tile] = acc[j];
                 }
                 cluster_sync();
-                if (ok) {
-                    for (int pass = rank; pass < 8; pass += p.cluster) {
-                        long long t[4] = {0, 0, 0, 0};
-                        const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
-                        for (int q = 0; q < p.cluster; ++q) {
+            }
+            auto store = [&](auto read_c, auto scale) {
+                if (p.cluster == 1) {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) t[j] += ld_cluster(at + j * BM * 8, q);
-                        }
-                        emit(pass, t);
+                    for (int pass = 0; pass < 8; ++pass) {
+                        const long long t[4] = {acc[pass * 4], acc[pass * 4 + 1], acc[pass * 4 + 2], acc[pass * 4 + 3]};
+                        emit(read_c, scale, pass, t);
                     }
+                    return;
                 }
+#pragma unroll 1
+                for (int pass = rank; pass < 8; pass += p.cluster) {
+                    long long t[4] = {0, 0, 0, 0};
+                    const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
+                    for (int q = 0; q < p.cluster; ++q) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) t[j] += ld_cluster(at + j * BM * 8, q);
+                    }
+                    emit(read_c, scale, pass, t);
+                }
+            };
+            if (ok) {
+                if (p.alpha_one == 0) {
+                    if (p.read_c) store(std::true_type{}, std::true_type{});
+                    else store(std::false_type{}, std::true_type{});
+                } else if (p.read_c) {
+                    store(std::true_type{}, std::false_type{});
+                } else {
+                    store(std::false_type{}, std::false_type{});
+                }
+            }
+            if (p.cluster > 1) {
                 // the next tile's copies come after these reads and writes of the ring
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 cluster_sync();
