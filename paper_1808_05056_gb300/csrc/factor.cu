@@ -737,13 +737,21 @@ struct Dev {
     int oz_slices = kOzakiSlicesFactor;
 };
 
+// Flops below which an in-HBM update of an Ozaki call takes the FP64 tile kernel: the two
+// splits and the tensor-core launch take 42-55 us of which little depends on the size, and
+// the FP64 tiles do this much in that time, and more exactly (64 x 1504 x 64: 21 us against
+// 46, 64 x 3072 x 64: 34 against 53, 128 x 1504 x 128: 53 against 43, 128 x 3072 x 128: 108
+// against 52).
+constexpr double kOzakiMinFlops = 4e7;
+
 // One in-HBM update C = alpha op(A) op(B) + beta C: the Ozaki form when the call
-// asked for it and its digit planes fit the scratch, else the FP64 tile kernel.
+// asked for it, it is large enough and its digit planes fit the scratch, else the FP64
+// tile kernel.
 int dev_gemm(Dev& d, bool a_k, bool b_k, int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda,
              const double* B, int64_t ldb, double beta, bool read_c, double* C, int64_t ldc, std::string& why,
              int tri = 0, int64_t tri_off = 0)
 {
-    if (d.oz && K > 0 && ozaki_device_scratch(M, N, K, d.oz_slices) <= d.oz_bytes) {
+    if (d.oz && 2.0 * M * N * K >= kOzakiMinFlops && ozaki_device_scratch(M, N, K, d.oz_slices) <= d.oz_bytes) {
         d.launches += 2 * split_ozaki_launches(K) + 1;  // two splits, one tensor-core launch
         return ozaki_gemm_device(a_k, b_k, M, N, K, alpha, A, lda, B, ldb, beta, read_c, C, ldc, d.oz_slices, d.oz,
                                  d.oz_bytes, d.err, d.st, why, tri, tri_off);
