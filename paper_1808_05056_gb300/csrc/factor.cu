@@ -39,6 +39,11 @@ namespace {
 
 constexpr int kSmall = 64;     // order of the triangular blocks the small kernels take
 
+// Out of line, or zeros would go through it too: inlined, it is computed for every lane
+// outside the corrected range and selected afterwards (a block of 64 with 1024 columns of
+// the identity: 80 us, 23 so).
+__device__ __noinline__ double divided(double s, double d) { return s / d; }
+
 // x = s / d from the reciprocal `inv` of d (Markstein's correction: the residual of
 // the rounded product is exact in a fused multiply-add, and adding it back rounds to
 // the quotient): three instructions on the FP64 pipe, which a division would hold for
@@ -49,8 +54,9 @@ __device__ __forceinline__ double quotient(double s, double d, double inv)
     const double q = s * inv;
     const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 0x7FFu;
     if (e - 64u < 0x780u) return fma(fma(-q, d, s), inv, q);
-    if ((__double_as_longlong(s) << 1) == 0 && inv == inv) return q;  // zero over a regular divisor
-    return s / d;
+    const bool regular = (__double2hiint(inv) & 0x7FFFFFFF) < 0x7FF00000;
+    if ((__double_as_longlong(s) << 1) == 0 && regular) return q;  // zero over a regular divisor
+    return divided(s, d);
 }
 
 __device__ __forceinline__ double reciprocal_of(double d)
@@ -84,11 +90,14 @@ __global__ void __launch_bounds__(kTrsmThreads) trsm_small_kernel(const double* 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31, l = lane & (L - 1);
     const int64_t v = ((int64_t)blockIdx.x * (kTrsmThreads / 32) + warp) * (32 / L) + lane / L;
+    // lanes past the last vector solve it again: zeros in their place took another path, and a
+    // warp runs both (1500 vectors: 81 us, 1504: 30; now 27 either way)
+    const int64_t vr = min(v, nvec - 1);
     double x[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {
         const int i = j * L + l, e = lower ? i : n - 1 - i;
-        x[j] = i < n && v < nvec ? P[e * es + v * vs] : 0.0;
+        x[j] = i < n ? P[e * es + vr * vs] : 0.0;
     }
 #pragma unroll 8
     for (int idx = tid; idx < kSmall * kSmall; idx += kTrsmThreads) {
