@@ -351,9 +351,23 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
             // covers 8 rows x 4 consecutive columns of C.  alpha * (hi + lo) + beta * C_old in
             // FP32 double-float steps (TwoSum, products split with fma), rounded once at the
             // end: on this part the FP64 pipe would take ~18 us per tile for it, holding the
-            // accumulators the MMAs wait for
+            // accumulators the MMAs wait for.  The old values of a pass are fetched together,
+            // before its arithmetic (each loaded between two stores, which it may alias, waited
+            // for the one before: 10 us more for a 128 x 128 tile that reads C)
+            const int64_t row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
             auto emit = [&](int pass, const float (&h)[4], const float (&l)[4]) {
-                const int64_t c0 = (int64_t)tn * BN + quarter * 32 + pass * 4;
+                const int64_t col = (int64_t)tn * BN + quarter * 32 + pass * 4 + (lane & 3);
+                float* const cp = p.C + row0 * p.ldc + col;
+                bool keep[4];
+                float old[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t row = row0 + i;
+                    keep[i] = col < p.N && row < p.M &&
+                              (p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off));
+                    old[i] = 0.f;
+                    if (p.read_c && keep[i]) old[i] = cp[i * p.ldc];
+                }
                 double v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -365,27 +379,21 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     v[j] = __longlong_as_double((long long)pack2(__float_as_uint(ph), __float_as_uint(pl)));
                 }
                 transpose4(v, lane);
-                const int64_t col = c0 + (lane & 3), row0 = (int64_t)tm * BM + q4 * 32 + (lane & ~3);
-                if (col >= p.N) return;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int64_t row = row0 + i;
-                    const bool keep = p.tri == 0 || (p.tri == 1 ? col - row <= p.tri_off : col - row >= p.tri_off);
-                    if (row < p.M && keep) {
-                        const uint64_t w = (uint64_t)__double_as_longlong(v[i]);
-                        const float ph = unpack2(w, 0), pl = unpack2(w, 1);
-                        float* cp = p.C + row * p.ldc + col;
-                        if (p.read_c) {
-                            // beta * c = qh + ql and ph + qh = th + tl exactly; one rounding left
-                            const float old = *cp;
-                            const float qh = __fmul_rn(p.beta, old), ql = __fmaf_rn(p.beta, old, -qh);
-                            const float th = __fadd_rn(ph, qh), bq = __fsub_rn(th, ph);
-                            const float tl = __fadd_rn(__fsub_rn(ph, __fsub_rn(th, bq)), __fsub_rn(qh, bq));
-                            *cp = __fadd_rn(th, __fadd_rn(tl, __fadd_rn(pl, ql)));
-                        } else {
-                            *cp = __fadd_rn(ph, pl);
-                        }
+                    const uint64_t w = (uint64_t)__double_as_longlong(v[i]);
+                    const float ph = unpack2(w, 0), pl = unpack2(w, 1);
+                    float c;
+                    if (p.read_c) {
+                        // beta * c = qh + ql and ph + qh = th + tl exactly; one rounding left
+                        const float qh = __fmul_rn(p.beta, old[i]), ql = __fmaf_rn(p.beta, old[i], -qh);
+                        const float th = __fadd_rn(ph, qh), bq = __fsub_rn(th, ph);
+                        const float tl = __fadd_rn(__fsub_rn(ph, __fsub_rn(th, bq)), __fsub_rn(qh, bq));
+                        c = __fadd_rn(th, __fadd_rn(tl, __fadd_rn(pl, ql)));
+                    } else {
+                        c = __fadd_rn(ph, pl);
                     }
+                    if (keep[i]) cp[i * p.ldc] = c;
                 }
             };
             if (p.cluster == 1) {
