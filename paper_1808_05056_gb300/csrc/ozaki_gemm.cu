@@ -443,10 +443,7 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                 for (int pass = rank; pass < 8; pass += p.cluster) {
                     long long t[4] = {0, 0, 0, 0};
                     const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
-                    for (int q = 0; q < p.cluster; ++q) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) t[j] += ld_cluster(at + j * BM * 8, q);
-                    }
+                    for_each_rank<4>(at, BM * 8, rank, p.cluster, [&](int j, long long w) { t[j] += w; });
                     emit(read_c, scale, pass, t);
                 }
             };

@@ -34,8 +34,9 @@
 // fills Y1 and X1.  m x (h, m) fills both Y.
 //
 // Clusters: when a launch has fewer tiles than SMs, the CTAs of a cluster share each
-// tile's K blocks and add their double-float partial sums, in rank order, through
-// distributed shared memory.  Cluster barriers sit in loops that every thread walks
+// tile's K blocks and add their double-float partial sums through distributed shared
+// memory, each CTA a share of the columns, from its own rank on (the order of a column's
+// sums follows from the column alone).  Cluster barriers sit in loops that every thread walks
 // whatever happens, so a CTA whose bounded wait gave up still arrives.
 //
 // The ring releases whole stages: finer slots (one 16 KiB plane tile each, with a wait
@@ -423,13 +424,9 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     for (int pass = rank; pass < 8; pass += p.cluster) {
                         float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
                         const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
-                        for (int q = 0; q < p.cluster; ++q) {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const uint64_t w = (uint64_t)ld_cluster(at + j * BM * 8, q);
-                                add_double_float(h[j], l[j], unpack2(w, 0), unpack2(w, 1));
-                            }
-                        }
+                        for_each_rank<4>(at, BM * 8, rank, p.cluster, [&](int j, long long w) {
+                            add_double_float(h[j], l[j], unpack2((uint64_t)w, 0), unpack2((uint64_t)w, 1));
+                        });
                         emit(pass, h, l);
                     }
                 }
