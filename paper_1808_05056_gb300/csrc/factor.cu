@@ -613,58 +613,73 @@ __global__ void __launch_bounds__(kLuThreads) lu_cluster_kernel(double* P, int64
 // that is final; a row below k1 ends with c of the last swap with that pivot.  Each CTA
 // finds the earlier swaps by comparison, follows the links to the original rows, then
 // moves a strip of columns through shared memory.  n = k1 - k0 <= kLaswpMax.
-constexpr int kLaswpMax = 512, kLaswpCols = 8, kLaswpThreads = 256;
+//
+// Loads in turn are what it would wait for (8 bytes of a strip at a time, 1 us each from host
+// memory, and 1500 shared-memory reads to resolve 512 swaps): comparisons go by eights, and
+// eight values a thread are on their way together (260 launches of an LU of order 4096 6.03 ->
+// 3.23 ms; strips of 16 columns and at most 256 swaps: 3.39).
+constexpr int kLaswpMax = 512, kLaswpCols = 8, kLaswpThreads = 256, kLaswpBatch = 8;
 __global__ void __launch_bounds__(kLaswpThreads) laswp_kernel(double* P, int64_t ldp, int64_t ncols,
                                                               const int64_t* __restrict__ piv, int64_t k0, int n,
                                                               int64_t rows)
 {
     extern __shared__ double vals[];   // [2 n][kLaswpCols]: what rows k0 + k and piv[k] end with
-    __shared__ int64_t pv[kLaswpMax];
+    __shared__ __align__(16) int pv[kLaswpMax + 8];  // pivots, rows counted from k0; -1 past the last
     __shared__ int up[kLaswpMax];      // the earlier swap that made c(k); itself: the original row
-    __shared__ int64_t top[kLaswpMax]; // original row that row k0 + k ends with
-    __shared__ int64_t out[kLaswpMax]; // original row that row piv[k] ends with; -1: not decided by swap k
+    __shared__ int from[2 * kLaswpMax];  // original rows that row k0 + k, then row piv[k], end with; -1: not by swap k
     // a row outside the matrix (a panel kernel that gave up leaves its pivots unset) is no exchange
-    for (int k = threadIdx.x; k < n; k += kLaswpThreads) {
-        const int64_t p = piv[k0 + k];
-        pv[k] = p >= k0 + k && p < rows ? p : k0 + k;
+    for (int k = threadIdx.x; k < n + 8; k += kLaswpThreads) {
+        const int64_t p = k < n ? piv[k0 + k] : -1;
+        pv[k] = k >= n ? -1 : (int)(p >= k0 + k && p < rows ? p - k0 : k);
     }
     __syncthreads();
-    auto latest = [&](int64_t row, int before) {
-        int q = before - 1;
-        while (q >= 0 && pv[q] != row) --q;
-        return q;
+    auto latest = [&](int row, int before) {  // the last swap before `before` whose pivot is `row`, or -1
+        for (int q = (before - 1) & ~7; q >= 0; q -= 8) {
+            const int4 a = *reinterpret_cast<const int4*>(pv + q), b = *reinterpret_cast<const int4*>(pv + q + 4);
+            const unsigned hit = (a.x == row ? 1u : 0u) | (a.y == row ? 2u : 0u) | (a.z == row ? 4u : 0u) |
+                                 (a.w == row ? 8u : 0u) | (b.x == row ? 16u : 0u) | (b.y == row ? 32u : 0u) |
+                                 (b.z == row ? 64u : 0u) | (b.w == row ? 128u : 0u);
+            const unsigned valid = before - q >= 8 ? hit : hit & ((1u << (before - q)) - 1u);
+            if (valid) return q + 31 - __clz(valid);
+        }
+        return -1;
     };
     for (int k = threadIdx.x; k < n; k += kLaswpThreads) {
-        const int q = latest(k0 + k, k);
+        const int q = latest(k, k);
         up[k] = q >= 0 ? q : k;
     }
     __syncthreads();
     auto origin = [&](int k) {  // original row of c(k)
         while (up[k] != k) k = up[k];
-        return k0 + k;
+        return k;
     };
     for (int k = threadIdx.x; k < n; k += kLaswpThreads) {
-        const int64_t p = pv[k];
-        const int q = p == k0 + k ? k : latest(p, k);
-        top[k] = q >= 0 ? origin(q) : p;
-        bool last = p >= k0 + n;
-        for (int z = k + 1; last && z < n; ++z) last = pv[z] != p;
-        out[k] = last ? origin(k) : -1;
+        const int p = pv[k];
+        const int q = p == k ? k : latest(p, k);
+        from[k] = q >= 0 ? origin(q) : p;
+        from[n + k] = p >= n && latest(p, n) == k ? origin(k) : -1;
     }
     __syncthreads();
+    double* const base = P + k0 * ldp;
+    const int total = 2 * n * kLaswpCols;
     for (int64_t c0 = (int64_t)blockIdx.x * kLaswpCols; c0 < ncols; c0 += (int64_t)gridDim.x * kLaswpCols) {
         const int w = (int)min((int64_t)kLaswpCols, ncols - c0);
-        for (int e = threadIdx.x; e < 2 * n * kLaswpCols; e += kLaswpThreads) {
-            const int k = e / kLaswpCols, c = e % kLaswpCols;
-            const int64_t from = k < n ? top[k] : out[k - n];
-            if (c < w && from >= 0) vals[e] = P[from * ldp + c0 + c];
+        const int c = threadIdx.x % kLaswpCols;  // kLaswpThreads is a multiple of kLaswpCols
+        for (int e0 = threadIdx.x; e0 < total; e0 += kLaswpBatch * kLaswpThreads) {
+            double v[kLaswpBatch];
+#pragma unroll
+            for (int u = 0; u < kLaswpBatch; ++u) {
+                const int e = e0 + u * kLaswpThreads, f = e < total && c < w ? from[e / kLaswpCols] : -1;
+                v[u] = f >= 0 ? base[f * ldp + c0 + c] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kLaswpBatch; ++u)
+                if (e0 + u * kLaswpThreads < total) vals[e0 + u * kLaswpThreads] = v[u];
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < 2 * n * kLaswpCols; e += kLaswpThreads) {
-            const int k = e / kLaswpCols, c = e % kLaswpCols;
-            if (c >= w) continue;
-            if (k < n) P[(k0 + k) * ldp + c0 + c] = vals[e];
-            else if (out[k - n] >= 0) P[pv[k - n] * ldp + c0 + c] = vals[e];
+        for (int e = threadIdx.x; e < total; e += kLaswpThreads) {
+            const int k = e / kLaswpCols;
+            if (c < w && from[k] >= 0) base[(k < n ? k : pv[k - n]) * ldp + c0 + c] = vals[e];
         }
         __syncthreads();
     }
@@ -1529,7 +1544,7 @@ int ooc_dgetrf(int64_t N, double* A, int64_t lda, int64_t* ipiv, size_t device_b
         if (trace && (rc = dr.drain())) return rc;
         const auto p1 = now();
         // 2. its interchanges on every other column (L to the left, the trailing matrix to the
-        // right): by the device in host memory, in stream order (1024 rows of 24 KiB: 0.95 ms, against 1.7 ms by 16
+        // right): by the device in host memory, in stream order (1024 rows of 24 KiB: 0.5 ms, against 1.7 ms by 16
         // host threads behind two synchronisations), or by the host
         if (dA) {
             double* rows = dA + c0 * lda;
