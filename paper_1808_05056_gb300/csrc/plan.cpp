@@ -87,7 +87,8 @@ FormModel form_model(int form, int slices_opt, double host_bytes)
         f.products = 6; f.slices = 3;
         f.split_bytes = 10;
     } else {
-        // 72 TFLOP/s (21 products) there; one tile of K 4096 57 us, 192 of K 64 49 us
+        // 72 TFLOP/s (21 products) there; one tile of K 4096 57 us, 192 of K 64 49 us (81, 47 and
+        // 36 with the epilogue of today, figures that choose the same blocks for nine problems in ten)
         const int s = slices_opt > 0 ? slices_opt : kOzakiSlicesGemm;
         const int planes = ozaki_planes(s);
         f.rate = 1.5e15 / (planes * (planes + 1) / 2); f.exchange = 4e-6; f.launch = 18e-6;
