@@ -39,6 +39,8 @@ namespace {
 
 constexpr int kSmall = 64;     // order of the triangular blocks the small kernels take
 
+int64_t round_up64(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
+
 // Out of line, or zeros would go through it too: inlined, it is computed for every lane
 // outside the corrected range and selected afterwards (a block of 64 with 1024 columns of
 // the identity: 80 us, 23 so).
@@ -781,7 +783,7 @@ int dev_gemm(Dev& d, bool a_k, bool b_k, int64_t M, int64_t N, int64_t K, double
              int tri = 0, int64_t tri_off = 0)
 {
     if (d.oz && 2.0 * M * N * K >= kOzakiMinFlops && ozaki_device_scratch(M, N, K, d.oz_slices) <= d.oz_bytes) {
-        d.launches += 2 * split_ozaki_launches(K) + 1;  // two splits, one tensor-core launch
+        d.launches += 2 * split_ozaki_launches(K) + ozaki_tile_launches(round_up64(K, 64), ozaki_planes(d.oz_slices));
         return ozaki_gemm_device(a_k, b_k, M, N, K, alpha, A, lda, B, ldb, beta, read_c, C, ldc, d.oz_slices, d.oz,
                                  d.oz_bytes, d.err, d.st, why, tri, tri_off);
     }
@@ -1034,8 +1036,6 @@ int panel_lu(double* P, int64_t ldp, int64_t m, int64_t n, int64_t* piv, int64_t
     }
     return OOC_OK;
 }
-
-int64_t round_up64(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 bool is_l(char c) { return c == 'L' || c == 'l'; }
 bool is_r(char c) { return c == 'R' || c == 'r'; }

@@ -18,8 +18,12 @@
 // 2^-frac): to an integer by packed FP32 additions of large constants (the conversion
 // unit is a quarter as wide as these pipes), then one wide multiply-add.  In FP64 the same drain is bound by the FP64 pipe
 // (1.75 additions a clock and SM: 9400 clocks per 128 x 128 sum, which takes the
-// tensor cores 4096 clocks to make).  Integer sums are exact whatever their order, so
-// the result does not depend on how a tile's work is cut (cut_stages).
+// tensor cores 4096 clocks to make).  Sums on diagonals 8 m <= frac are added exactly,
+// finer ones are rounded to the unit first; seven and eight planes, which hold more bits
+// than such a unit, sum their finest diagonals in a launch of their own with a unit that
+// holds them whole (launch_ozaki_tiles).  The order of integer additions does not matter,
+// and rounded sums are cut where they are rounded (cut_stages), so the result does not
+// depend on how a tile's work is cut.
 //
 // Kernel shape: tile 128 x 128, 64 of K per stage, 18 warps.
 //   warp 0      TMA producer: the bf16 tiles of one A plane and of two neighbouring B
@@ -677,10 +681,10 @@ constexpr int kShortSplit = 1024;
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Groups and units of a launch (kernel comment, "Order of the products") for S planes
-// and `kblocks` K blocks, and each accumulator's weight: a sum of digit products
-// with s + t = m counts 2^(frac - 8 m) units.
-void plan_units(Args& a, int S)
+// Groups and units of a launch (kernel comment, "Order of the products") for the pairs
+// (d, d + 1) of S planes with lo <= d <= hi and `kblocks` K blocks, and each accumulator's
+// weight: a sum of digit products with s + t = m counts 2^(frac - 8 m) units.
+void plan_units(Args& a, int S, int lo, int hi)
 {
     int ng = 0, nu = 0;
     auto weigh = [&](Unit& u, int q, int m) {
@@ -704,6 +708,7 @@ void plan_units(Args& a, int S)
     // diagonals 2 .. S + 1 in pairs (d, d + 1); an odd number of them leaves 2 to itself, a
     // single product, which a pair (1, 2) describes
     for (int d = S % 2 ? 1 : 2; d <= S; d += 2) {
+        if (d < lo || d > hi) continue;
         const int first = ng;
         for (int s = 1; s < d; ++s) a.group[ng++] = Group{(int8_t)(s - 1), (int8_t)(d - s - 1), 2, 0};
         a.group[ng++] = Group{(int8_t)(d - 1), 0, 1, 0};
@@ -729,10 +734,11 @@ int64_t tile_cost(const Args& a)
 
 // Cut a tile's stages (in walk()'s order) into `cluster` shares of about equal cost; returns
 // the largest.  Sums that are rounded to the integers' unit are cut at drains only, so that
-// what is rounded, and with it the result, does not depend on the cut.
-int64_t cut_stages(Args& a, int cluster, int planes)
+// what is rounded, and with it the result, does not depend on the cut.  finest: the launch's
+// last diagonal.
+int64_t cut_stages(Args& a, int cluster, int finest)
 {
-    const bool anywhere = a.frac >= DIGIT * (planes + 1);
+    const bool anywhere = a.frac >= DIGIT * finest;
     const int64_t total = tile_cost(a);
     int64_t cost = 0, largest = 0, begun = 0;
     int pos = 0, next = 1;
@@ -768,21 +774,47 @@ int64_t cut_stages(Args& a, int cluster, int planes)
 // a tile's stages; the exchange of their partial sums costs about as much as kExchange
 // stages.  Leaves the chosen size and its cuts in `a`.
 constexpr int64_t kExchange = 16;
-void choose_cluster(Args& a, int planes, const ClusterCounts& counts)
+void choose_cluster(Args& a, int finest, const ClusterCounts& counts)
 {
     int best = 1;
     int64_t cost = INT64_MAX;
     for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
         const int n = counts.at_once[c];
         if (n <= 0) continue;
-        const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c, planes) + (c > 1 ? kExchange : 0));
+        const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c, finest) + (c > 1 ? kExchange : 0));
         if (t < cost) { cost = t; best = c; }
     }
     a.cluster = best;
-    cut_stages(a, best, planes);
+    cut_stages(a, best, finest);
 }
 
+// K of one stretch: the integers' unit, see launch_ozaki_tiles
+constexpr int64_t kStretch = 1 << 18;
+
+// The integers' unit of a launch over `kblocks` K blocks: |sum| <= (128 / 255)^2 K < 0.253 K,
+// so 2^(64 - ceil(log2 K)) units stay below 2^62.02.
+int unit_bits(int64_t kblocks)
+{
+    int lg = 6;
+    while (((int64_t)1 << lg) < kblocks * BK) ++lg;
+    return 64 - lg;
+}
+
+// Whether that unit holds the sums of `planes` planes with room: all of them exactly, or what
+// is rounded costs less than the products that S = 4/3 planes slices of 6 bits drop.  Those are
+// sqrt(K) 2^(-6 S - 2.3) of the operands' largest entries; one rounding in 1024 of K of each
+// sum finer than the unit, 11 to 22 of them, is sqrt(K) 2^(-frac - 5) and less.
+bool one_unit(int planes, int frac) { return frac >= std::min(6 * planes + 10, DIGIT * (planes + 1)); }
+
 }  // namespace
+
+int ozaki_tile_launches(int64_t k_pad, int planes)
+{
+    int n = 0;
+    for (int64_t kb = 0; kb == 0 || kb < k_pad / BK; kb += kStretch / BK)
+        n += one_unit(planes, unit_bits(std::min(kStretch / BK, k_pad / BK - kb))) ? 1 : 2;
+    return n;
+}
 
 int split_ozaki_launches(int64_t K) { return K > kShortSplit ? 2 : 1; }
 
@@ -848,31 +880,41 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     a.row_exp = P.row_exp; a.col_exp = P.col_exp;
     a.err = P.err;
     a.tri = P.tri; a.tri_off = P.tri_off;
-    // The integers' unit: |sum| <= (128 / 255)^2 K < 0.253 K, so 2^(64 - ceil(log2 K)) units stay
-    // below 2^62.02.  Sums too fine for it are rounded to it; a longer K goes in stretches of
-    // kStretch (each added into C in FP64) so that the unit stays at or below 2^-46, under what
-    // the dropped products cost.
-    constexpr int64_t kStretch = 1 << 18;
+    // K goes in stretches of kStretch (each added into C in FP64), so that the unit stays at or
+    // below 2^-46, under what the dropped products of six planes cost.  Seven and eight planes
+    // promise more (one_unit): there the diagonals whose sums the unit holds exactly go first,
+    // and the finer ones in a second launch, in the unit of the finest, where all are exact
+    // (they add up to less than 2^59 of it).  Rounded to the first unit as those of six planes
+    // are, they made ten slices 2 to 60 times less accurate than FP64 sums of the digit products
+    // from K 2048 to 65536 (N(0,1) 9.8e-16 for 1.2e-16 at 4096, 2.4e-14 for 3.7e-16 at 65536) and
+    // nine up to ten times from 16384 (4.7e-14 for 4.8e-15 at 65536, sign 10^U(-4,4)); so, the
+    // error is a third of those sums' or less throughout (4.4e-17 and 6.2e-16 at 65536).
     const int64_t kb_total = P.k_pad / BK, kb_step = kStretch / BK;
+    bool fresh = true;  // the call's first launch applies beta
     for (int64_t kb0 = 0; kb0 == 0 || kb0 < kb_total; kb0 += kb_step) {
         a.kb0 = (int)kb0;
         a.kblocks = (int)std::min(kb_step, kb_total - kb0);
-        a.beta = kb0 == 0 ? P.beta : 1.0;
-        a.read_c = kb0 == 0 ? (P.read_c ? 1 : 0) : 1;
-        int lg = 6;
-        while (((int64_t)1 << lg) < (int64_t)a.kblocks * BK) ++lg;
-        a.frac = 64 - lg;
-        plan_units(a, P.planes);
-        choose_cluster(a, P.planes, counts);
-        cudaLaunchConfig_t cfg;
-        cudaLaunchAttribute at;
-        cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, SMEM_BYTES,
-                       static_cast<cudaStream_t>(stream));
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel, ma, mb, a);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            why = std::string("ozaki tile launch: ") + cudaGetErrorString(e);
-            return OOC_ERR_CUDA;
+        const int bits = unit_bits(a.kblocks), finest = P.planes + 1;
+        const bool one = one_unit(P.planes, bits);
+        for (int part = 0; part < (one ? 1 : 2); ++part) {
+            // the last pair (d, d + 1) of the first launch: 8 (d + 1) <= bits
+            const int exact = bits / DIGIT - 1;
+            a.frac = part == 0 ? bits : DIGIT * finest;
+            a.beta = fresh ? P.beta : 1.0;
+            a.read_c = fresh ? (P.read_c ? 1 : 0) : 1;
+            fresh = false;
+            plan_units(a, P.planes, part == 0 ? 1 : exact + 1, one || part == 1 ? P.planes : exact);
+            choose_cluster(a, one || part == 1 ? finest : exact + 1, counts);
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute at;
+            cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, SMEM_BYTES,
+                           static_cast<cudaStream_t>(stream));
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel, ma, mb, a);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                why = std::string("ozaki tile launch: ") + cudaGetErrorString(e);
+                return OOC_ERR_CUDA;
+            }
         }
     }
     return OOC_OK;
