@@ -86,3 +86,13 @@ def test_triangular_update(ooc, uplo):
     bd = bounds.ozaki_bound(a, a.T, 1.5, 0.5, np.nan_to_num(c0), 10)
     assert bounds.worst_ratio(got[~keep], ref[~keep], bd[~keep]) <= 1.0
     assert np.array_equal(got[keep], c0[keep], equal_nan=True)
+
+
+# K beyond 262,144: a second stretch that adds into C, in one launch each or two
+@pytest.mark.parametrize("S,launches", [(8, 2), (9, 3)])
+def test_stretches(ooc, S, launches):
+    K = (1 << 18) + 200   # nine slices: the last, short stretch needs one launch
+    A, B, c0, got, st = _run(ooc, 40, 30, K, S, synth.LOGSPREAD, 4.0, alpha=-2.5, beta=0.5, budget=4 << 30, kb=K)
+    assert st.kernel_launches == 4 + launches
+    ref = oracle.gemm("N", "N", -2.5, A, B, 0.5, c0)
+    assert bounds.worst_ratio(got, ref, bounds.ozaki_bound(A, B, -2.5, 0.5, c0, S)) <= 1.0
