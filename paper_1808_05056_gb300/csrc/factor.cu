@@ -50,12 +50,15 @@ __device__ __noinline__ double divided(double s, double d) { return s / d; }
 // the rounded product is exact in a fused multiply-add, and adding it back rounds to
 // the quotient): three instructions on the FP64 pipe, which a division would hold for
 // about twenty.  `inv` is NaN where the correction could leave the normal range
-// (reciprocal_of); a quotient near the ends of it goes through the division too.
+// (reciprocal_of); a quotient near the ends of it goes through the division too, and so does
+// a dividend below 2^-959, whose residual, down to 2^-105 of it, need not be a multiple of the
+// smallest subnormal.
 __device__ __forceinline__ double quotient(double s, double d, double inv)
 {
     const double q = s * inv;
     const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 0x7FFu;
-    if (e - 64u < 0x780u) return fma(fma(-q, d, s), inv, q);
+    const unsigned es = ((unsigned)__double2hiint(s) >> 20) & 0x7FFu;
+    if (e - 64u < 0x780u && es >= 64u) return fma(fma(-q, d, s), inv, q);
     const bool regular = (__double2hiint(inv) & 0x7FFFFFFF) < 0x7FF00000;
     if ((__double_as_longlong(s) << 1) == 0 && regular) return q;  // zero over a regular divisor
     return divided(s, d);
