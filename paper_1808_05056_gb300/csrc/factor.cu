@@ -909,6 +909,23 @@ int launch_laswp(double* P, int64_t ldp, int64_t rows, int64_t ncols, const int6
     return OOC_OK;
 }
 
+// Rows that launch_laswp reads, and writes, for the n interchanges k <-> piv[k], k < n: per launch
+// its own and the distinct pivot rows below them.
+int64_t laswp_rows(const int64_t* piv, int64_t n)
+{
+    int64_t rows = 0;
+    std::vector<int64_t> below;
+    for (int64_t k0 = 0; k0 < n; k0 += kLaswpMax) {
+        const int64_t k1 = std::min<int64_t>(n, k0 + kLaswpMax);
+        below.clear();
+        for (int64_t k = k0; k < k1; ++k)
+            if (piv[k] >= k1) below.push_back(piv[k]);
+        std::sort(below.begin(), below.end());
+        rows += k1 - k0 + (std::unique(below.begin(), below.end()) - below.begin());
+    }
+    return rows;
+}
+
 void lu_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, size_t smem, cudaStream_t st)
 {
     cfg = {};
@@ -1542,6 +1559,11 @@ int ooc_dgetrf(int64_t N, double* A, int64_t lda, int64_t* ipiv, size_t device_b
             if (cudaMemcpy(hpiv.data(), dpiv, (size_t)tk * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
                 return fail(OOC_ERR_CUDA, "pivot read failed");
             for (int64_t q = 0; q < tk; ++q) ipiv[c0 + q] = c0 + hpiv[q];
+            if (dA) {  // the interchanges of step 2 cross the link both ways
+                const double bytes = (double)laswp_rows(hpiv.data(), tk) * (double)(c0 + rest) * 8;
+                dr.h2d += bytes;
+                dr.d2h += bytes;
+            }
             return OOC_OK;
         };
         if (trace && (rc = dr.drain())) return rc;
