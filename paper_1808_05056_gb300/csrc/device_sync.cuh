@@ -168,9 +168,4 @@ __device__ __forceinline__ void for_each_rank(uint32_t addr, uint32_t step, int 
     }
 }
 
-__device__ __forceinline__ bool launch_failed(const int* err)
-{
-    return *reinterpret_cast<const volatile int*>(err) != 0;
-}
-
 }  // namespace ooc

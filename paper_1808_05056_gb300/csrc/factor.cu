@@ -32,6 +32,7 @@
 
 #include "device_sync.cuh"
 #include "ooc_internal.hpp"
+#include "tc_common.cuh"
 
 namespace ooc {
 
@@ -926,20 +927,6 @@ int64_t laswp_rows(const int64_t* piv, int64_t n)
     return rows;
 }
 
-void lu_cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int cluster, size_t smem, cudaStream_t st)
-{
-    cfg = {};
-    cfg.gridDim = dim3((unsigned)cluster);
-    cfg.blockDim = dim3(kLuThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)cluster;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-}
-
 // CTAs of the cluster that takes an m-row sub-panel (0: too tall): at least 32 rows each,
 // so that a warp's instructions carry 32 rows, and as many CTAs as that leaves -- the
 // update's FP64 work is spread over their SMs.
@@ -958,7 +945,7 @@ int lu_cluster_size(int64_t m)
         for (int c = kLuClusterMax; c >= 1 && !largest; c /= 2) {
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute at;
-            lu_cluster_config(cfg, at, c, kLuClusterSmem, nullptr);
+            cluster_config(cfg, at, c, 1, kLuThreads, kLuClusterSmem, nullptr);
             int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, lu_cluster_kernel, &cfg) != cudaSuccess) cudaGetLastError();
             else if (n > 0) largest = c;
@@ -983,7 +970,7 @@ int panel_lu(double* P, int64_t ldp, int64_t m, int64_t n, int64_t* piv, int64_t
         const int rows = (int)((m + cluster - 1) / cluster);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute at;
-        lu_cluster_config(cfg, at, cluster, (size_t)rows * kLuClusterLd * sizeof(double), d.st);
+        cluster_config(cfg, at, cluster, 1, kLuThreads, (size_t)rows * kLuClusterLd * sizeof(double), d.st);
         const cudaError_t e =
             cudaLaunchKernelEx(&cfg, lu_cluster_kernel, P, ldp, (int)m, (int)n, rows, piv, d.info, gofs, d.err);
         ++d.launches;

@@ -78,7 +78,7 @@ constexpr int EPI_WARPS = 16;                         // 4 per TMEM lane quadran
 constexpr int THREADS = (2 + EPI_WARPS) * 32;
 constexpr int KSTEPS = BK / 16;
 constexpr int MAX_PLANES = 8;
-constexpr int MAX_GROUPS = 28;                        // 8 planes: 16 double and 4 single groups
+constexpr int MAX_GROUPS = 20;                        // 8 planes: 16 double and 4 single groups
 constexpr int MAX_UNITS = MAX_GROUPS;
 constexpr int MAX_CLUSTER = 8;
 static_assert(RING_BYTES >= (uint32_t)BM * BN * 8, "the ring holds a tile of 64-bit partial sums");
@@ -141,27 +141,12 @@ __device__ __forceinline__ bool walk(const Args& p, int begin, int end, Fn fn)
     return true;
 }
 
-// Packed pairs of FP32 values (element 2j in the low half).
 __device__ __forceinline__ uint64_t f2fma(uint64_t a, uint64_t b, uint64_t c)
 {
     uint64_t d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-__device__ __forceinline__ uint64_t f2add(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t f2sub(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t pair(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
-__device__ __forceinline__ uint64_t pair(float x) { return pair(__float_as_uint(x), __float_as_uint(x)); }
 
 // v * sc for two FP32 sums v, |v * sc| <= 2^24, rounded to the nearest integer (ties to
 // even).  Adding 1.5 2^25 rounds to a multiple of 4, h, and leaves h / 4 in the low bits;

@@ -93,21 +93,6 @@ struct TcArgs {
     int64_t tri_off;
 };
 
-// Packed pairs of FP32 values (element 2j in the low half): Blackwell's f32x2
-// arithmetic does two of the drain's additions per instruction.
-__device__ __forceinline__ uint64_t f2add(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t f2sub(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
 __device__ __forceinline__ float unpack2(uint64_t v, int j) { return __uint_as_float((uint32_t)(v >> (32 * j))); }
 
 // Drains of the small-product accumulators: every SMALL_EVERY chunks and at the last
@@ -312,7 +297,7 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     for (int j = 0; j < 4; ++j) {
                         // TwoSum on pairs: hi + x = sum + e exactly, e added into lo
                         uint64_t& h = hi2[cc * 4 + j];
-                        const uint64_t x = pack2(v[2 * j], v[2 * j + 1]);
+                        const uint64_t x = pair(v[2 * j], v[2 * j + 1]);
                         const uint64_t sum = f2add(h, x);
                         const uint64_t bp = f2sub(sum, h);
                         const uint64_t e = f2add(f2sub(h, f2sub(sum, bp)), f2sub(x, bp));
@@ -339,7 +324,7 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                         tmem_wait_ld();
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            lo2[(cc & 3) * 4 + j] = f2add(lo2[(cc & 3) * 4 + j], pack2(v[2 * j], v[2 * j + 1]));
+                            lo2[(cc & 3) * 4 + j] = f2add(lo2[(cc & 3) * 4 + j], pair(v[2 * j], v[2 * j + 1]));
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -377,7 +362,7 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
                     const float sl = __fadd_rn(__fsub_rn(h[j], __fsub_rn(sh, bp)), __fsub_rn(l[j], bp));
                     const float ph = __fmul_rn(p.alpha, sh);
                     const float pl = __fmaf_rn(p.alpha, sl, __fmaf_rn(p.alpha, sh, -ph));
-                    v[j] = __longlong_as_double((long long)pack2(__float_as_uint(ph), __float_as_uint(pl)));
+                    v[j] = __longlong_as_double((long long)pair(__float_as_uint(ph), __float_as_uint(pl)));
                 }
                 transpose4(v, lane);
 #pragma unroll
@@ -417,7 +402,7 @@ __global__ void __launch_bounds__(THREADS, 1) bf16x3_tile_kernel(const __grid_co
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
                         part[(quarter * 32 + j) * BM + row_in_tile] =
-                            pack2(__float_as_uint(unpack2(hi2[j >> 1], j & 1)), __float_as_uint(unpack2(lo2[j >> 1], j & 1)));
+                            pair(__float_as_uint(unpack2(hi2[j >> 1], j & 1)), __float_as_uint(unpack2(lo2[j >> 1], j & 1)));
                 }
                 cluster_sync();
                 if (ok) {
