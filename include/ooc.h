@@ -59,7 +59,7 @@ extern "C" {
 /* ---- contraction forms ----------------------------------------------- */
 #define OOC_FORM_AUTO 0    /* dgemm: FP64; sgemm: BF16x3                                 */
 #define OOC_FORM_FP64 1    /* plain FP64 tiles (FP64 tensor-core MMA)                    */
-#define OOC_FORM_OZAKI 2   /* FP64-accurate: Ozaki bf16 slice products, FP64 accumulate  */
+#define OOC_FORM_OZAKI 2   /* FP64-accurate: exact products of bf16 digits, 64-bit fixed-point sums */
 #define OOC_FORM_BF16X3 3  /* FP32-accurate: three-piece bf16 split, six products        */
 
 /* ---- plan selection flags (ooc_opts.flags) --------------------------- */
@@ -127,7 +127,10 @@ int ooc_dgemm(char transA, char transB, int64_t M, int64_t N, int64_t K, double 
 /*
  * Out-of-core SGEMM with FP32-accurate BF16x3 tiles: FP32 host operands and
  * result, the same problem statement as ooc_dgemm.  alpha and beta are
- * applied in FP64 before the result is rounded to FP32.
+ * applied to a two-term FP32 sum, which is rounded to FP32 once.  Where a step
+ * has few tiles several CTAs share one and add parts of its K, so the last
+ * bits of a result depend on the blocking: equal calls agree bit for bit, calls
+ * with another budget or other block sizes within the form's accuracy.
  */
 int ooc_sgemm(char transA, char transB, int64_t M, int64_t N, int64_t K, float alpha,
               const float* A, int64_t lda, const float* B, int64_t ldb, float beta,
@@ -243,7 +246,7 @@ int ooc_dgemmt(char uplo, char transA, char transB, int64_t N, int64_t K, double
  * N x N matrix C; trans 'N': A is stored N x K (lda >= K) and the update is
  * A A^T; 'T': A is stored K x N (lda >= N) and the update is A^T A.  Same
  * rules as ooc_dgemmt.  ooc_ssyrk takes FP32 operands and runs the BF16x3
- * form (alpha and beta applied in FP64 before rounding to FP32).
+ * form (see ooc_sgemm).
  */
 int ooc_dsyrk(char uplo, char trans, int64_t N, int64_t K, double alpha, const double* A,
               int64_t lda, double beta, double* C, int64_t ldc, size_t device_budget_bytes,
@@ -292,9 +295,11 @@ int ooc_dpotrf(char uplo, int64_t N, double* A, int64_t lda, size_t device_budge
  * is never chosen while a number remains; a column with no comparable entry
  * keeps row j).  Right-
  * looking over panels of t columns: the (N - c0) x t panel is factored in
- * device memory (recursive halving; 64-column panels by one cooperative kernel
- * with a bounded grid barrier per pivot), its interchanges are applied to the
- * other columns on the host, U12 = L11^{-1} A12 is solved in device memory,
+ * device memory (recursive halving; 32 columns at a time by one cluster, above
+ * 11,776 rows 64 by one cooperative kernel, every wait bounded), its
+ * interchanges are applied to the other columns by the device in host memory
+ * (by host threads when A is not one page-locked range mapped to the device)
+ * and count in h2d_bytes and d2h_bytes, U12 = L11^{-1} A12 is solved in device memory,
  * and the trailing matrix is updated with one out-of-core GEMM.  *info is 0, or j + 1
  * for the first exactly zero pivot (the factorisation still completes, as in
  * LAPACK).  The budget must hold one N x 64 panel.  opts->form: FP64 or Ozaki

@@ -11,8 +11,9 @@
 //      blocked algorithm: triangular blocks of at most 64 by the substitution
 //      and Cholesky kernels below, everything else by the tile kernels.
 // LU is right-looking: each panel is factored in device memory (recursive
-// halving down to a cooperative 64-column kernel), then the trailing matrix
-// gets one out-of-core GEMM.  So nearly all flops run in the pipelined GEMM,
+// halving down to 32 columns in one cluster, 64 in a cooperative kernel where
+// the rows are too many for that), then the trailing matrix gets one
+// out-of-core GEMM.  So nearly all flops run in the pipelined GEMM,
 // in the caller's form (FP64 tiles, or the FP64-accurate Ozaki tensor-core form).
 #include <cuda_runtime.h>
 

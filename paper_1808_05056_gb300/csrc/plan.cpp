@@ -62,8 +62,13 @@ FormModel form_model(int form, int slices_opt, double host_bytes)
     FormModel f{};
     f.ctas_per_sm = 1;
     f.cluster = 1;
-    // strided copies with short rows slowed down in pipelines over tens of GiB of host memory;
-    // over less they run at two thirds of the link's rate
+    // Strided copies with short rows run at two thirds of the link's rate while a machine's host
+    // memory is fresh and slower the more of it pipelines have touched: BF16x3 40000^3 (19 GB of
+    // operands, 640 x 5760 blocks) took 0.55 s in the first process, 0.73 and 1.12 s in the third and
+    // fifth, and the two charges estimate 0.61 and 0.86 s.  The slow one is kept for operands of tens
+    // of GiB, whose plans were measured with it.  8 GiB itself is no measured boundary: 26700^3 (8.6
+    // GB) takes 197 ms on either side of it, and both charges choose the same blocks for square
+    // BF16x3 products from 16000 to 65536.
     f.rows_slow = host_bytes > 8.0 * (1ull << 30);
     if (form == OOC_FORM_FP64) {
         f.tile = 16; f.grain = 64; f.rate = 1.09e12;
