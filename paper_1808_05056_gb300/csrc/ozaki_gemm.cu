@@ -787,8 +787,8 @@ int unit_bits(int64_t kblocks)
 
 // Whether that unit holds the sums of `planes` planes with room: all of them exactly, or what
 // is rounded costs less than the products that S = 4/3 planes slices of 6 bits drop.  Those are
-// sqrt(K) 2^(-6 S - 2.3) of the operands' largest entries; one rounding in 1024 of K of each
-// sum finer than the unit, 11 to 22 of them, is sqrt(K) 2^(-frac - 5) and less.
+// sqrt(K) 2^(-6 S - 2.2) of the operands' scales; one rounding in 1024 of K of each sum finer
+// than the unit, 11 to 22 of them, is sqrt(K) 2^(-frac - 4.5) or less.
 bool one_unit(int planes, int frac) { return frac >= std::min(6 * planes + 10, DIGIT * (planes + 1)); }
 
 }  // namespace
@@ -870,10 +870,12 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     // promise more (one_unit): there the diagonals whose sums the unit holds exactly go first,
     // and the finer ones in a second launch, in the unit of the finest, where all are exact
     // (they add up to less than 2^59 of it).  Rounded to the first unit as those of six planes
-    // are, they made ten slices 2 to 60 times less accurate than FP64 sums of the digit products
+    // are, they made ten slices 3 to 66 times less accurate than FP64 sums of the digit products
     // from K 2048 to 65536 (N(0,1) 9.8e-16 for 1.2e-16 at 4096, 2.4e-14 for 3.7e-16 at 65536) and
     // nine up to ten times from 16384 (4.7e-14 for 4.8e-15 at 65536, sign 10^U(-4,4)); so, the
-    // error is a third of those sums' or less throughout (4.4e-17 and 6.2e-16 at 65536).
+    // error is half of those sums' or less throughout (4.4e-17 and 6.2e-16 at 65536).  The second
+    // launch reads C again and has its own tail: 9 slices 4096 x 4096 x 8192 10.2 -> 10.9 ms, 10
+    // slices 4096 x 4096 x 2048 3.17 -> 3.52 ms.
     const int64_t kb_total = P.k_pad / BK, kb_step = kStretch / BK;
     bool fresh = true;  // the call's first launch applies beta
     for (int64_t kb0 = 0; kb0 == 0 || kb0 < kb_total; kb0 += kb_step) {
