@@ -788,7 +788,7 @@ int dev_gemm(Dev& d, bool a_k, bool b_k, int64_t M, int64_t N, int64_t K, double
              int tri = 0, int64_t tri_off = 0)
 {
     if (d.oz && 2.0 * M * N * K >= kOzakiMinFlops && ozaki_device_scratch(M, N, K, d.oz_slices) <= d.oz_bytes) {
-        d.launches += 2 * split_ozaki_launches(K) + ozaki_tile_launches(round_up64(K, 64), ozaki_planes(d.oz_slices));
+        d.launches += 2 * split_ozaki_launches(K) + 1;  // two splits, one tensor-core launch
         return ozaki_gemm_device(a_k, b_k, M, N, K, alpha, A, lda, B, ldb, beta, read_c, C, ldc, d.oz_slices, d.oz,
                                  d.oz_bytes, d.err, d.st, why, tri, tri_off);
     }

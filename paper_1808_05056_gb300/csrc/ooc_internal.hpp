@@ -279,8 +279,6 @@ struct OzakiProblem {
     int64_t tri_off = 0;
 };
 int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why);
-// kernels launch_ozaki_tiles launches
-int ozaki_tile_launches(int64_t k_pad, int planes);
 // `planes` digit planes of an operand and its row exponents, and how many kernels that launches
 int split_ozaki_launches(int64_t K);
 int launch_split_ozaki(const double* X, int64_t sr, int64_t sk, int rows, int K, int rows_pad, int k_pad, int planes,

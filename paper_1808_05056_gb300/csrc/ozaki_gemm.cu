@@ -19,11 +19,13 @@
 // unit is a quarter as wide as these pipes), then one wide multiply-add.  In FP64 the same drain is bound by the FP64 pipe
 // (1.75 additions a clock and SM: 9400 clocks per 128 x 128 sum, which takes the
 // tensor cores 4096 clocks to make).  Sums on diagonals 8 m <= frac are added exactly,
-// finer ones are rounded to the unit first; seven and eight planes, which hold more bits
-// than such a unit, sum their finest diagonals in a launch of their own with a unit that
-// holds them whole (launch_ozaki_tiles).  The order of integer additions does not matter,
-// and rounded sums are cut where they are rounded (cut_stages), so the result does not
-// depend on how a tile's work is cut.
+// finer ones are rounded to the unit first.  Where that would cost more than the dropped
+// products (seven and eight planes but for short K, six beyond K 2^18; one_unit), the wide
+// kernel takes the fine diagonals first, in a unit 2^16 times finer, puts the low 16 bits
+// of their sums away in shared memory and goes on with the rest shifted to the unit: 80 bits
+// in all, rounded once.  The order of integer additions does not matter, and rounded sums are
+// cut where they are rounded (cut_stages), so the result does not depend on how a tile's
+// work is cut.
 //
 // Kernel shape: tile 128 x 128, 64 of K per stage, 18 warps.
 //   warp 0      TMA producer: the bf16 tiles of one A plane and of two neighbouring B
@@ -73,6 +75,7 @@ constexpr uint32_t TILE_BYTES = BM * BK * 2u;         // one plane tile: 128 row
 constexpr uint32_t STAGE_BYTES = 3 * TILE_BYTES;      // A plane, two B planes
 constexpr int STAGES = 4;
 constexpr uint32_t RING_BYTES = STAGES * STAGE_BYTES;
+constexpr uint32_t LOW_BYTES = BM * BN * 2u;          // wide kernel: 16 low bits per output
 constexpr size_t SMEM_BYTES = 1024 + RING_BYTES + 256;
 constexpr int EPI_WARPS = 16;                         // 4 per TMEM lane quadrant, 32 columns each
 constexpr int THREADS = (2 + EPI_WARPS) * 32;
@@ -82,6 +85,7 @@ constexpr int MAX_GROUPS = 20;                        // 8 planes: 16 double and
 constexpr int MAX_UNITS = MAX_GROUPS;
 constexpr int MAX_CLUSTER = 8;
 static_assert(RING_BYTES >= (uint32_t)BM * BN * 8, "the ring holds a tile of 64-bit partial sums");
+static_assert(SMEM_BYTES + LOW_BYTES <= 227 * 1024, "the wide kernel fits an SM");
 
 // One group: A plane a with B planes b and b + 1 (nb == 2), or with plane b alone, whose
 // product goes into the second accumulator.
@@ -91,9 +95,10 @@ struct Group {
 
 // A unit shares one accumulator pair: `ngroups` groups from `first`, drained every
 // `chunk` K blocks.  The two accumulators' weights as a factor applied in FP32 (a
-// power of two, sums are rounded to integers after it) and a left shift.
+// power of two, sums are rounded to integers after it) and a left shift.  fine: in the wide
+// kernel's finer unit; those units come first.
 struct Unit {
-    int16_t first, ngroups, chunk, pad;
+    int16_t first, ngroups, chunk, fine;
     float scale[2];
     int32_t shift[2];
 };
@@ -187,6 +192,17 @@ __device__ __forceinline__ double fixed_to_f64(long long t, int e)
     return top ? __hiloint2double((int)hi, (int)(uint32_t)m) : 0.0;
 }
 
+// The leading bits of 2^16 t + r (0 <= r < 2^16) as one integer times 2^up, with room for its
+// negation.  Bits that do not fit set the lowest one (rounding to odd): at least 60 bits are
+// left then, so that rounding to 53 sees the same as from all of them.
+__device__ __forceinline__ long long joined(long long t, uint32_t r, int& up)
+{
+    const int s = min(16, max(0, __clzll(t ^ (t >> 63)) - 2));
+    up = 16 - s;
+    return (long long)((unsigned long long)t << s) | (r >> up) | ((r & ((1u << up) - 1u)) != 0 ? 1 : 0);
+}
+
+template <bool kWide>
 __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                 const __grid_constant__ CUtensorMap tmB,
                                                                 const __grid_constant__ Args p)
@@ -200,6 +216,7 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
     uint64_t* acc_empty = acc_full + 2;
     uint64_t* done = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* low = reinterpret_cast<uint64_t*>(ring + RING_BYTES + 256);  // [4 columns][row], 16 bits each
 
     // the shuffle tells the compiler that the warp index is the same in all lanes
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
@@ -321,6 +338,20 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
             long long acc[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) acc[j] = 0;
+            uint64_t* const low_me = low + quarter * 8 * BM + row_in_tile;
+            auto put_away = [&] {
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    uint64_t w = 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        w |= (uint64_t)(acc[j + i] & 0xFFFF) << (16 * i);
+                        acc[j + i] >>= 16;
+                    }
+                    low_me[j / 4 * BM] = w;
+                }
+            };
+            bool fine = kWide;  // the sums so far are in the finer unit
             if (ok)
                 ok = walk(p, begin, end, [&](const Unit& un, int, int nk, int lo, int) {
                     // every lane gives up together (the warp shuffles and syncs below need all 32)
@@ -328,6 +359,12 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                         return false;
                     tc_fence_after();
                     const uint32_t t0 = tmem_base + lane_off + (uint32_t)(b.s * 2 * BN + quarter * 32);
+                    if constexpr (kWide) {
+                        if (fine && !un.fine) {
+                            put_away();
+                            fine = false;
+                        }
+                    }
                     // the pair's single product comes last: alone, it leaves the first accumulator unused
                     const int q0 = p.group[un.first + lo / nk].nb == 2 ? 0 : 1;
 #pragma unroll 1
@@ -360,6 +397,9 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     b.next(2);
                     return true;
                 });
+            if constexpr (kWide) {
+                if (fine) put_away();
+            }
             // the tile's result, 4 columns at a time: each lane forms its own row's values,
             // transpose4 hands lane 4g + j column j of rows 4g .. 4g + 3, and each store then
             // covers 8 rows x 4 consecutive columns of C (whole 32-byte sectors).  The old values
@@ -373,7 +413,8 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
             double* const c_lane = p.C + (int64_t)row0 * p.ldc + col0;
             const int rows_left = p.M - row0;
             // read_c and scale are compile-time: a predicated-off instruction holds the FP64 pipe too
-            auto emit = [&](auto read_c, auto scale, int pass, const long long (&t)[4]) {
+            // t: sums in the unit; r: the wide kernel's 16 bits below it
+            auto emit = [&](auto read_c, auto scale, int pass, const long long (&t)[4], const uint32_t (&r)[4]) {
                 const int col = col0 + pass * 4;
                 double* const c = c_lane + pass * 4;
                 bool keep[4];
@@ -394,8 +435,10 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                 double v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    v[j] = fixed_to_f64(p.alpha_one < 0 ? -t[j] : t[j],
-                                        re + __shfl_sync(0xffffffffu, ce_lane, pass * 4 + j));
+                    int up = 16;
+                    const long long w = kWide ? joined(t[j], r[j], up) : t[j];
+                    v[j] = fixed_to_f64(p.alpha_one < 0 ? -w : w,
+                                        re + up - 16 + __shfl_sync(0xffffffffu, ce_lane, pass * 4 + j));
                 }
                 if constexpr (scale.value) {
 #pragma unroll
@@ -424,7 +467,12 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
 #pragma unroll
                     for (int pass = 0; pass < 8; ++pass) {
                         const long long t[4] = {acc[pass * 4], acc[pass * 4 + 1], acc[pass * 4 + 2], acc[pass * 4 + 3]};
-                        emit(read_c, scale, pass, t);
+                        uint32_t r[4] = {0, 0, 0, 0};
+                        if constexpr (kWide) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) r[j] = (uint32_t)(low_me[pass * BM] >> (16 * j)) & 0xFFFFu;
+                        }
+                        emit(read_c, scale, pass, t, r);
                     }
                     return;
                 }
@@ -433,7 +481,19 @@ __global__ void __launch_bounds__(THREADS, 1) ozaki_tile_kernel(const __grid_con
                     long long t[4] = {0, 0, 0, 0};
                     const uint32_t at = smem_u32(part + (quarter * 32 + pass * 4) * BM + row_in_tile);
                     for_each_rank<4>(at, BM * 8, rank, p.cluster, [&](int j, long long w) { t[j] += w; });
-                    emit(read_c, scale, pass, t);
+                    uint32_t r[4] = {0, 0, 0, 0};
+                    if constexpr (kWide) {
+                        for_each_rank<1>(smem_u32(low_me + pass * BM), 0, rank, p.cluster, [&](int, long long w) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) r[j] += (uint32_t)((uint64_t)w >> (16 * j)) & 0xFFFFu;
+                        });
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            t[j] += r[j] >> 16;
+                            r[j] &= 0xFFFFu;
+                        }
+                    }
+                    emit(read_c, scale, pass, t, r);
                 }
             };
             if (ok) {
@@ -666,16 +726,45 @@ constexpr int kShortSplit = 1024;
 
 int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
-// Groups and units of a launch (kernel comment, "Order of the products") for the pairs
-// (d, d + 1) of S planes with lo <= d <= hi and `kblocks` K blocks, and each accumulator's
-// weight: a sum of digit products with s + t = m counts 2^(frac - 8 m) units.
-void plan_units(Args& a, int S, int lo, int hi)
+// The integers' unit of a launch over `kblocks` K blocks, 2^-frac: |sum| <= (128 / 255)^2 K <
+// 0.253 K, so 2^(64 - ceil(log2 K)) units stay below 2^62.02.
+int unit_bits(int64_t kblocks)
+{
+    int lg = 6;
+    while (((int64_t)1 << lg) < kblocks * BK) ++lg;
+    return 64 - lg;
+}
+
+// Whether that unit holds the sums of `planes` planes with room: all of them exactly, or what
+// is rounded costs less than the products that S = 4/3 planes slices of 6 bits drop.  Those are
+// sqrt(K) 2^(-6 S - 2.2) of the operands' scales; one rounding in 1024 of K of each sum finer
+// than the unit, 11 to 22 of them, is sqrt(K) 2^(-frac - 4.5) or less.  So one unit does to K
+// 2^18 for six planes, 4096 for seven, 64 for eight.  With one throughout, ten slices were 3 to
+// 66 times less accurate than FP64 sums of the digit products from K 2048 to 65536 (N(0,1)
+// 9.8e-16 for 1.2e-16 at 4096, 2.4e-14 for 3.7e-16 at 65536) and nine up to ten times from 16384
+// (4.7e-14 for 4.8e-15 at 65536, sign 10^U(-4,4)); the wide kernel's error is half of those sums'
+// or less throughout (below 1e-16 and 1e-15 at 65536) and costs 1-8 % (9 slices 4096 x 4096 x
+// 8192 10.3 -> 10.6 ms, 3000 x 2000 x 16384 in 256 MiB 37.1 -> 40.0; 10 slices 4096 x 4096 x 2048
+// 3.18 -> 3.30; a solve of order 12288 60.5 -> 61.9).  The same sums as two launches that add
+// into C took 10.9, 40.6, 3.53 and 62.7 ms, and parts that overflow to opposite sides left NaN.
+bool one_unit(int planes, int frac) { return frac >= std::min(6 * planes + 10, DIGIT * (planes + 1)); }
+
+// First diagonal pair whose sums the wide kernel takes in the finer unit: from 5 on K products on
+// each add up to less than 2^57 of 2^-(frac + 16), while pairs below stay at or under diagonal 5,
+// which the unit holds exactly to K 2^24, the longest a launch takes.
+constexpr int kFinePair = 5;
+constexpr int64_t kStretch = 1 << 24;
+
+// Groups and units of a launch (kernel comment, "Order of the products") for S planes and
+// `kblocks` K blocks, and each accumulator's weight: a sum of digit products with s + t = m
+// counts 2^(frac - 8 m) units.
+void plan_units(Args& a, int S, bool wide)
 {
     int ng = 0, nu = 0;
     auto weigh = [&](Unit& u, int q, int m) {
         // a left shift of the converted sum (at most 2^24 in magnitude); below 0: bits rounded
         // off in the conversion.  2^31 as a signed multiplier is -2^31, so the sum changes sign
-        int sh = a.frac - DIGIT * m;
+        int sh = a.frac + (u.fine ? 16 : 0) - DIGIT * m;
         float sc = 1.0f;
         if (sh < 0) { sc = std::ldexp(1.0f, sh); sh = 0; }
         else if (sh == 31) sc = -1.0f;
@@ -687,13 +776,13 @@ void plan_units(Args& a, int S, int lo, int hi)
         u.first = (int16_t)first;
         u.ngroups = (int16_t)n;
         u.chunk = (int16_t)std::max(1, chunk);
+        u.fine = wide && d >= kFinePair;
         weigh(u, 0, d);
         weigh(u, 1, d + 1);
     };
     // diagonals 2 .. S + 1 in pairs (d, d + 1); an odd number of them leaves 2 to itself, a
     // single product, which a pair (1, 2) describes
-    for (int d = S % 2 ? 1 : 2; d <= S; d += 2) {
-        if (d < lo || d > hi) continue;
+    auto add_pair = [&](int d) {
         const int first = ng;
         for (int s = 1; s < d; ++s) a.group[ng++] = Group{(int8_t)(s - 1), (int8_t)(d - s - 1), 2, 0};
         a.group[ng++] = Group{(int8_t)(d - 1), 0, 1, 0};
@@ -701,7 +790,10 @@ void plan_units(Args& a, int S, int lo, int hi)
         if (cdiv(a.kblocks, shared) <= d * cdiv(a.kblocks, EXACT_KBLOCKS)) add_unit(first, d, shared, d);
         else
             for (int g = first; g < ng; ++g) add_unit(g, 1, EXACT_KBLOCKS, d);
-    }
+    };
+    for (int fine = wide ? 1 : 0; fine >= 0; --fine)
+        for (int d = S % 2 ? 1 : 2; d <= S; d += 2)
+            if (!wide || (d >= kFinePair) == (fine == 1)) add_pair(d);
     a.nunits = nu;
 }
 
@@ -719,11 +811,12 @@ int64_t tile_cost(const Args& a)
 
 // Cut a tile's stages (in walk()'s order) into `cluster` shares of about equal cost; returns
 // the largest.  Sums that are rounded to the integers' unit are cut at drains only, so that
-// what is rounded, and with it the result, does not depend on the cut.  finest: the launch's
-// last diagonal.
-int64_t cut_stages(Args& a, int cluster, int finest)
+// what is rounded, and with it the result, does not depend on the cut.
+int64_t cut_stages(Args& a, int cluster)
 {
-    const bool anywhere = a.frac >= DIGIT * finest;
+    bool anywhere = true;
+    for (int u = 0; u < a.nunits; ++u)
+        anywhere = anywhere && std::min(std::fabs(a.unit[u].scale[0]), std::fabs(a.unit[u].scale[1])) == 1.0f;
     const int64_t total = tile_cost(a);
     int64_t cost = 0, largest = 0, begun = 0;
     int pos = 0, next = 1;
@@ -759,47 +852,40 @@ int64_t cut_stages(Args& a, int cluster, int finest)
 // a tile's stages; the exchange of their partial sums costs about as much as kExchange
 // stages.  Leaves the chosen size and its cuts in `a`.
 constexpr int64_t kExchange = 16;
-void choose_cluster(Args& a, int finest, const ClusterCounts& counts)
+void choose_cluster(Args& a, const ClusterCounts& counts)
 {
     int best = 1;
     int64_t cost = INT64_MAX;
     for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
         const int n = counts.at_once[c];
         if (n <= 0) continue;
-        const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c, finest) + (c > 1 ? kExchange : 0));
+        const int64_t t = cdiv(a.tiles, n) * (cut_stages(a, c) + (c > 1 ? kExchange : 0));
         if (t < cost) { cost = t; best = c; }
     }
     a.cluster = best;
-    cut_stages(a, best, finest);
+    cut_stages(a, best);
 }
 
-// K of one stretch: the integers' unit, see launch_ozaki_tiles
-constexpr int64_t kStretch = 1 << 18;
-
-// The integers' unit of a launch over `kblocks` K blocks: |sum| <= (128 / 255)^2 K < 0.253 K,
-// so 2^(64 - ceil(log2 K)) units stay below 2^62.02.
-int unit_bits(int64_t kblocks)
+template <bool kWide>
+int launch_kernel(const CUtensorMap& ma, const CUtensorMap& mb, Args& a, cudaStream_t st, std::string& why)
 {
-    int lg = 6;
-    while (((int64_t)1 << lg) < kblocks * BK) ++lg;
-    return 64 - lg;
+    constexpr size_t smem = SMEM_BYTES + (kWide ? LOW_BYTES : 0);
+    static const ClusterCounts counts = count_clusters((const void*)ozaki_tile_kernel<kWide>, THREADS, smem);
+    if (counts.at_once[1] <= 0) { why = "ozaki tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
+    choose_cluster(a, counts);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, smem, st);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel<kWide>, ma, mb, a);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        why = std::string("ozaki tile launch: ") + cudaGetErrorString(e);
+        return OOC_ERR_CUDA;
+    }
+    return OOC_OK;
 }
-
-// Whether that unit holds the sums of `planes` planes with room: all of them exactly, or what
-// is rounded costs less than the products that S = 4/3 planes slices of 6 bits drop.  Those are
-// sqrt(K) 2^(-6 S - 2.2) of the operands' scales; one rounding in 1024 of K of each sum finer
-// than the unit, 11 to 22 of them, is sqrt(K) 2^(-frac - 4.5) or less.
-bool one_unit(int planes, int frac) { return frac >= std::min(6 * planes + 10, DIGIT * (planes + 1)); }
 
 }  // namespace
-
-int ozaki_tile_launches(int64_t k_pad, int planes)
-{
-    int n = 0;
-    for (int64_t kb = 0; kb == 0 || kb < k_pad / BK; kb += kStretch / BK)
-        n += one_unit(planes, unit_bits(std::min(kStretch / BK, k_pad / BK - kb))) ? 1 : 2;
-    return n;
-}
 
 int split_ozaki_launches(int64_t K) { return K > kShortSplit ? 2 : 1; }
 
@@ -840,8 +926,6 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     if (P.M <= 0 || P.N <= 0) return OOC_OK;
     if (P.planes < 1 || P.planes > MAX_PLANES) { why = "digit plane count out of range"; return OOC_ERR_INVALID_ARG; }
     if (P.k_pad % BK) { why = "K padding not a multiple of the K block"; return OOC_ERR_INVALID_ARG; }
-    static const ClusterCounts counts = count_clusters((const void*)ozaki_tile_kernel, THREADS, SMEM_BYTES);
-    if (counts.at_once[1] <= 0) { why = "ozaki tile kernel: shared memory attribute"; return OOC_ERR_CUDA; }
     CUtensorMap ma, mb;
     std::memset(&ma, 0, sizeof(ma));
     std::memset(&mb, 0, sizeof(mb));
@@ -865,44 +949,20 @@ int launch_ozaki_tiles(const OzakiProblem& P, void* stream, std::string& why)
     a.row_exp = P.row_exp; a.col_exp = P.col_exp;
     a.err = P.err;
     a.tri = P.tri; a.tri_off = P.tri_off;
-    // K goes in stretches of kStretch (each added into C in FP64), so that the unit stays at or
-    // below 2^-46, under what the dropped products of six planes cost.  Seven and eight planes
-    // promise more (one_unit): there the diagonals whose sums the unit holds exactly go first,
-    // and the finer ones in a second launch, in the unit of the finest, where all are exact
-    // (they add up to less than 2^59 of it).  Rounded to the first unit as those of six planes
-    // are, they made ten slices 3 to 66 times less accurate than FP64 sums of the digit products
-    // from K 2048 to 65536 (N(0,1) 9.8e-16 for 1.2e-16 at 4096, 2.4e-14 for 3.7e-16 at 65536) and
-    // nine up to ten times from 16384 (4.7e-14 for 4.8e-15 at 65536, sign 10^U(-4,4)); so, the
-    // error is half of those sums' or less throughout (4.4e-17 and 6.2e-16 at 65536).  The second
-    // launch reads C again and has its own tail: 9 slices 4096 x 4096 x 8192 10.2 -> 10.9 ms, 10
-    // slices 4096 x 4096 x 2048 3.17 -> 3.52 ms.
+    // Longer K in stretches, each added into C: sums must not go through C where that can be
+    // helped, since parts that overflow to opposite sides leave NaN.
     const int64_t kb_total = P.k_pad / BK, kb_step = kStretch / BK;
-    bool fresh = true;  // the call's first launch applies beta
     for (int64_t kb0 = 0; kb0 == 0 || kb0 < kb_total; kb0 += kb_step) {
         a.kb0 = (int)kb0;
         a.kblocks = (int)std::min(kb_step, kb_total - kb0);
-        const int bits = unit_bits(a.kblocks), finest = P.planes + 1;
-        const bool one = one_unit(P.planes, bits);
-        for (int part = 0; part < (one ? 1 : 2); ++part) {
-            // the last pair (d, d + 1) of the first launch: 8 (d + 1) <= bits
-            const int exact = bits / DIGIT - 1;
-            a.frac = part == 0 ? bits : DIGIT * finest;
-            a.beta = fresh ? P.beta : 1.0;
-            a.read_c = fresh ? (P.read_c ? 1 : 0) : 1;
-            fresh = false;
-            plan_units(a, P.planes, part == 0 ? 1 : exact + 1, one || part == 1 ? P.planes : exact);
-            choose_cluster(a, one || part == 1 ? finest : exact + 1, counts);
-            cudaLaunchConfig_t cfg;
-            cudaLaunchAttribute at;
-            cluster_config(cfg, at, a.cluster, std::min(a.tiles, counts.at_once[a.cluster]), THREADS, SMEM_BYTES,
-                           static_cast<cudaStream_t>(stream));
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_tile_kernel, ma, mb, a);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                why = std::string("ozaki tile launch: ") + cudaGetErrorString(e);
-                return OOC_ERR_CUDA;
-            }
-        }
+        a.beta = kb0 == 0 ? P.beta : 1.0;
+        a.read_c = kb0 == 0 ? (P.read_c ? 1 : 0) : 1;
+        a.frac = unit_bits(a.kblocks);
+        const bool wide = !one_unit(P.planes, a.frac);
+        plan_units(a, P.planes, wide);
+        cudaStream_t st = static_cast<cudaStream_t>(stream);
+        const int rc = wide ? launch_kernel<true>(ma, mb, a, st, why) : launch_kernel<false>(ma, mb, a, st, why);
+        if (rc) return rc;
     }
     return OOC_OK;
 }

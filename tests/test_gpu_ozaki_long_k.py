@@ -1,14 +1,13 @@
 """Ozaki form with 9 and 10 slices over a long K: sums finer than the kernel's usual 64-bit unit.
 
-Seven and eight planes of 8-bit digits sum their finest diagonals in a launch of their own
-(csrc/ozaki_gemm.cu, launch_ozaki_tiles), from K 4097 and 65 on.  The rms error over a block of
-dot products, in units of 2^(e_i + f_j) (operands scaled below 1), is made of
+From K 4097 and 65 on seven and eight planes of 8-bit digits sum their finest diagonals in a unit
+2^16 times finer, six planes from K 262,145 on (csrc/ozaki_gemm.cu, the wide kernel).  The rms
+error over a block of dot products, in units of 2^(e_i + f_j) (operands scaled below 1), is made of
     the dropped products      sqrt((P - 1) K) 5461 2^(2 - 8 (P + 2)): P - 1 of them per k on the first
                               diagonal left out, digits spread evenly over +-128 (mean square 5461);
                               a digit count P and weight 2^2 for the two scales 2^(e + 1), 2^(f + 1)
     the rounded operands      0.29 2^(1 - 8 P) (|x| + |y|), Euclidean norms
-    FP64 roundings of C       of each of two sums, of C after each and of alpha and beta's
-                              products: 6 2^-53 rms |C|
+    FP64 roundings of C       at most six of 2^-53 rms |C|
 and may be twice that.  The reference sums in long double (K 2^-64 of it and less).
 """
 import numpy as np
@@ -49,17 +48,14 @@ def test_slices_keep_their_accuracy(ooc, S, K, kind, param):
     assert rms(((got - ref) / scale).astype(np.float64)) <= 2 * (dropped + operands + rounding)
 
 
-# the last K of one launch and the first of two (64 for eight planes, 4096 for seven), where the
-# diagonals' division moves, long and ragged K; alpha and beta are applied once
+# the last K of one unit and the first of two (64 for eight planes, 4096 for seven), a drain's
+# K blocks, long and ragged K
 @pytest.mark.parametrize("S,K", [(10, 64), (10, 65), (10, 257), (10, 1000), (10, 5000), (9, 4096), (9, 4097),
                                  (9, 8200), (9, 70000)])
-def test_launches_and_bounds(ooc, S, K):
+def test_bounds(ooc, S, K):
     A, B, c0, got, st = _run(ooc, 130, 140, K, S, synth.LOGSPREAD, 4.0, alpha=-2.5, beta=0.5, kb=K)
     ref = oracle.gemm("N", "N", -2.5, A, B, 0.5, c0)
     assert bounds.worst_ratio(got, ref, bounds.ozaki_bound(A, B, -2.5, 0.5, c0, S)) <= 1.0
-    two = K > (64 if S == 10 else 4096)
-    splits = 2 if K > 1024 else 1
-    assert st.kernel_launches == 2 * splits + (2 if two else 1)
 
 
 @pytest.mark.parametrize("S", [9, 10])
@@ -72,7 +68,7 @@ def test_result_does_not_depend_on_the_cut(ooc, S):
 
 @pytest.mark.parametrize("uplo", "LU")
 def test_triangular_update(ooc, uplo):
-    """The second launch keeps to the triangle as the first does (the rest comes back as it was)."""
+    """Masked stores of the wide kernel: the rest comes back as it was."""
     N, K = 300, 500
     A, C = pinned_from(98, 0, N, K, synth.NORMAL), pinned_from(98, 2, N, N, synth.NORMAL)
     keep = np.triu(np.ones((N, N), bool), 1) if uplo == "L" else np.tril(np.ones((N, N), bool), -1)
@@ -88,11 +84,59 @@ def test_triangular_update(ooc, uplo):
     assert np.array_equal(got[keep], c0[keep], equal_nan=True)
 
 
-# K beyond 262,144: a second stretch that adds into C, in one launch each or two
-@pytest.mark.parametrize("S,launches", [(8, 2), (9, 3)])
-def test_stretches(ooc, S, launches):
-    K = (1 << 18) + 200   # nine slices: the last, short stretch needs one launch
+@pytest.mark.parametrize("S", [8, 9])
+def test_six_planes_beyond_one_unit(ooc, S):
+    K = (1 << 18) + 200
     A, B, c0, got, st = _run(ooc, 40, 30, K, S, synth.LOGSPREAD, 4.0, alpha=-2.5, beta=0.5, budget=4 << 30, kb=K)
-    assert st.kernel_launches == 4 + launches
     ref = oracle.gemm("N", "N", -2.5, A, B, 0.5, c0)
     assert bounds.worst_ratio(got, ref, bounds.ozaki_bound(A, B, -2.5, 0.5, c0, S)) <= 1.0
+
+
+# one unit and two: sums beyond the largest FP64 number are infinite with the sum's sign, whatever
+# the signs of its coarse and fine parts
+@pytest.mark.parametrize("S,K", [(8, 200), (10, 200), (9, 5000), (8, (1 << 18) + 200)])
+def test_overflow_is_infinite(ooc, S, K):
+    M, N = 12, 10
+    A, B = pinned_from(94, 0, M, K, synth.NORMAL), pinned_from(94, 1, K, N, synth.NORMAL)
+    C = pinned_from(94, 2, M, N, synth.NORMAL)
+    exact = A.numpy().astype(np.longdouble) @ B.numpy().astype(np.longdouble)
+    assert np.abs(exact).min() > 1e-6
+    A.mul_(2.0 ** 560)
+    B.mul_(2.0 ** 560)
+    rc = ooc.ooc_dgemm("N", "N", M, N, K, 1.0, A, K, B, N, 0.5, C, N, 4 << 30,
+                       ooc.make_opts(form=ooc.OOC_FORM_OZAKI, slices=S, kb=K), None)
+    assert rc == 0, ooc.ooc_last_error()
+    assert np.array_equal(np64(C), np.where(exact > 0, np.inf, -np.inf))
+
+
+def test_stretches(ooc):
+    """K beyond 2^24: a second launch that adds into C (three rows of digit planes, 52 GB of them)."""
+    K = (1 << 24) + 200
+    A, B, c0, got, _ = _run(ooc, 3, 2, K, 8, synth.NORMAL, alpha=-2.5, beta=0.5, budget=80 << 30, kb=K)
+    ref = oracle.gemm("N", "N", -2.5, A, B, 0.5, c0)
+    assert bounds.worst_ratio(got, ref, bounds.ozaki_bound(A, B, -2.5, 0.5, c0, 8)) <= 1.0
+
+
+@pytest.mark.parametrize("S", [9, 10])
+def test_signs_and_ties_of_the_low_bits(ooc, S):
+    """Sums whose leading part is small, zero or negative, and results half way between two FP64
+    numbers: integers with few bits, exact in every digit, against exact integers rounded once."""
+    M, N, K = 64, 48, 5000
+    rng = np.random.default_rng(S)
+    a = np.zeros((M, K))
+    b = np.zeros((K, N))
+    a[:, :8] = rng.integers(-2 ** 26, 2 ** 26, (M, 8))
+    b[:8] = rng.integers(-2 ** 26, 2 ** 26, (8, N))
+    a[:, 8], b[8] = 2.0 ** 27, 0.0                    # the rows' and columns' largest entries
+    a[:, 9], b[9] = 0.0, 2.0 ** 27
+    a[::3, 10], b[10] = 1.0, 1.0                      # odd sums above 2^53
+    a[:5, :8] = 0.0                                   # 1 or 0 alone: fine diagonals only
+    A, B, C = (pinned_from(93, s, *x, synth.NORMAL) for s, x in ((0, a.shape), (1, b.shape), (2, (M, N))))
+    A.numpy()[:], B.numpy()[:] = a, b
+    for alpha in (1.0, -1.0):
+        rc = ooc.ooc_dgemm("N", "N", M, N, K, alpha, A, K, B, N, 0.0, C, N, 1 << 30,
+                           ooc.make_opts(form=ooc.OOC_FORM_OZAKI, slices=S, kb=K), None)
+        assert rc == 0, ooc.ooc_last_error()
+        ia, ib = a[:, :11].astype(np.int64).astype(object), b[:11].astype(np.int64).astype(object)
+        exact = ia.dot(ib)
+        assert np.array_equal(np64(C), alpha * np.array([[float(x) for x in r] for r in exact]))
